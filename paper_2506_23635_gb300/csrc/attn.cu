@@ -146,6 +146,12 @@ k_sa_setup(int T, int32_t *offsets) {
     write_trivial_dispatch(T, offsets);
 }
 
+// The decode attention's counters start at zero (threads of one block).
+__device__ __forceinline__ void zero_dec_count(int *count) {
+    if (count)
+        for (int i = threadIdx.x; i < kAttnDecodeMaxCtas; i += blockDim.x) count[i] = 0;
+}
+
 // qkv [T, (Hq + 2 Hkv) 128] fp32 (the sum of n_part partial projections
 // part_stride floats apart) -> q [T, Hq, 128] fp32 (rotated); rotated keys
 // and the values to the caches [n_seq, Hkv, L, 128] in bf16.  A block holds
@@ -159,12 +165,13 @@ k_rope_cache(int T, int Hq, int Hkv, int n_seq, int L, RopeRates rates,
              const int32_t *__restrict__ seq, const int32_t *__restrict__ pos,
              const float *__restrict__ qkv, int n_part, long long part_stride,
              float *__restrict__ q, bf16 *__restrict__ q16, bf16 *__restrict__ kc,
-             bf16 *__restrict__ vc, unsigned *err) {
+             bf16 *__restrict__ vc, int *__restrict__ dec_count, unsigned *err) {
     // a decode-type call (no 128-token prefill tile): the tensor-core decode
     // attention, one CTA per SM on the SMs this small grid leaves free, may
     // launch now and set itself up while this kernel runs
     if (T < kAttnTcTile) ptx::launch_dependents();
     ptx::grid_dependency_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0) zero_dec_count(dec_count);
     constexpr int H2 = kHeadDim / 2;
     static_assert(kRopeTokens * H2 <= kRopeRows * H2, "one thread per (token, pair)");
     __shared__ float cs_s[kRopeTokens][H2], sn_s[kRopeTokens][H2];
@@ -488,8 +495,10 @@ k_attn_merge(int n_split, const float *__restrict__ part_ml, const float *__rest
 // brings its own queries (moe_sa_attend); in the whole block the rotary
 // kernel writes it.  n4 groups of four elements.
 __global__ void __launch_bounds__(256)
-k_q_bf16(long long n4, const float *__restrict__ q, bf16 *__restrict__ q16) {
+k_q_bf16(long long n4, const float *__restrict__ q, bf16 *__restrict__ q16,
+         int *__restrict__ dec_count) {
     ptx::grid_dependency_wait();
+    if (blockIdx.x == 0) zero_dec_count(dec_count);
     const float4 *a = reinterpret_cast<const float4 *>(q);
     __nv_bfloat162 *o = reinterpret_cast<__nv_bfloat162 *>(q16);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
@@ -591,7 +600,7 @@ k_residual_prenorm(int T, int D, int n_part, float *__restrict__ resid, const fl
 // ---- host ------------------------------------------------------------------------
 
 struct SaWs {
-    size_t offsets, xn, qkv, q, q16, tile_ok, part_ml, part_acc, ctx, total;
+    size_t offsets, xn, qkv, q, q16, tile_ok, part_ml, part_acc, dec_count, dec_part, ctx, total;
 };
 
 SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
@@ -612,6 +621,8 @@ SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
     L.tile_ok = o; o += up((size_t)(T + kAttnTcTile - 1) / kAttnTcTile * 4);
     L.part_ml = o; o += up(splits * 2 * 4);
     L.part_acc = o; o += up(splits * kHeadDim * 4);
+    L.dec_count = o; o += up(kAttnDecodeMaxCtas * 4);
+    L.dec_part = o; o += up(T <= kAttnDecodeMaxTokens ? kAttnDecodePartFloats * 4 : 0);
     L.ctx = o; o += up((size_t)T * nq * 2);
     L.total = o;
     return L;
@@ -700,8 +711,9 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
     bf16 *kcp = static_cast<bf16 *>(kc), *vcp = static_cast<bf16 *>(vc);
     unsigned *err = device_info().err;
     int Tv = c.T;
+    int *dec_count = q16 ? at<int>(c.ws, c.L.dec_count) : nullptr;
     void *args[] = {&Tv,     &Hq,      &Hkv, &ns,  &Lv,  &rates, &seq, &pos,
-                    &qkvc,   &n_part,  &pstride, &q, &q16, &kcp, &vcp, &err};
+                    &qkvc,   &n_part,  &pstride, &q, &q16, &kcp, &vcp, &dec_count, &err};
     LaunchScope ls("rope_cache", c.st);
     const int rows = Hq + 2 * Hkv;
     return launch_pdl((const void *)k_rope_cache,
@@ -742,9 +754,9 @@ cudaError_t attend(const SaCall &c, const float *q, const int32_t *seq, const in
         if (e != cudaSuccess) return e;
         ns = 1;
     } else if (q16 && decode_tc()) {
-        // splits merged inside the kernel (a cluster per token and key/value head)
-        return launch_attn_decode_tc(c.T, Hq, Hkv, n_seq, L, attn_decode_tc_splits(c.T, Hkv, L),
-                                     seq, pos, q16, kc, vc, ctx, c.st);
+        return launch_attn_decode_tc(c.T, Hq, Hkv, n_seq, L, seq, pos, q16, kc, vc, ctx,
+                                     at<float>(c.ws, c.L.dec_part), at<int>(c.ws, c.L.dec_count),
+                                     c.st);
     }
     const void *kern = nullptr;
     switch (G) {
@@ -925,7 +937,8 @@ moe_status moe_sa_attend(const moe_sa_dims *dims, int32_t T, const float *q, con
         q16 = at<bf16>(ws, c.L.q16);
         long long n4 = (long long)T * dims->n_heads * dims->head_dim / 4;
         const float *qc = q;
-        void *args[] = {&n4, &qc, &q16};
+        int *dec_count = at<int>(ws, c.L.dec_count);
+        void *args[] = {&n4, &qc, &q16, &dec_count};
         const int blocks = (int)std::min<long long>((n4 + 255) / 256, 4LL * device_info().sm_count);
         LaunchScope ls("q_bf16", c.st);
         cudaError_t e = launch_pdl((const void *)k_q_bf16, dim3(std::max(blocks, 1)), dim3(256), 0,

@@ -12,22 +12,33 @@
 //                       MN-major A operand), P_j K-major in shared memory
 //
 // with S^T and O^T in tensor memory (lane = position, resp. dim; column =
-// head).  One CTA per (position split c, token t, key/value head g); the
-// splits of (t, g) share the position tiles of t's sequence (128 positions
-// each): split c takes tiles c, c + n_split, c + 2 n_split first, then one
-// at a time from a counter in the cluster's CTA 0, so a split whose share
-// of the memory bandwidth runs ahead takes more tiles.  A CTA's j-th tile
-// goes to its stages in order and is published in a ring of tile indices
-// (-1 after its last):
+// head).  Two schedules (template parameter SPLIT):
 //
-//   warp 0      TMA: the group's bf16 query rows once, then key and value
-//               tiles into three-stage rings (each 32 KB: two boxes of 64
-//               dims with the 128-byte swizzle), the first three before the
-//               block-wide barrier of the set-up;
+//   shares   the position tiles (128 positions each) of every (token,
+//            key/value head), token by token, are one list; CTA b of G (one
+//            per SM) takes the contiguous share [W b / G, W (b + 1) / G) of its
+//            W tiles, so every SM streams the same number of bytes whatever
+//            the sequences' lengths.  A share is a run of pieces: the end of
+//            one (token, head)'s tiles, whole ones, the start of another's.
+//            (One CTA per (token, head) before: 88 of 152 SMs with 11
+//            sequences, all waiting for the longest; 1488-4096 positions, 118
+//            MB of keys and values: 42.2 us before, 30.6 us, of which ~8 us are
+//            launch, first load and drain.)
+//   splits   few (token, head)s: the n_split (up to 8) CTAs of a cluster share
+//            the tiles of one: split c takes tiles c, c + n_split, c + 2
+//            n_split first, then one at a time from a counter in the cluster's
+//            CTA 0, so a split whose share of the memory bandwidth runs ahead
+//            takes more.
+//
+//   warp 0      TMA: a piece's bf16 query rows into one of four buffers, key
+//               and value tiles into three-stage rings (each 32 KB: two boxes
+//               of 64 dims with the 128-byte swizzle), the first three before
+//               the block-wide barrier of the set-up; each tile is described
+//               to the other warps in a ring of DecDesc;
 //   warp 1      tensor memory (S^T twice, O^T: 48 of 64 columns) and the
 //               MMAs: S_{j+1} is issued as soon as its key tile has landed
 //               and the softmax has read S_{j-1}, O += P_j V_j once P_j is
-//               written;
+//               written (a piece's first tile overwrites O);
 //   warps 2-5   softmax, one thread per position of the tile (its tensor-
 //               memory lane): the tile maximum of every head across the
 //               128 positions (a warp maximum, then the four warps' through
@@ -40,19 +51,26 @@
 //               sequence's last position zeroed (0 * NaN is NaN; those cache
 //               rows may hold anything).
 //
-// The end: each thread owns dim r of O^T; per head the row sums of the four
-// warps are added.  A single split writes ctx.  Several splits of one
-// (token, key/value head) are the CTAs of one thread-block cluster (at most
-// 8), and CTA c owns the heads h = c, c + n_split, ...: every CTA stores its
+// The end of a piece: each thread owns dim r of O^T; per head the row sums of
+// the four warps are added.  Shares: a (token, head) that lies in one share is
+// written to ctx at once; otherwise every share that holds a piece of it
+// leaves (base, sum) and O^T in the workspace and, its share done, counts
+// itself on the (token, head)'s counter; the one that counts last merges the
+// pieces in order and writes ctx (no CTA waits for another).  Splits: CTA c of
+// the cluster owns the heads h = c, c + n_split, ...; every CTA stores its
 // (base, sum) and O^T row of each head straight into the owner's shared
-// memory with asynchronous stores that count their bytes on the owner's
-// merge barrier (the owner expects all splits' bytes from its start), so
-// no sender waits for its stores or fences them; the owner's acquire wait
-// on the barrier sees every split's partials, then it combines its heads
-// and writes their ctx.  (The stores wait until every CTA of the cluster
-// has initialised its barriers: each arrives on the cluster barrier at its
-// start and waits on it before storing, by when the wait is long
-// satisfied.)
+// memory with asynchronous stores that count their bytes on the owner's merge
+// barrier (the owner expects all splits' bytes from its start), so no sender
+// waits for its stores or fences them; the owner's acquire wait on the barrier
+// sees every split's partials, then it combines its heads and writes their
+// ctx.  (The stores wait until every CTA of the cluster has initialised its
+// barriers: each arrives on the cluster barrier at its start and waits on it
+// before storing, by when the wait is long satisfied.)
+//
+// The kernel launches while the one ahead of it (which writes the call's new
+// cache rows and the queries) runs; key and value tiles that lie wholly before
+// the call's own positions do not depend on it and are loaded at once (0.5-1.5
+// us of the attention block at 1-11 sequences).
 //
 // Numerics as the prefill flash attention: bf16 queries and probabilities,
 // fp32 scores and accumulation; the row sum takes the probabilities as
@@ -61,6 +79,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "tc.cuh"
 
@@ -73,30 +92,37 @@ constexpr int kDecPos = 128;   // positions per key/value tile: the MMA's M
 constexpr int kDecN = 16;      // the MMA's N: the group's query heads, zero-padded
 constexpr int kDecMaxG = 8;    // query heads per key/value head
 constexpr int kDecThreads = 6 * 32;
+constexpr int kDecMaxTokens = kAttnDecodeMaxTokens;
+static_assert(kDecMaxTokens == 4 * 32, "four tokens a lane in the set-up");
 constexpr int kDecStages = 3;     // key and value tiles in flight
 constexpr int kDecMaxSplit = 8;   // splits of one (token, key/value head): a portable cluster
-// the position tiles of a CTA are published in a ring: the producer
-// publishes its tile j once S_{j-3} has been computed (after the softmax
-// took S_{j-5}, so after it read tile j-5), so a slot is rewritten long
-// after both its readers (issuer, softmax) took it
+// query buffers: a piece's rows replace those of the piece four before it,
+// whose last tile is at least four tiles back; the stage the new piece's
+// first key tile goes to is free once the tile three back has been scored
+constexpr int kDecQBufs = 4;
+// the tiles of a CTA are described in a ring: the producer publishes its tile
+// j once S_{j-3} has been computed (after the softmax took S_{j-5}, so after
+// it read description j-5), so a slot is rewritten long after both its
+// readers (issuer, softmax) took it
 constexpr int kDecRing = 8;
 constexpr uint32_t kDecHalf = kDecPos * 128;  // one 64-dim box of a key/value tile: 16 KB
 constexpr uint32_t kDecTile = 2 * kDecHalf;   // 32 KB
 constexpr uint32_t kDecNHalf = kDecN * 128;   // 16 rows x 64 elements: 2 KB
 constexpr uint32_t kDecQ = 2 * kDecNHalf;     // query rows, 128 dims
 constexpr uint32_t kDecP = 2 * kDecNHalf;     // probabilities, 128 positions
-// shared memory (1024-byte aligned): K[3], V[3], Q, P[2], the O^T rows the
-// splits store for the heads this CTA merges, header
+// shared memory (1024-byte aligned): K[3], V[3], Q[4], P[2], header
 constexpr uint32_t kDecOffK = 0;
 constexpr uint32_t kDecOffV = kDecOffK + kDecStages * kDecTile;
 constexpr uint32_t kDecOffQ = kDecOffV + kDecStages * kDecTile;
-constexpr uint32_t kDecOffP = kDecOffQ + kDecQ;
-constexpr uint32_t kDecOffX = kDecOffP + 2 * kDecP;
-// [heads this CTA owns <= ceil(8 / n_split)][n_split][128] floats: at most
-// 14 rows (8 heads over 7 splits)
-constexpr uint32_t kDecXBytes = 14 * 128 * 4;
-constexpr uint32_t kDecOffHdr = kDecOffX + kDecXBytes;
-constexpr uint32_t kDecHdrBytes = 2048;
+constexpr uint32_t kDecOffP = kDecOffQ + kDecQBufs * kDecQ;
+constexpr uint32_t kDecOffHdr = kDecOffP + 2 * kDecP;
+// cluster: the O^T rows the splits store for the heads this CTA merges, where
+// the second to fourth query buffers are otherwise (a split has one piece):
+// [heads this CTA owns <= ceil(8 / n_split)][n_split][128] floats, at most 14
+// rows (8 heads over 7 splits)
+constexpr uint32_t kDecOffX = kDecOffQ + kDecQ;
+static_assert(14 * 128 * 4 <= (kDecQBufs - 1) * kDecQ, "the merge rows fit the query buffers");
+constexpr uint32_t kDecHdrBytes = 4096;
 constexpr size_t kDecSmem = 1024 + kDecOffHdr + kDecHdrBytes;
 static_assert(kDecSmem <= 227 * 1024, "shared memory");
 // kind::f16: bf16 A and B, fp32 D, M = 128, N = 16; A and B K-major
@@ -109,23 +135,50 @@ constexpr uint32_t kDecColS = 0, kDecColO = 2 * kDecN;
 // base-2 distance the tile maximum may run ahead of a head's exponent base
 constexpr float kDecRescale = 8.f;
 
+// One position tile of a CTA's share.
+struct DecDesc {
+    int tile;     // position tile of the sequence; -1: the share has ended
+    int tg;       // token * Hkv + key/value head
+    int n;        // positions the token attends to (0: outside the cache)
+    int flags;    // kDecFirst, kDecLast: of its piece; kDecWhole: the piece is the
+                  // whole (token, head); from bit 4: the query buffer
+    int b0, parts;  // not whole: the first CTA with a piece of it, and how many have one
+    int start;      // not whole: this piece is its start
+    int pad;
+};
+// a part's slot in the workspace: 8 rows of O^T, 8 pairs (base, sum)
+constexpr int kDecSlot = kDecMaxG * (128 + 2);
+static_assert(2 * kAttnDecodeMaxCtas * kDecSlot <= (int)kAttnDecodePartFloats, "two slots a CTA");
+// shares of fewer tiles than this leave SMs out: two tiles' copies are in
+// flight together and cost little more than one's, a part to merge 2-3 us
+constexpr int kDecMinTiles = 2;
+// a share's end inside a (token, head) of at most this many tiles moves to the
+// nearer end of it
+constexpr int kDecMaxWhole = 4;
+enum : int { kDecFirst = 1, kDecLast = 2, kDecWhole = 4, kDecQShift = 4 };
+
 struct DecHeader {
-    uint64_t q_full;
     uint64_t k_full[kDecStages], k_empty[kDecStages];  // key tile j in stage j % 3
     uint64_t v_full[kDecStages], v_empty[kDecStages];  // value tile j in stage j % 3
     uint64_t s_full[2];              // S_j written (buffer j % 2)
     uint64_t s_empty[2];             // S_j read by the four softmax warps
     uint64_t p_ready[2];             // P_j written (four softmax warps)
     uint64_t p_empty[2];             // P_j V_j finished
-    uint64_t t_full[kDecRing];       // tile index j of this CTA published (producer)
+    uint64_t t_full[kDecRing];       // description of tile j published (producer)
     uint64_t done;
-    uint64_t merge_full;             // every split's partials stored here (their bytes)
+    uint64_t merge_full;             // cluster: every split's partials stored here (their bytes)
     uint32_t tmem_base;
     uint32_t next_tile;              // the cluster's tile counter (in CTA 0)
-    int tidx[kDecRing];              // position tile of this CTA's j-th tile, -1 past the last
-    float red[2][4][kDecMaxG];  // the warps' tile maxima, by tile parity
+    int last;                        // this CTA counted last on its first (1), last (2) piece
+    int any;                         // the CTA's share has tiles
+    alignas(16) DecDesc desc[kDecRing];
+    float red[4][kDecMaxG];     // the warps' tile maxima
     float lsum[4][kDecMaxG];    // the warps' row sums at the end
-    alignas(8) float ml[kDecMaxG][kDecMaxSplit][2];  // (base, sum) of the owned heads, by split
+    alignas(8) float ml[kDecMaxG][kDecMaxSplit][2];  // cluster: (base, sum) of the owned heads
+    // the call's tokens: row of the caches' sequence, positions, and the
+    // position tiles of the tokens before it (entry T: of all of them)
+    int seq[kDecMaxTokens], n[kDecMaxTokens];
+    int before[kDecMaxTokens + 1];
 };
 static_assert(sizeof(DecHeader) <= kDecHdrBytes, "decode attention header");
 
@@ -257,187 +310,415 @@ __device__ __forceinline__ void dec_issue_pv(uint32_t d_tmem, uint32_t v_smem, u
     }
 }
 
+// The maximum over the warp (NaN scores give way to numbers, as with fmaxf).
+__device__ __forceinline__ float warp_max(float v) {
+    float m;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+    return m;
+}
+
+// Barrier over `threads` threads that also tells whether any of them had p.
+__device__ __forceinline__ bool named_bar_or(uint32_t id, uint32_t threads, bool p) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %3, 0;\n\t"
+        "barrier.cta.red.or.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(id), "r"(threads), "r"((uint32_t)p)
+        : "memory");
+    return r != 0;
+}
+
+// Shares of W tiles among G CTAs: CTA c starts at tile W c / G, and tile x is
+// in CTA ((x + 1) G - 1) / W.  (In 32 bits where the products fit: a 64-bit
+// division takes a few hundred cycles.)
+__device__ __forceinline__ long long dec_start(long long W, int c, int G) {
+    if (W < (1 << 24)) return (unsigned)W * (unsigned)c / (unsigned)G;
+    return W * c / G;
+}
+__device__ __forceinline__ int dec_owner(long long x, long long W, int G) {
+    if (W < (1 << 24)) return (int)((((unsigned)x + 1u) * (unsigned)G - 1u) / (unsigned)W);
+    return (int)(((x + 1) * G - 1) / W);
+}
+static_assert(kAttnDecodeMaxCtas < 256, "the 32-bit products of dec_start and dec_owner");
+
+// Row 0 of the group's heads in ctx.
 template <int G>
+__device__ __forceinline__ bf16 *dec_ctx(bf16 *ctx, int tg, int Hq, int Hkv) {
+    const int t = tg / Hkv, g = tg - t * Hkv;
+    return ctx + ((size_t)t * Hq + g * G) * 128;
+}
+
+// Weighted values over the sum of weights (a sum of probabilities of at most
+// 2^8 each: far inside the fast division's range); zero where nothing is.
+__device__ __forceinline__ bf16 dec_mean(float a, float s) {
+    return __float2bfloat16_rn(s > 0.f ? __fdividef(a, s) : 0.f);
+}
+
+// The parts of a (token, head) in the workspace, merged in order, thread r its
+// dim: part q is CTA b0 + q's, in its first slot (the start of the (token,
+// head), which ends CTA b0's share, in its second).  Four parts' loads go out
+// together, past L1.
+template <int G>
+__device__ __forceinline__ void dec_merge(const float *part, int b0, int parts, int r, bf16 *dst) {
+    float M[G], A[G], S[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+        M[h] = -INFINITY;
+        A[h] = S[h] = 0.f;
+    }
+    for (int q0 = 0; q0 < parts; q0 += 4) {
+        float2 bl[4][G];
+        float ov[4][G];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = q0 + u;
+            const float *pq = part + (size_t)(2 * (b0 + q) + (q == 0 ? 1 : 0)) * kDecSlot;
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+                bl[u][h] = make_float2(-INFINITY, 0.f);
+                ov[u][h] = 0.f;
+                if (q < parts) {
+                    bl[u][h] = __ldcg(reinterpret_cast<const float2 *>(pq + kDecMaxG * 128 + 2 * h));
+                    ov[u][h] = __ldcg(pq + h * 128 + r);
+                }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+            const float mn = fmaxf(M[h], fmaxf(fmaxf(bl[0][h].x, bl[1][h].x),
+                                               fmaxf(bl[2][h].x, bl[3][h].x)));
+            if (mn == -INFINITY) continue;  // parts of a wait that gave up
+            const float c = dec_exp2(M[h] - mn);
+            M[h] = mn;
+            A[h] *= c;
+            S[h] *= c;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float w = dec_exp2(bl[u][h].x - mn);
+                S[h] = fmaf(w, bl[u][h].y, S[h]);
+                A[h] = fmaf(w, ov[u][h], A[h]);
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < G; ++h) dst[h * 128] = dec_mean(A[h], S[h]);
+}
+
+// The token that holds tile x: the last with `before` tiles ahead of it.
+__device__ __forceinline__ int dec_token(const int *before, int T, int Hkv, long long x) {
+    int t = 0;
+    for (int step = kDecMaxTokens / 2; step > 0; step >>= 1)
+        if (t + step < T && (long long)before[t + step] * Hkv <= x) t += step;
+    return t;
+}
+
+// SPLIT: the n_split >= 2 CTAs of a cluster share one (token, key/value head);
+// otherwise n_split is 1 and every CTA has a share of all tiles.  (One kernel
+// that held both forms took 11.5-12.3 us where the cluster form alone takes
+// 10.6-12.0, one sequence of 300-2048 positions.)
+template <int G, bool SPLIT>
 __global__ void __launch_bounds__(kDecThreads, 1)
 k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                 const __grid_constant__ CUtensorMap tmV, int Hq, int Hkv, int n_seq, int L,
-                 int n_split, const int32_t *__restrict__ seq, const int32_t *__restrict__ pos,
-                 bf16 *__restrict__ ctx, unsigned *err) {
+                 const __grid_constant__ CUtensorMap tmV, int T, int Hq, int Hkv, int n_seq, int L,
+                 const int32_t *__restrict__ seq, const int32_t *__restrict__ pos,
+                 bf16 *__restrict__ ctx, float *__restrict__ part, int *__restrict__ count,
+                 int n_split, unsigned *err) {
     static_assert(G >= 1 && G <= kDecMaxG, "query heads per key/value head");
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     DecHeader *hd = reinterpret_cast<DecHeader *>(smem + kDecOffHdr);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s = blockIdx.x, tg = blockIdx.y;
-    const int t = tg / Hkv, g = tg - t * Hkv;
-    // the token's sequence and position are inputs of the call, complete
-    // before it in stream order (no kernel of the library writes them): read
-    // first, their latency behind the set-up
-    const int sq = seq[t], p = pos[t];
 
-    const int c = s;  // rank in the cluster (the splits of one pair)
-
-    if (threadIdx.x == 0) {
-        ptx::mbar_init(&hd->q_full, 1);
-        for (int b = 0; b < kDecStages; ++b) {
-            ptx::mbar_init(&hd->k_full[b], 1);
-            ptx::mbar_init(&hd->k_empty[b], 1);
-            ptx::mbar_init(&hd->v_full[b], 1);
-            ptx::mbar_init(&hd->v_empty[b], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(&hd->s_full[b], 1);
-            ptx::mbar_init(&hd->s_empty[b], 4);
-            ptx::mbar_init(&hd->p_ready[b], 4);
-            ptx::mbar_init(&hd->p_empty[b], 1);
-        }
-        for (int b = 0; b < kDecRing; ++b) ptx::mbar_init(&hd->t_full[b], 1);
-        ptx::mbar_init(&hd->done, 1);
-        ptx::mbar_init(&hd->merge_full, 1);
-        hd->next_tile = 0u;
-        if (n_split > 1) {
-            // the bytes every split stores here: an O^T row and (base, sum)
-            // for each head this CTA merges
-            const int owned = c < G ? (G - 1 - c) / n_split + 1 : 0;
-            ptx::mbar_arrive_expect_tx(&hd->merge_full,
-                                       (uint32_t)(n_split * owned * (kDecPos * 4 + 8)));
-        }
-        ptx::fence_barrier_init();
-        ptx::prefetch_tmap(&tmQ);
-        ptx::prefetch_tmap(&tmK);
-        ptx::prefetch_tmap(&tmV);
-    }
-    if (n_split > 1) {
-        // this CTA's barriers and tile counter are initialised: the
-        // cluster's other CTAs may use them once they pass the matching wait
-        // (the arrival releases thread 0's stores at cluster scope)
-        __syncthreads();
-        cluster_arrive_release();
-    }
-    if (warp == 1) tmem_alloc(&hd->tmem_base, kDecTmemCols);
+    const int cta = (int)blockIdx.x;
     // the output projection may launch now: it streams its weights into the
     // SMs this grid leaves free while the attention runs
     ptx::launch_dependents();
-    ptx::grid_dependency_wait();  // queries and caches come from the previous kernel
-    const bool ok = sq >= 0 && sq < n_seq && p >= 0 && p < L;
-    // the position tiles of the sequence: the splits share them, the first
-    // kDecStages of each split fixed (tile c + i n_split for split c), the
-    // rest taken one by one from a counter in CTA 0 of the cluster by
-    // whichever split frees a stage first (the splits' shares of the memory
-    // bandwidth differ); only the last tile of the sequence is partial
-    const int n = ok ? p + 1 : 0;
-    const int n_all = (n + kDecPos - 1) / kDecPos;
-    const int row0 = (sq * Hkv + g) * L;
-    int n_first = 0;  // fixed tiles of this split that exist
-    for (int i = 0; i < kDecStages; ++i) n_first += c + i * n_split < n_all ? 1 : 0;
-    // the producer (thread 0, which initialised the barriers) sends the
-    // query rows and the fixed tiles before the block-wide barrier: their
-    // stages are empty yet
-    if (threadIdx.x == 0) {
-        if (n_first > 0) {
-            const uint64_t pol_kv = ptx::policy_evict_first();  // read once
-            ptx::mbar_arrive_expect_tx(&hd->q_full, kDecQ);
-            for (int half = 0; half < 2; ++half)
-                ptx::tma_load_2d(smem + kDecOffQ + half * kDecNHalf, &tmQ, half * 64,
-                                 t * Hq + g * G, &hd->q_full, ptx::policy_evict_normal());
-            for (int j = 0; j < n_first; ++j) {
-                const int row = row0 + (c + j * n_split) * kDecPos;
-                ptx::mbar_arrive_expect_tx(&hd->k_full[j], kDecTile);
-                for (int half = 0; half < 2; ++half)
-                    ptx::tma_load_2d(smem + kDecOffK + j * kDecTile + half * kDecHalf, &tmK,
-                                     half * 64, row, &hd->k_full[j], pol_kv);
-                ptx::mbar_arrive_expect_tx(&hd->v_full[j], kDecTile);
-                for (int half = 0; half < 2; ++half)
-                    ptx::tma_load_2d(smem + kDecOffV + j * kDecTile + half * kDecHalf, &tmV,
-                                     half * 64, row, &hd->v_full[j], pol_kv);
-                hd->tidx[j] = c + j * n_split;
-                ptx::mbar_arrive(&hd->t_full[j]);
+
+    // The producer warp sets up the barriers, finds the CTA's share and sends
+    // its first tiles before the block-wide barrier.
+    // the next tile to send: token, head, tile of its sequence, and the
+    // sequence's tiles
+    struct At {
+        int t, g, tile, nt;
+    } at = {0, 0, 0, 1};
+    long long W = 0, lo = 0;
+    int total = 0, n_cta = 1, early = 0;
+    const uint64_t pol_kv = ptx::policy_evict_first();  // key and value tiles are read once
+    // the tile after a, this CTA's j-th; false: there is none.  A split's
+    // first kDecStages tiles are fixed (c, c + n_split, ...); `taken` is then
+    // the next one from the cluster's counter
+    auto advance = [&](At &a, int j, int taken) -> bool {
+        if constexpr (SPLIT) {
+            a.tile = j < kDecStages ? a.tile + n_split : taken;
+            return a.tile < a.nt;
+        }
+        if (j >= total) return false;
+        if (++a.tile == a.nt) {
+            a.tile = 0;
+            if (++a.g == Hkv) {
+                a.g = 0;
+                ++a.t;
+                a.nt = hd->before[a.t + 1] - hd->before[a.t];
             }
         }
-        if (n_first < kDecStages) {
-            // no tile past these: the end is published now
-            hd->tidx[n_first] = -1;
-            ptx::mbar_arrive(&hd->t_full[n_first]);
+        return true;
+    };
+    if (warp == 0) {
+        // the tokens' sequences and positions are inputs of the call, complete
+        // before it in stream order (no kernel of the library writes them):
+        // read first, their latency behind the set-up of the barriers.  A token
+        // outside the cache is given one tile with no valid position: its ctx
+        // is zero.
+        int tok_seq[4], tok_n[4];  // tokens 4 lane + i
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = 4 * lane + i;
+            tok_seq[i] = t < T ? seq[t] : -1;
+            tok_n[i] = t < T ? pos[t] : -1;
+        }
+        if (lane == 0) {
+            for (int b = 0; b < kDecStages; ++b) {
+                ptx::mbar_init(&hd->k_full[b], 1);
+                ptx::mbar_init(&hd->k_empty[b], 1);
+                ptx::mbar_init(&hd->v_full[b], 1);
+                ptx::mbar_init(&hd->v_empty[b], 1);
+            }
+            for (int b = 0; b < 2; ++b) {
+                ptx::mbar_init(&hd->s_full[b], 1);
+                ptx::mbar_init(&hd->s_empty[b], 4);
+                ptx::mbar_init(&hd->p_ready[b], 4);
+                ptx::mbar_init(&hd->p_empty[b], 1);
+            }
+            for (int b = 0; b < kDecRing; ++b) ptx::mbar_init(&hd->t_full[b], 1);
+            ptx::mbar_init(&hd->done, 1);
+            ptx::mbar_init(&hd->merge_full, 1);
+            hd->next_tile = 0u;
+            if constexpr (SPLIT) {
+                // the bytes every split stores here: an O^T row and (base, sum)
+                // for each head this CTA merges
+                const int c = cta % n_split;
+                const int owned = c < G ? (G - 1 - c) / n_split + 1 : 0;
+                ptx::mbar_arrive_expect_tx(&hd->merge_full,
+                                           (uint32_t)(n_split * owned * (kDecPos * 4 + 8)));
+            }
+            ptx::fence_barrier_init();
+            ptx::prefetch_tmap(&tmK);
+            ptx::prefetch_tmap(&tmV);
+            ptx::prefetch_tmap(&tmQ);
+        }
+        int nt[4], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = 4 * lane + i;
+            const bool ok = tok_seq[i] >= 0 && tok_seq[i] < n_seq && tok_n[i] >= 0 && tok_n[i] < L;
+            tok_seq[i] = ok ? tok_seq[i] : -1;
+            tok_n[i] = ok ? tok_n[i] + 1 : 0;
+            nt[i] = t < T ? max(1, (tok_n[i] + kDecPos - 1) / kDecPos) : 0;
+            sum += nt[i];
+            if (t < T) {
+                hd->seq[t] = ok ? tok_seq[i] : 0;
+                hd->n[t] = tok_n[i];
+            }
+        }
+        if constexpr (SPLIT) {
+            // a split: its first tile of the cluster's (token, head)
+            __syncwarp();
+            const int tg = cta / n_split;
+            at.t = tg / Hkv;
+            at.g = tg - at.t * Hkv;
+            at.tile = cta - tg * n_split;
+            at.nt = max(1, (hd->n[at.t] + kDecPos - 1) / kDecPos);
+            total = at.tile < at.nt ? 1 : 0;  // (whether it has any)
+        } else {
+            // the tiles before each token, and this CTA's share of all
+            int incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            int run = incl - sum;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                hd->before[4 * lane + i] = run;
+                run += nt[i];
+            }
+            if (lane == 31) hd->before[kDecMaxTokens] = run;
+            __syncwarp();
+            W = (long long)hd->before[kDecMaxTokens] * Hkv;
+            n_cta = (int)min((long long)gridDim.x,
+                             max(1LL, W < (1 << 24) ? (unsigned)W / (unsigned)kDecMinTiles
+                                                    : W / kDecMinTiles));
+            long long x = W;  // even lanes: the share's start, odd lanes: its end
+            if (cta + (lane & 1) < n_cta) {
+                x = dec_start(W, cta + (lane & 1), n_cta);
+                const int t = dec_token(hd->before, T, Hkv, x);
+                const int ntx = hd->before[t + 1] - hd->before[t];
+                if (ntx <= kDecMaxWhole) {
+                    const int o =
+                        (int)((unsigned)(x - (long long)hd->before[t] * Hkv) % (unsigned)ntx);
+                    x += 2 * o < ntx ? -o : ntx - o;
+                }
+            }
+            lo = __shfl_sync(0xffffffffu, x, 0);
+            total = (int)(__shfl_sync(0xffffffffu, x, 1) - lo);
+            at.t = dec_token(hd->before, T, Hkv, lo);
+            at.nt = hd->before[at.t + 1] - hd->before[at.t];
+            const long long in_t = lo - (long long)hd->before[at.t] * Hkv;
+            at.g = in_t < (1 << 30) ? (int)((unsigned)in_t / (unsigned)at.nt) : (int)(in_t / at.nt);
+            at.tile = (int)(in_t - (long long)at.g * at.nt);
+        }
+        if (lane == 0) hd->any = total > 0 ? 1 : 0;
+        // key and value tiles that no token of this call writes into (all of
+        // the sequence's positions in them lie before the call's first one)
+        // hold what earlier calls left, complete before the kernel ahead of
+        // this one began: the first stages of them are loaded before the wait
+        // for that kernel
+        At a = at;
+        bool have = total > 0;
+#pragma unroll 1
+        for (int j = 0; j < kDecStages && have; ++j) {
+            const int sq = hd->seq[a.t];
+            int first_pos = 0x7fffffff;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (tok_seq[i] == sq) first_pos = min(first_pos, tok_n[i] - 1);
+            first_pos = __reduce_min_sync(0xffffffffu, first_pos);
+            if (hd->n[a.t] > 0 && (a.tile + 1) * kDecPos <= first_pos) {
+                early |= 1 << j;
+                if (lane == 0) {
+                    const int row = (sq * Hkv + a.g) * L + a.tile * kDecPos;
+                    const bool first = j == 0 || (!SPLIT && a.tile == 0);
+                    ptx::mbar_arrive_expect_tx(&hd->k_full[j], kDecTile + (first ? kDecQ : 0u));
+                    ptx::mbar_arrive_expect_tx(&hd->v_full[j], kDecTile);
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffK + j * kDecTile + half * kDecHalf, &tmK,
+                                         half * 64, row, &hd->k_full[j], pol_kv);
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffV + j * kDecTile + half * kDecHalf, &tmV,
+                                         half * 64, row, &hd->v_full[j], pol_kv);
+                }
+            }
+            have = j + 1 < kDecStages && advance(a, j + 1, 0);
         }
     }
+    if (warp == 1) tmem_alloc(&hd->tmem_base, kDecTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // this CTA's barriers are initialised: the cluster's other CTAs may store
+    // to it once they pass the matching wait (the arrival releases the
+    // initialising thread's stores at cluster scope)
+    if constexpr (SPLIT) cluster_arrive_release();
     const uint32_t tmem = hd->tmem_base;
     const uint32_t sbase = ptx::smem_u32(smem);
+    const bool any = hd->any != 0;  // the share has tiles
+    ptx::grid_dependency_wait();    // queries and new cache rows come from the previous kernel
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        // (CTA 0's counter is initialised before the first take)
-        if (n_split > 1) cluster_wait();
-        if (lane == 0 && n_first == kDecStages) {
-            const uint64_t pol_kv = ptx::policy_evict_first();
+        const uint64_t pol_q = ptx::policy_evict_normal();
+        if (lane == 0 && any) {  // the first piece's query rows
+            if (!(early & 1)) ptx::mbar_arrive_expect_tx(&hd->k_full[0], kDecTile + kDecQ);
+            for (int half = 0; half < 2; ++half)
+                ptx::tma_load_2d(smem + kDecOffQ + half * kDecNHalf, &tmQ, half * 64,
+                                 at.t * Hq + at.g * G, &hd->k_full[0], pol_q);
+        }
+        if constexpr (SPLIT) cluster_wait();  // CTA 0's counter is initialised before the first take
+        if (lane == 0) {
             const uint32_t counter = ptx::map_rank(ptx::smem_u32(&hd->next_tile), 0u);
-            // the next tile is taken one ahead: its counter round trip runs
-            // while the stage it goes to frees
-            int taken = 0;  // (a single split counts alone)
-            auto take = [&]() -> int {
-                return kDecStages * n_split +
-                       (n_split > 1 ? (int)dec_take(counter) : taken++);
-            };
-            int nxt = take();
-            int k_issued = kDecStages, v_issued = kDecStages;
-            for (int j = kDecStages;; ++j) {
-                const int tile = nxt;
-                if (tile >= n_all) {
-                    hd->tidx[j % kDecRing] = -1;
+            int piece = -1, k_issued = 0, v_issued = 0, taken = 0;
+            DecDesc d;
+            At nxt = at;
+            bool have = total > 0;
+            bool more = have && advance(nxt, 1, 0);
+            for (int j = 0;; ++j) {
+                const int b = j % kDecStages;
+                const uint32_t ph = ((j / kDecStages) & 1) ^ 1;
+                if (!have) {
+                    hd->desc[j % kDecRing].tile = -1;
                     ptx::mbar_arrive(&hd->t_full[j % kDecRing]);
                     break;
                 }
-                nxt = take();
-                const int b = j % kDecStages;
-                const uint32_t ph = ((j / kDecStages) & 1) ^ 1;
-                const int row = row0 + tile * kDecPos;
+                // (taken two tiles ahead: the counter's round trip runs while
+                // a stage frees)
+                if (SPLIT && more && j + 2 >= kDecStages)
+                    taken = kDecStages * n_split + (int)dec_take(counter);
+                const bool first = j == 0 || (!SPLIT && at.tile == 0);
+                const bool last = !more || (!SPLIT && at.tile == at.nt - 1);
+                if (first) {
+                    ++piece;
+                    d.tg = at.t * Hkv + at.g;
+                    d.n = hd->n[at.t];
+                    const bool whole = !SPLIT && at.tile == 0 && at.nt <= total - j;
+                    d.b0 = d.parts = d.start = d.pad = 0;
+                    if (!whole && !SPLIT) {
+                        const long long f0 = lo + j - at.tile;  // the (token, head)'s first tile
+                        d.b0 = dec_owner(f0, W, n_cta);
+                        d.parts = dec_owner(f0 + at.nt - 1, W, n_cta) - d.b0 + 1;
+                        d.start = at.tile == 0 ? 1 : 0;
+                    }
+                    d.flags = (whole ? kDecWhole : 0) | ((piece % kDecQBufs) << kDecQShift);
+                }
+                d.tile = at.tile;
+                d.flags = (d.flags & ~(kDecFirst | kDecLast)) | (first ? kDecFirst : 0) |
+                          (last ? kDecLast : 0);
+                const int row = (hd->seq[at.t] * Hkv + at.g) * L + at.tile * kDecPos;
+                const bool sent = j < kDecStages && ((early >> j) & 1);  // before the wait above
                 if (!dec_wait(&hd->k_empty[b], ph, err)) break;
-                ptx::mbar_arrive_expect_tx(&hd->k_full[b], kDecTile);
-                for (int half = 0; half < 2; ++half)
-                    ptx::tma_load_2d(smem + kDecOffK + b * kDecTile + half * kDecHalf, &tmK,
-                                     half * 64, row, &hd->k_full[b], pol_kv);
+                if (!sent && j > 0)
+                    ptx::mbar_arrive_expect_tx(&hd->k_full[b], kDecTile + (first ? kDecQ : 0u));
+                if (first && j > 0)
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffQ + (piece % kDecQBufs) * kDecQ +
+                                             half * kDecNHalf,
+                                         &tmQ, half * 64, at.t * Hq + at.g * G, &hd->k_full[b],
+                                         pol_q);
+                if (!sent)
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffK + b * kDecTile + half * kDecHalf, &tmK,
+                                         half * 64, row, &hd->k_full[b], pol_kv);
                 k_issued = j + 1;
-                hd->tidx[j % kDecRing] = tile;
+                hd->desc[j % kDecRing] = d;
                 ptx::mbar_arrive(&hd->t_full[j % kDecRing]);
                 if (!dec_wait(&hd->v_empty[b], ph, err)) break;
-                ptx::mbar_arrive_expect_tx(&hd->v_full[b], kDecTile);
-                for (int half = 0; half < 2; ++half)
-                    ptx::tma_load_2d(smem + kDecOffV + b * kDecTile + half * kDecHalf, &tmV,
-                                     half * 64, row, &hd->v_full[b], pol_kv);
+                if (!sent) {
+                    ptx::mbar_arrive_expect_tx(&hd->v_full[b], kDecTile);
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffV + b * kDecTile + half * kDecHalf, &tmV,
+                                         half * 64, row, &hd->v_full[b], pol_kv);
+                }
                 v_issued = j + 1;
+                at = nxt;
+                have = more;
+                more = more && advance(nxt, j + 2, taken);
             }
             // copies still in flight land before the block can exit
-            dec_wait(&hd->q_full, 0, err);
             for (int j = std::max(0, k_issued - kDecStages); j < k_issued; ++j)
                 dec_wait(&hd->k_full[j % kDecStages], (j / kDecStages) & 1, err);
             for (int j = std::max(0, v_issued - kDecStages); j < v_issued; ++j)
                 dec_wait(&hd->v_full[j % kDecStages], (j / kDecStages) & 1, err);
-        } else if (lane == 0 && n_first > 0) {
-            dec_wait(&hd->q_full, 0, err);
-            for (int j = 0; j < n_first; ++j) {
-                dec_wait(&hd->k_full[j], 0, err);
-                dec_wait(&hd->v_full[j], 0, err);
-            }
         }
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && n_first > 0) {
-            bool good = dec_wait(&hd->q_full, 0, err) && dec_wait(&hd->k_full[0], 0, err);
+        if (lane == 0 && any) {
+            bool good = dec_wait(&hd->t_full[0], 0, err) && dec_wait(&hd->k_full[0], 0, err);
             if (good) {
                 tc_fence_after();
                 dec_issue_qk(tmem + kDecColS, sbase + kDecOffK, sbase + kDecOffQ);
                 mma_commit(&hd->s_full[0]);
                 mma_commit(&hd->k_empty[0]);
             }
+            bool first = true;  // tile j is its piece's first
             for (int j = 0; good; ++j) {
                 // is there a tile j + 1 (published by the producer)?
                 const int r1 = (j + 1) % kDecRing;
                 if (!(good = dec_wait(&hd->t_full[r1], ((j + 1) / kDecRing) & 1, err))) break;
-                const bool more = hd->tidx[r1] >= 0;
+                const bool more = hd->desc[r1].tile >= 0;
+                const int fl1 = more ? hd->desc[r1].flags : 0;
                 if (more) {
                     // S_{j+1} into the buffer of S_{j-1}, once the softmax has read it
                     const int sb1 = (j + 1) & 1, kb1 = (j + 1) % kDecStages;
@@ -446,7 +727,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     if (!good) break;
                     tc_fence_after();
                     dec_issue_qk(tmem + kDecColS + sb1 * kDecN, sbase + kDecOffK + kb1 * kDecTile,
-                                 sbase + kDecOffQ);
+                                 sbase + kDecOffQ + (uint32_t)(fl1 >> kDecQShift) * kDecQ);
                     mma_commit(&hd->s_full[sb1]);
                     mma_commit(&hd->k_empty[kb1]);
                 }
@@ -455,11 +736,14 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                        dec_wait(&hd->p_ready[pb], (j >> 1) & 1, err);
                 if (!good) break;
                 tc_fence_after();
+                // (P_j of a piece's first tile comes after the softmax has
+                // taken the piece before it out of O)
                 dec_issue_pv(tmem + kDecColO, sbase + kDecOffV + vb * kDecTile,
-                             sbase + kDecOffP + pb * kDecP, j != 0);
+                             sbase + kDecOffP + pb * kDecP, !first);
                 mma_commit(&hd->p_empty[pb]);
                 mma_commit(&hd->v_empty[vb]);
                 if (!more) break;
+                first = (fl1 & kDecFirst) != 0;
             }
             mma_commit(&hd->done);
             dec_wait(&hd->done, 0, err);
@@ -478,29 +762,44 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 half[kPadRow + i % kPad] = make_uint4(0u, 0u, 0u, 0u);
             }
         }
-        // every CTA of the cluster has initialised its barriers before this
-        // one's merge stores (waited here, long before they are needed)
-        if (n_split > 1) cluster_wait();
         const int qd = warp & 3;       // tensor-memory lane quarter
         const int r = qd * 32 + lane;  // position of the tile; dim of O^T
         const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
         const float sl2 = 1.4426950408889634f / sqrtf(128.f);
-        float base[G], l[G];
+        // every CTA of the cluster has initialised its barriers before this
+        // one's merge stores (waited here, long before they are needed)
+        if constexpr (SPLIT) cluster_wait();
+        float base[G], l[G], o[16], Ls[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) {
             base[h] = -INFINITY;
-            l[h] = 0.f;
+            l[h] = Ls[h] = 0.f;
         }
-        bool good = true;
-        int had = 0;  // tiles this split has had
-        for (int j = 0;; ++j) {
+#pragma unroll
+        for (int h = 0; h < 16; ++h) o[h] = 0.f;
+        // the share's first and last piece where they are parts of a (token,
+        // head) of which other CTAs hold parts too (parts > 0): which, the
+        // first CTA with a part, how many
+        int pend_tg[2], pend_b0[2], pend_parts[2] = {0, 0};
+        bool good = any;  // (an empty share has nothing to wait for)
+        for (int j = 0; any; ++j) {
             const int b = j & 1;
             good = good && dec_wait(&hd->t_full[j % kDecRing], (j / kDecRing) & 1, err);
             // (lane 0's reading steers the warp: its loop stays converged)
-            const int tile =
-                __shfl_sync(0xffffffffu, good ? hd->tidx[j % kDecRing] : -1, 0);
+            const DecDesc *dj = &hd->desc[j % kDecRing];
+            const int tile = __shfl_sync(0xffffffffu, good ? dj->tile : -1, 0);
             if (tile < 0) break;
-            had = j + 1;
+            const int n = __shfl_sync(0xffffffffu, dj->n, 0);
+            const int flags = __shfl_sync(0xffffffffu, dj->flags, 0);
+            const int tg = __shfl_sync(0xffffffffu, dj->tg, 0);
+            const int b0 = dj->b0, parts = dj->parts, start = dj->start;
+            if (flags & kDecFirst) {
+#pragma unroll
+                for (int h = 0; h < G; ++h) {
+                    base[h] = -INFINITY;
+                    l[h] = 0.f;
+                }
+            }
             const int pj = tile * kDecPos + r;
             const bool valid = pj < n;
             // (the load runs on every lane whatever its waits returned: it is
@@ -513,27 +812,35 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&hd->s_empty[b]);
-            // the tile maximum of every head (finite: the tile has a valid position)
-            float x[G];
+            // the exponent base of a head moves when a score of the tile
+            // passes it by more than 8 (always on a piece's first tile, whose
+            // bases are -inf); only then the tile maxima are formed: a warp
+            // maximum, then the four warps' through shared memory.  (A token
+            // outside the cache has no valid position: nothing moves.)
+            float x[G], corr[G];
+            bool over = false;
 #pragma unroll
             for (int h = 0; h < G; ++h) {
                 x[h] = valid ? v[h] * sl2 : -INFINITY;
-                float m = x[h];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if (lane == 0) hd->red[b][qd][h] = m;
+                corr[h] = 1.f;
+                over |= x[h] > base[h] + kDecRescale;
             }
-            ptx::named_bar_sync(1, 128);
-            float corr[G];
-            bool bump_any = false;
+            const bool bump_any = (flags & kDecFirst) || named_bar_or(1, 128, over);
+            if (bump_any) {
 #pragma unroll
-            for (int h = 0; h < G; ++h) {
-                const float tm = fmaxf(fmaxf(hd->red[b][0][h], hd->red[b][1][h]),
-                                       fmaxf(hd->red[b][2][h], hd->red[b][3][h]));
-                const bool bump = tm > base[h] + kDecRescale;
-                corr[h] = bump ? exp2f(base[h] - tm) : 1.f;  // 0 on the first tile
-                if (bump) base[h] = tm;
-                bump_any |= bump;
+                for (int h = 0; h < G; ++h) {
+                    const float m = warp_max(x[h]);
+                    if (lane == 0) hd->red[qd][h] = m;
+                }
+                ptx::named_bar_sync(1, 128);
+#pragma unroll
+                for (int h = 0; h < G; ++h) {
+                    const float tm = fmaxf(fmaxf(hd->red[0][h], hd->red[1][h]),
+                                           fmaxf(hd->red[2][h], hd->red[3][h]));
+                    const bool bump = tm > base[h] + kDecRescale;
+                    corr[h] = bump ? exp2f(base[h] - tm) : 1.f;  // 0 on the first tile
+                    if (bump) base[h] = tm;
+                }
             }
             // P_j into buffer b, free once P_{j-2} V_{j-2} has finished
             good = good && (j < 2 || dec_wait(&hd->p_empty[b], ((j - 2) >> 1) & 1, err));
@@ -564,78 +871,91 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             }
             // a moved base rescales O^T (each thread its dim's row) once
             // P_{j-1} V_{j-1} has finished; P_j V_j waits for this warp
-            if (j >= 1 && bump_any) {
+            if (!(flags & kDecFirst) && bump_any) {
                 good = good && dec_wait(&hd->p_empty[(j - 1) & 1], ((j - 1) >> 1) & 1, err);
                 if (__all_sync(0xffffffffu, good)) {
                     tc_fence_after();
-                    float o[16];
-                    tmem_ld16(tmem + lane_base + kDecColO, o);
+                    float so[16];
+                    tmem_ld16(tmem + lane_base + kDecColO, so);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int h = 0; h < G; ++h) o[h] *= corr[h];
-                    tmem_st16(tmem + lane_base + kDecColO, o);
+                    for (int h = 0; h < G; ++h) so[h] *= corr[h];
+                    tmem_st16(tmem + lane_base + kDecColO, so);
                 }
             }
             fence_proxy_async_smem();  // P_j and the zeroed value rows
             tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&hd->p_ready[b]);
-        }
-        // the split's result: O^T row r (dim r) of every head, the row sums
-        // of the four warps added in warp order
-        bool fin = good && had > 0;
-        if (fin) fin = dec_wait(&hd->p_empty[(had - 1) & 1], ((had - 1) >> 1) & 1, err);
-        fin = __all_sync(0xffffffffu, fin);
-#pragma unroll
-        for (int h = 0; h < G; ++h) {
-            const float ws = warp_sum(l[h]);
-            if (lane == 0) hd->lsum[qd][h] = ws;
-        }
-        ptx::named_bar_sync(1, 128);
-        float o[16];
-#pragma unroll
-        for (int h = 0; h < 16; ++h) o[h] = 0.f;
-        if (fin) {
-            tc_fence_after();
-            tmem_ld16(tmem + lane_base + kDecColO, o);
-            tmem_ld_wait();
-        }
-        if (n_split == 1) {
+            if (!(flags & kDecLast)) continue;
+
+            // the piece's result: O^T row r (dim r) of every head, the row
+            // sums of the four warps added in warp order
+            bool fin = good && dec_wait(&hd->p_empty[b], (j >> 1) & 1, err);
+            fin = __all_sync(0xffffffffu, fin);
+            good = good && fin;
 #pragma unroll
             for (int h = 0; h < G; ++h) {
-                const float Ls = fin ? (hd->lsum[0][h] + hd->lsum[1][h]) +
-                                           (hd->lsum[2][h] + hd->lsum[3][h])
-                                     : 0.f;
-                ctx[((size_t)t * Hq + g * G + h) * 128 + r] =
-                    __float2bfloat16_rn(Ls > 0.f ? __fdividef(o[h], Ls) : 0.f);
+                const float ws = warp_sum(l[h]);
+                if (lane == 0) hd->lsum[qd][h] = ws;
             }
-        } else {
-            float *xo = reinterpret_cast<float *>(smem + kDecOffX);
+            ptx::named_bar_sync(1, 128);
+            if (fin) {
+                tc_fence_after();
+                tmem_ld16(tmem + lane_base + kDecColO, o);
+                tmem_ld_wait();
+                tc_fence_before();
+            }
+#pragma unroll
+            for (int h = 0; h < G; ++h)
+                Ls[h] = fin ? (hd->lsum[0][h] + hd->lsum[1][h]) + (hd->lsum[2][h] + hd->lsum[3][h])
+                            : 0.f;
+            if constexpr (SPLIT) continue;  // (the share's only piece)
+            if (flags & kDecWhole) {
+                bf16 *dst = dec_ctx<G>(ctx, tg, Hq, Hkv) + r;
+#pragma unroll
+                for (int h = 0; h < G; ++h) dst[h * 128] = dec_mean(o[h], Ls[h]);
+                continue;
+            }
+            // a part: its slot holds G rows of O^T, then G pairs (base, sum)
+            float *mine = part + (size_t)(2 * cta + start) * kDecSlot;
 #pragma unroll
             for (int h = 0; h < G; ++h) {
-                // head h belongs to CTA h % n_split, row slot h / n_split;
-                // the stores count their bytes on the owner's merge barrier
+                mine[h * 128 + r] = o[h];
+                if (r == 0)
+                    *reinterpret_cast<float2 *>(mine + kDecMaxG * 128 + 2 * h) =
+                        make_float2(fin ? base[h] : -INFINITY, Ls[h]);
+            }
+            // (start 0: the share begins inside the (token, head))
+            if (start) pend_tg[1] = tg, pend_b0[1] = b0, pend_parts[1] = parts;
+            else pend_tg[0] = tg, pend_b0[0] = b0, pend_parts[0] = parts;
+        }
+        if constexpr (SPLIT) {
+            // every split sends its part of head h to the CTA that owns it,
+            // h % n_split, row slot h / n_split; the stores count their bytes
+            // on the owner's merge barrier
+            float *xo = reinterpret_cast<float *>(smem + kDecOffX);
+            const int tg = cta / n_split, c = cta - tg * n_split;
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
                 const uint32_t owner = (uint32_t)(h % n_split);
                 const int slot = h / n_split;
                 st_async_f32(&xo[((size_t)slot * n_split + c) * 128 + r], owner, &hd->merge_full,
-                             fin ? o[h] : 0.f);
-                if (r == 0) {
-                    const float Ls = fin ? (hd->lsum[0][h] + hd->lsum[1][h]) +
-                                               (hd->lsum[2][h] + hd->lsum[3][h])
-                                         : 0.f;
+                             good ? o[h] : 0.f);
+                if (r == 0)
                     st_async_v2f32(&hd->ml[slot][c][0], owner, &hd->merge_full,
-                                   fin ? base[h] : -INFINITY, Ls);
-                }
+                                   good ? base[h] : -INFINITY, good ? Ls[h] : 0.f);
             }
             // the heads this CTA owns (base 2: split weight 2^(base_s - M)),
             // once every split's bytes have landed
             const bool got = ptx::mbar_wait_cluster(&hd->merge_full, 0, err);
+            bf16 *dst = dec_ctx<G>(ctx, tg, Hq, Hkv) + r;
             // (unrolled to the bounds and predicated, so that the heads' and
             // the splits' loads go out together: n_split >= 2 leaves at most
             // (G + 1) / 2 heads to a CTA)
 #pragma unroll
             for (int slot = 0; slot < (G + 1) / 2; ++slot) {
-                const int h = (int)c + slot * n_split;
+                const int h = c + slot * n_split;
                 if (!got || h >= G) continue;
                 float bq[kDecMaxSplit], M = -INFINITY;
 #pragma unroll
@@ -643,91 +963,165 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     bq[q] = q < n_split ? hd->ml[slot][q][0] : -INFINITY;
                     M = fmaxf(M, bq[q]);
                 }
-                float A = 0.f, Ls = 0.f;
+                float A = 0.f, S = 0.f;
                 if (M != -INFINITY) {
 #pragma unroll
                     for (int q = 0; q < kDecMaxSplit; ++q) {
                         if (q < n_split) {
                             const float w = dec_exp2(bq[q] - M);
-                            Ls = fmaf(w, hd->ml[slot][q][1], Ls);
+                            S = fmaf(w, hd->ml[slot][q][1], S);
                             A = fmaf(w, xo[(slot * n_split + q) * 128 + r], A);
                         }
                     }
                 }
-                // (Ls is a sum of probabilities of at most 2^8 each: far
-                // inside the fast division's range)
-                ctx[((size_t)t * Hq + g * G + h) * 128 + r] =
-                    __float2bfloat16_rn(Ls > 0.f ? __fdividef(A, Ls) : 0.f);
+                dst[h * 128] = dec_mean(A, S);
             }
+        } else if (pend_parts[0] > 0 || pend_parts[1] > 0) {
+            // count this share's parts; the CTA that counts last on a (token,
+            // head) finds every part of it stored
+            ptx::named_bar_sync(1, 128);
+            if (r == 0) {
+                __threadfence();  // the warps' stores (ordered by the barrier) before the counts
+                int last = 0;
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (pend_parts[i] > 0 &&
+                        atomicAdd(&count[pend_b0[i]], 1) == pend_parts[i] - 1)
+                        last |= 1 << i;
+                hd->last = last;
+                __threadfence();  // the counts before the loads of the other parts
+            }
+            ptx::named_bar_sync(1, 128);
+#pragma unroll 1
+            for (int i = 0; i < 2; ++i)
+                if ((hd->last >> i) & 1)
+                    dec_merge<G>(part, pend_b0[i], pend_parts[i], r,
+                                 dec_ctx<G>(ctx, pend_tg[i], Hq, Hkv) + r);
         }
     }
-    // (the aligned wait of every thread: producer and softmax warps waited
-    // at their start)
-    if (n_split > 1 && warp == 1) cluster_wait();
+    // (the aligned wait of every thread: the others waited at their start)
+    if (SPLIT && warp == 1) cluster_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem, kDecTmemCols);
 }
 
+template <bool SPLIT>
+const void *dec_kernel(int G) {
+    switch (G) {
+        case 1: return (const void *)k_attn_decode_tc<1, SPLIT>;
+        case 2: return (const void *)k_attn_decode_tc<2, SPLIT>;
+        case 3: return (const void *)k_attn_decode_tc<3, SPLIT>;
+        case 4: return (const void *)k_attn_decode_tc<4, SPLIT>;
+        case 5: return (const void *)k_attn_decode_tc<5, SPLIT>;
+        case 6: return (const void *)k_attn_decode_tc<6, SPLIT>;
+        case 7: return (const void *)k_attn_decode_tc<7, SPLIT>;
+        default: return (const void *)k_attn_decode_tc<8, SPLIT>;
+    }
+}
+
+// Clusters of c CTAs of this kernel the current device keeps resident at once
+// (GPCs hold a whole number of clusters: 15 of 8 CTAs and 23 of 6 on a GB300's
+// 152 SMs; a call that needs one more waits for a whole wave), looked up once
+// per device.
+struct DecClusters {
+    int resident[kDecMaxSplit + 1];
+};
+
+const DecClusters &dec_clusters() {
+    static DecClusters info[64];
+    static std::once_flag once[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+    std::call_once(once[dev], [dev] {
+        const void *kern = (const void *)k_attn_decode_tc<1, true>;
+        const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kDecSmem) == cudaSuccess;
+        for (int c = 2; c <= kDecMaxSplit; ++c) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(c * kAttnDecodeMaxCtas);
+            cfg.blockDim = dim3(kDecThreads);
+            cfg.dynamicSmemBytes = kDecSmem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = c;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (!ok || cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) n = 0;
+            info[dev].resident[c] = n;
+        }
+        (void)cudaGetLastError();
+    });
+    return info[dev];
+}
+
+// CTAs for each of `pairs` (token, key/value head)s: the largest cluster that
+// is resident for all of them at once (attention block of DBRX at 2 sequences
+// of 2048 positions: 6 CTAs 50.0 us, 8 CTAs, one cluster left over, 54.3 us).
+// 1: the shares of all tiles.  They lose to clusters while those fill the SMs
+// (8 sequences: 59.4 against 57.0 us at 2048 positions, the same up to 4096)
+// -- a part left in the workspace costs its CTA a fence and a count, the
+// merging CTA two more trips to L2 -- and win where clusters would leave more
+// than a quarter of the SMs out (6 sequences, clusters of 2: 63.5 against 65.5
+// us up to 4096 positions, 58.8 against 57.4 us at 2048), unless there are so
+// few (token, head)s that most would be merged (2 sequences: 53-56 us).
+int dec_splits(int pairs, int max_tiles, int sms) {
+    const DecClusters &dc = dec_clusters();
+    int n = std::min(max_tiles, kDecMaxSplit);
+    while (n > 1 && dc.resident[n] < pairs) --n;
+    if (4 * n * pairs < 3 * sms && 4 * pairs > sms) n = 1;
+    return std::max(1, n);
+}
+
 }  // namespace
 
 bool attn_decode_tc_ok() { return encode_fn() != nullptr; }
 
-int attn_decode_tc_splits(int T, int Hkv, int max_len) {
-    // one wave of one-CTA-per-SM blocks, at least one position tile a
-    // split, at most a portable cluster of splits
-    const int tg = std::max(1, T * Hkv);
-    int ns = std::max(1, device_info().sm_count / tg);
-    ns = std::min(ns, (max_len + kDecPos - 1) / kDecPos);
-    return std::max(1, std::min(ns, kDecMaxSplit));
-}
-
-cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, int n_split,
-                                  const int32_t *seq, const int32_t *pos, const void *q16,
-                                  const void *k_cache, const void *v_cache, void *ctx,
+cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
+                                  const int32_t *pos, const void *q16, const void *k_cache,
+                                  const void *v_cache, void *ctx, float *part, int *count,
                                   cudaStream_t st) {
     const int G = Hq / Hkv;
-    if (G < 1 || G > kDecMaxG || G * Hkv != Hq || n_split < 1 || n_split > kDecMaxSplit)
+    if (G < 1 || G > kDecMaxG || G * Hkv != Hq || T < 1 || T > kDecMaxTokens)
         return cudaErrorInvalidValue;
     CUtensorMap mq, mk, mv;
     const uint64_t rows = (uint64_t)n_seq * Hkv * L;
     if (!make_map(&mq, q16, (uint64_t)T * Hq, 128, kDecN) ||
         !make_map(&mk, k_cache, rows, 128, kDecPos) || !make_map(&mv, v_cache, rows, 128, kDecPos))
         return cudaErrorInvalidValue;
-    const void *kern = nullptr;
-    switch (G) {
-        case 1: kern = (const void *)k_attn_decode_tc<1>; break;
-        case 2: kern = (const void *)k_attn_decode_tc<2>; break;
-        case 3: kern = (const void *)k_attn_decode_tc<3>; break;
-        case 4: kern = (const void *)k_attn_decode_tc<4>; break;
-        case 5: kern = (const void *)k_attn_decode_tc<5>; break;
-        case 6: kern = (const void *)k_attn_decode_tc<6>; break;
-        case 7: kern = (const void *)k_attn_decode_tc<7>; break;
-        default: kern = (const void *)k_attn_decode_tc<8>; break;
-    }
+    unsigned *err = device_info().err;
+    bf16 *cp = static_cast<bf16 *>(ctx);
+    int Tv = T, Hqv = Hq, Hkvv = Hkv, ns = n_seq, Lv = L;
+    // few (token, key/value head)s: a cluster of CTAs for each; otherwise one
+    // share of all tiles per SM
+    const int pairs = T * Hkv, sms = std::min(device_info().sm_count, kAttnDecodeMaxCtas);
+    const int max_tiles = (L + kDecPos - 1) / kDecPos;
+    int n_split = dec_splits(pairs, max_tiles, sms);
+    const void *kern = n_split > 1 ? dec_kernel<true>(G) : dec_kernel<false>(G);
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
     if (e != cudaSuccess) return e;
-    unsigned *err = device_info().err;
-    bf16 *cp = static_cast<bf16 *>(ctx);
-    int Hqv = Hq, Hkvv = Hkv, ns = n_seq, Lv = L, nsp = n_split;
-    void *args[] = {&mq, &mk, &mv, &Hqv, &Hkvv, &ns, &Lv, &nsp, &seq, &pos, &cp, &err};
-    // the splits of a (token, key/value head) form one cluster
+    void *args[] = {&mq,  &mk,  &mv, &Tv,   &Hqv,   &Hkvv,    &ns, &Lv,
+                    &seq, &pos, &cp, &part, &count, &n_split, &err};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_split, T * Hkv);
+    cfg.gridDim = dim3(n_split > 1 ? (unsigned)(n_split * pairs)
+                                   : (unsigned)std::min<long long>((long long)pairs * max_tiles, sms));
     cfg.blockDim = dim3(kDecThreads);
     cfg.dynamicSmemBytes = kDecSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = n_split;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = n_split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = n_split > 1 ? 2 : 1;
     LaunchScope ls("attention_decode_tc", st);
     return cudaLaunchKernelExC(&cfg, kern, args);
 }

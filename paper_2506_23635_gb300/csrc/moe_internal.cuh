@@ -273,17 +273,19 @@ bool attn_prefill_tc_ok();
 cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
                                    const int32_t *pos, const void *q16, const void *k_cache,
                                    const void *v_cache, void *ctx, int *tile_ok, cudaStream_t st);
-// Decode attention on the tensor cores (attn_decode_tc.cu): every token of
-// the call over positions 0..pos[t] of its sequence, in n_split (<= 8)
-// position splits per (token, key/value head) that form a cluster and merge
-// through distributed shared memory; ctx written.  Queries as above; query
-// heads per key/value head <= 8.  attn_decode_tc_splits: the split count for
-// one wave of CTAs.
+// Decode attention on the tensor cores (attn_decode_tc.cu): every token of a
+// call of up to kAttnDecodeMaxTokens over positions 0..pos[t] of its
+// sequence; ctx written.  Queries as above; query heads per key/value head
+// <= 8.  part: kAttnDecodePartFloats floats for the results of (token,
+// key/value head)s that several CTAs share; count: kAttnDecodeMaxCtas ints,
+// zero at the start (the kernel that writes q16 zeroes them).
+constexpr int kAttnDecodeMaxTokens = 128;
+constexpr int kAttnDecodeMaxCtas = 160;
+constexpr size_t kAttnDecodePartFloats = (size_t)2 * kAttnDecodeMaxCtas * 8 * (128 + 2);
 bool attn_decode_tc_ok();
-int attn_decode_tc_splits(int T, int Hkv, int max_len);
-cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, int n_split,
-                                  const int32_t *seq, const int32_t *pos, const void *q16,
-                                  const void *k_cache, const void *v_cache, void *ctx,
+cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
+                                  const int32_t *pos, const void *q16, const void *k_cache,
+                                  const void *v_cache, void *ctx, float *part, int *count,
                                   cudaStream_t st);
 
 // name: the profiling name of the launch (default "gemm_down_tc").  y_tail

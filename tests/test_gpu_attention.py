@@ -497,3 +497,43 @@ def test_decode_random_launch_shapes(Hq, Hkv, n_seq, L, s):
     want = oracle.attention(oracle.round_bf16(q.astype(np.float64)), gen.to_f64(kc, "bf16"),
                             gen.to_f64(vc, "bf16"), seq, pos)
     assert_parity(to_numpy(ctx), want.reshape(n_seq, Hq * 128), "bf16", "attention ctx", True)
+
+
+# (Hq, Hkv, decode tokens, chunk, max_len): the decode kernel's shares of all
+# position tiles: 127 tokens with whole and split (token, head)s, one tile
+# each (ends moved to whole ones), one key/value head whose sequences are cut
+# into many parts, and few tokens (clusters); the chunk's tokens share a
+# sequence, so some read tiles that others of the call write.
+SHARES = [(16, 8, 100, 27, 700), (8, 4, 60, 3, 120), (6, 1, 100, 20, 3000), (6, 2, 9, 5, 1500)]
+
+
+@pytest.mark.parametrize("Hq,Hkv,n_dec,chunk,L", SHARES, ids=lambda v: str(v))
+def test_decode_shares_of_tiles(Hq, Hkv, n_dec, chunk, L):
+    """Mixed calls of under 128 tokens over caches that hold NaN wherever the
+    call itself writes and past every sequence's end (tiles loaded before the
+    call's rows are written must not reach those), against the oracle."""
+    m = moe()
+    rng = np.random.default_rng(7 * Hq + n_dec)
+    shape = gen.AttnShape(256, Hq, Hkv, 128, 10000.0, "bf16")
+    w_qkv, w_o = gen.host_attn_weights(shape, 61)
+    n_seq = n_dec + 1
+    kc, vc = gen.host_kv_cache(shape, n_seq, L, 61)
+    p0 = int(rng.integers(0, L - chunk))
+    seq = np.concatenate([np.arange(n_dec), np.full(chunk, n_dec)]).astype(np.int32)
+    pos = np.concatenate([rng.integers(0, L, size=n_dec), np.arange(p0, p0 + chunk)]).astype(np.int32)
+    pos[0], pos[1], pos[2] = 0, L - 1, min(L - 1, 128)
+    nan = gen.store(np.full(1, np.nan), "bf16")[0]
+    kc, vc = kc.copy(), vc.copy()
+    for s, p in zip(seq, pos):
+        kc[s, :, p:] = nan
+        vc[s, :, p:] = nan
+    x = rng.normal(size=(seq.size, shape.d_model)).astype(np.float32)
+    want, _, _ = oracle.sa_forward(x.astype(np.float64), w_qkv, w_o, "bf16", Hq, Hkv,
+                                   shape.rope_base, EPS, seq, pos, gen.to_f64(kc, "bf16"),
+                                   gen.to_f64(vc, "bf16"))
+    resid = torch.from_numpy(x).cuda()
+    m.sa_forward(_sa(m, shape), resid, dev(w_qkv, "bf16"), dev(w_o, "bf16"),
+                 torch.from_numpy(seq).cuda(), torch.from_numpy(pos).cuda(), dev(kc, "bf16"),
+                 dev(vc, "bf16"), eps=EPS)
+    assert m.get_last_error() == 0
+    assert_parity(to_numpy(resid) - x, want - x, "bf16", "mixed call below 128 tokens")
