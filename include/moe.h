@@ -380,13 +380,14 @@ moe_status moe_sa_qkv(const moe_sa_dims *dims, int32_t T, const void *x_norm,
 
 /* moe_sa_attend: ctx[t, h dh .. (h+1) dh) = softmax over positions
  * 0..pos[t] of bf16(q[t,h]) . K / sqrt(dh), applied to V (bf16 out): the
- * queries are read rounded to bf16.  As in moe_sa_forward, every 128
- * consecutive tokens that are positions p0..p0+127 of one sequence (a
- * prefill chunk) are attended by the tensor-core flash attention, and the
- * tokens of a call without such a chunk (decode steps) by the tensor-core
- * decode attention; other tokens by the CUDA-core kernel.
- * MOE_ATTN_CUDA_CORES=1 in the environment keeps decode steps on the
- * CUDA-core kernel. */
+ * queries are read rounded to bf16.  As in moe_sa_forward, 16 or more
+ * consecutive tokens that are consecutive positions of one sequence (a
+ * prefill chunk) are attended by the tensor-core flash attention in tiles of
+ * up to 128, all other tokens by the tensor-core decode attention.  (A call
+ * of up to 128 tokens with fewer than 16 more of them than the caches have
+ * sequences is taken as a decode step.)  MOE_ATTN_CUDA_CORES=1 in the
+ * environment keeps the tokens outside tiles, and calls of under 128 tokens,
+ * on the CUDA-core kernel. */
 moe_status moe_sa_attend(const moe_sa_dims *dims, int32_t T, const float *q,
                          const int32_t *seq, const int32_t *pos, int32_t n_seq,
                          int32_t max_len, const void *k_cache, const void *v_cache,

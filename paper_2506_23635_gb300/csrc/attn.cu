@@ -24,10 +24,11 @@
 //                  group's query heads against its positions, online softmax,
 //                  partial (max, sum, weighted values) per split;
 //   k_attn_merge   merges the splits, ctx in bf16 (a single split writes ctx
-//                  itself); in moe_sa_forward, calls of 128 tokens or more
-//                  first run the tensor-core prefill attention (attn_tc.cu)
-//                  on every full 128-token tile of consecutive positions of
-//                  one sequence, and the kernels above only on the rest;
+//                  itself); both run only where the tensor cores do not take
+//                  the tokens: the prefill attention (attn_tc.cu) the tiles
+//                  of consecutive positions that the plan finds (a block of
+//                  k_sa_prenorm), the decode attention (attn_decode_tc.cu)
+//                  every other token;
 //   projection     W_o . ctx (the same two kernels), its partial sums added to
 //                  the residual by k_residual_add.
 #include <math.h>
@@ -91,16 +92,141 @@ constexpr int kNormThreadsWide = 256;
 constexpr int kNormWideMinTokens = 64;
 constexpr int kNormMaxVec = 16;  // float4 per thread: D <= 4 * 16 * 256
 
+// What the attention's plan is made from, and where it goes (plan.head null:
+// the call needs none).
+struct PlanArgs {
+    const int32_t *seq, *pos;
+    int n_seq, L;
+    AttnPlan plan;
+};
+
+// The plan of an attention call, by one block of NT threads.  A run is the
+// longest stretch of tokens that are consecutive positions of one sequence;
+// its tiles are cut from its first token on.  Tiles of at least
+// kAttnTileMinRows tokens are listed by falling length (a counting sort over
+// their key/value tiles; tiles of the same length in any order: no result
+// depends on it), the tokens of the others in ascending order.  Run starts are
+// kept as one bit a token.  It runs beside the pre-norm's other blocks and is
+// done before the projection after them ends.
+constexpr int kPlanBins = 256;
+
+template <int NT>
+__device__ void plan_attention(int T, const PlanArgs &a) {
+    static_assert(NT >= kPlanBins && NT % 32 == 0, "a thread for each bin");
+    __shared__ uint32_t brk[kMaxSaTokens / 32];  // bit t: a run starts at token t
+    __shared__ int last[kMaxSaTokens / 32];      // the last run start ahead of each word
+    __shared__ int bins[kPlanBins];
+    __shared__ int wsum[NT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nw = (T + 31) / 32;
+    for (int t = tid; t < nw * 32; t += NT) {
+        bool b = false;
+        if (t < T) {
+            const int sq = a.seq[t], p = a.pos[t];
+            // (a token outside the cache is a run of its own)
+            b = t == 0 || sq < 0 || sq >= a.n_seq || p <= 0 || p >= a.L || a.seq[t - 1] != sq ||
+                a.pos[t - 1] != p - 1;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, b);
+        if (lane == 0) brk[t >> 5] = m;
+    }
+    if (tid < kPlanBins) bins[tid] = 0;
+    __syncthreads();
+    if (warp == 0) {
+        int run = 0;
+        for (int w0 = 0; w0 < nw; w0 += 32) {
+            const int w = w0 + lane;
+            int v = w < nw && brk[w] ? w * 32 + 31 - __clz(brk[w]) : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v = max(v, u);
+            }
+            v = max(v, run);
+            const int ahead = __shfl_up_sync(0xffffffffu, v, 1);
+            if (w < nw) last[w] = lane == 0 ? run : ahead;
+            run = __shfl_sync(0xffffffffu, v, 31);
+        }
+    }
+    __syncthreads();
+    // the tile of token t: its first token, and its tokens
+    auto tile_of = [&](int t, int &ts, int &rows) {
+        const uint32_t m = brk[t >> 5] & (0xffffffffu >> (31 - (t & 31)));
+        const int rs = m ? (t & ~31) + 31 - __clz(m) : last[t >> 5];
+        ts = rs + ((t - rs) & ~(kAttnTile - 1));
+        int end = min(ts + kAttnTile, T);
+        int w = (ts + 1) >> 5;
+        uint32_t n = w < nw ? brk[w] & (0xffffffffu << ((ts + 1) & 31)) : 0u;
+        while (n == 0 && (w + 1) * 32 < end) n = brk[++w];
+        if (n) end = min(end, w * 32 + __ffs(n) - 1);
+        rows = end - ts;
+    };
+    auto bin_of = [&](int ts, int rows) {  // falling length
+        return kPlanBins - 1 - min(kPlanBins - 1, (a.pos[ts] + rows - 1) / kAttnTile);
+    };
+    int n_left = 0;
+    for (int t0 = 0; t0 < T; t0 += NT) {
+        const int t = t0 + tid;
+        bool left = false;
+        if (t < T) {
+            int ts, rows;
+            tile_of(t, ts, rows);
+            left = rows < kAttnTileMinRows;
+            if (!left && t == ts) atomicAdd(&bins[bin_of(ts, rows)], 1);
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, left);
+        if (lane == 0) wsum[warp] = __popc(m);
+        __syncthreads();
+        int at = n_left + __popc(m & ((1u << lane) - 1u));
+        for (int w = 0; w < NT / 32; ++w) {
+            at += w < warp ? wsum[w] : 0;
+            n_left += wsum[w];
+        }
+        if (left) a.plan.left[at] = t;
+        __syncthreads();
+    }
+    if (warp == 0) {  // bins -> first place of each
+        int run = 0;
+        for (int b0 = 0; b0 < kPlanBins; b0 += 32) {
+            const int c = bins[b0 + lane];
+            int v = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            bins[b0 + lane] = run + v - c;
+            run += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) *a.plan.head = AttnPlanHead{run, n_left, 0, 0};
+    }
+    __syncthreads();
+    for (int t = tid; t < T; t += NT) {
+        int ts, rows;
+        tile_of(t, ts, rows);
+        if (t == ts && rows >= kAttnTileMinRows)
+            a.plan.tiles[atomicAdd(&bins[bin_of(ts, rows)], 1)] =
+                make_int4(ts, rows, a.pos[ts], a.seq[ts]);
+    }
+}
+
 template <int NT, int VEC>
 __global__ void __launch_bounds__(NT)
 k_sa_prenorm(int T, int D, const float *__restrict__ resid, bf16 *__restrict__ xn, float eps,
-             int32_t *offsets) {
+             int32_t *offsets, const PlanArgs pa) {
     // the projection after this kernel may start now: its weight loads do
     // not depend on anything here
     ptx::launch_dependents();
     ptx::grid_dependency_wait();
     __shared__ float red[NT / 32];
-    const int t = blockIdx.x;
+    int t = blockIdx.x;
+    if (pa.plan.head) {  // block 0 makes the attention's plan
+        if (t == 0) {
+            plan_attention<NT>(T, pa);
+            return;
+        }
+        --t;
+    }
     if (t == 0) write_trivial_dispatch(T, offsets);
     const float4 *r = reinterpret_cast<const float4 *>(resid + (size_t)t * D);
     const int nv = D >> 2;
@@ -166,10 +292,9 @@ k_rope_cache(int T, int Hq, int Hkv, int n_seq, int L, RopeRates rates,
              const float *__restrict__ qkv, int n_part, long long part_stride,
              float *__restrict__ q, bf16 *__restrict__ q16, bf16 *__restrict__ kc,
              bf16 *__restrict__ vc, int *__restrict__ dec_count, unsigned *err) {
-    // a decode-type call (no 128-token prefill tile): the tensor-core decode
-    // attention, one CTA per SM on the SMs this small grid leaves free, may
-    // launch now and set itself up while this kernel runs
-    if (T < kAttnTcTile) ptx::launch_dependents();
+    // the tensor-core attention, one CTA per SM on the SMs that this grid
+    // leaves free, may launch now and set itself up while this kernel runs
+    ptx::launch_dependents();
     ptx::grid_dependency_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0) zero_dec_count(dec_count);
     constexpr int H2 = kHeadDim / 2;
@@ -286,26 +411,19 @@ k_attn_partial(int Hq, int Hkv, int n_seq, int L, int n_split, int n_tg,
                const float *__restrict__ q, const bf16 *__restrict__ kc,
                const bf16 *__restrict__ vc, float *__restrict__ part_ml,
                float *__restrict__ part_acc, bf16 *__restrict__ ctx,
-               const int *__restrict__ tile_ok) {
+               const AttnPlan plan) {
     ptx::grid_dependency_wait();
     __shared__ __align__(16) float qs[G][kHeadDim];
     __shared__ float sm_m[kAttnWarps][G], sm_l[kAttnWarps][G];
     __shared__ float sm_acc[kAttnWarps][G][kHeadDim];
     __shared__ __align__(16) bf16 vtile[kAttnWarps][32][kHeadDim];  // each warp's value tile
-    __shared__ unsigned char s_ok[kMaxSaTokens / kAttnTcTile];
     const int s = blockIdx.x;
-    // (token, key/value head) items blockIdx.y, + gridDim.y, ...: a call
-    // whose prefill tiles went to the tensor cores launches a bounded grid
-    // that skips them (their flags read once into shared memory), instead
-    // of a block per item
-    if (tile_ok) {
-        const int n_tiles = (n_tg / Hkv + kAttnTcTile - 1) / kAttnTcTile;
-        for (int i = threadIdx.x; i < n_tiles; i += blockDim.x) s_ok[i] = tile_ok[i] ? 1 : 0;
-        __syncthreads();
-    }
+    // (token, key/value head) items blockIdx.y, + gridDim.y, ...: with a plan
+    // only those of the tokens that no tensor-core tile holds
+    if (plan.head) n_tg = plan.head->n_left * Hkv;
     for (int tg = blockIdx.y; tg < n_tg; tg += gridDim.y) {
-        const int t = tg / Hkv, g = tg - t * Hkv;
-        if (tile_ok && s_ok[t / kAttnTcTile]) continue;  // the tensor-core kernel has it
+        const int i0 = tg / Hkv, g = tg - i0 * Hkv;
+        const int t = plan.head ? plan.left[i0] : i0;
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         const int sq = seq[t], p = pos[t];
         const bool ok = sq >= 0 && sq < n_seq && p >= 0 && p < L;
@@ -495,10 +613,11 @@ k_attn_merge(int n_split, const float *__restrict__ part_ml, const float *__rest
 // brings its own queries (moe_sa_attend); in the whole block the rotary
 // kernel writes it.  n4 groups of four elements.
 __global__ void __launch_bounds__(256)
-k_q_bf16(long long n4, const float *__restrict__ q, bf16 *__restrict__ q16,
-         int *__restrict__ dec_count) {
+k_q_bf16(int T, long long n4, const float *__restrict__ q, bf16 *__restrict__ q16,
+         int *__restrict__ dec_count, const PlanArgs pa) {
     ptx::grid_dependency_wait();
     if (blockIdx.x == 0) zero_dec_count(dec_count);
+    if (blockIdx.x == 0 && pa.plan.head) plan_attention<256>(T, pa);
     const float4 *a = reinterpret_cast<const float4 *>(q);
     __nv_bfloat162 *o = reinterpret_cast<__nv_bfloat162 *>(q16);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
@@ -600,7 +719,7 @@ k_residual_prenorm(int T, int D, int n_part, float *__restrict__ resid, const fl
 // ---- host ------------------------------------------------------------------------
 
 struct SaWs {
-    size_t offsets, xn, qkv, q, q16, tile_ok, part_ml, part_acc, dec_count, dec_part, ctx, total;
+    size_t offsets, xn, qkv, q, q16, plan_head, plan_tiles, plan_left, part_ml, part_acc, dec_count, dec_part, ctx, total;
 };
 
 SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
@@ -618,11 +737,13 @@ SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
     L.qkv = o; o += up(parts * T * std::max(nr, (size_t)d.d_model) * 4);
     L.q = o; o += up((size_t)T * nq * 4);
     L.q16 = o; o += up((size_t)T * nq * 2);
-    L.tile_ok = o; o += up((size_t)(T + kAttnTcTile - 1) / kAttnTcTile * 4);
+    L.plan_head = o; o += up(sizeof(AttnPlanHead));
+    L.plan_tiles = o; o += up((size_t)(T / kAttnTileMinRows) * sizeof(int4));
+    L.plan_left = o; o += up((size_t)T * 4);
     L.part_ml = o; o += up(splits * 2 * 4);
     L.part_acc = o; o += up(splits * kHeadDim * 4);
     L.dec_count = o; o += up(kAttnDecodeMaxCtas * 4);
-    L.dec_part = o; o += up(T <= kAttnDecodeMaxTokens ? kAttnDecodePartFloats * 4 : 0);
+    L.dec_part = o; o += up(kAttnDecodePartFloats * 4);
     L.ctx = o; o += up((size_t)T * nq * 2);
     L.total = o;
     return L;
@@ -682,10 +803,6 @@ struct SaCall {
 };
 
 // W_qkv . xn -> qkv (fp32), then the rotary embedding and the cache writes.
-// Whether the call's attention takes the tensor-core prefill kernel for its
-// full 128-token tiles (the CUDA-core kernel keeps the others).
-bool tc_attention(int T) { return T >= kAttnTcTile && attn_prefill_tc_ok(); }
-
 cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const int32_t *seq,
                      const int32_t *pos, int n_seq, int L, float *q, void *kc, void *vc,
                      bf16 *q16 = nullptr) {
@@ -721,8 +838,8 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
                       dim3(kRopeRows * kHeadDim / 2), 0, c.st, args);
 }
 
-// Whether decode-type calls (no full prefill tile) attend on the tensor
-// cores; MOE_ATTN_CUDA_CORES=1 keeps them on the CUDA-core kernel.
+// Whether tokens that no prefill tile holds attend on the tensor cores;
+// MOE_ATTN_CUDA_CORES=1 keeps them on the CUDA-core kernel.
 bool decode_tc() {
     static const bool off = [] {
         const char *v = getenv("MOE_ATTN_CUDA_CORES");
@@ -731,33 +848,57 @@ bool decode_tc() {
     return !off && attn_decode_tc_ok();
 }
 
-// Whether a call of T tokens wants the bf16 copy of its queries (one of the
-// tensor-core attention kernels reads it).
-bool wants_q16(int T) { return tc_attention(T) || decode_tc(); }
+// Whether a call's tokens are sorted into prefill tiles and the rest.  A call
+// with hardly more tokens than the caches have sequences is a decode step:
+// every token goes to the decode kernel, which takes any.  (The attention block
+// of DBRX: 127 tokens from position 512 on 107 us one by one, each streaming
+// its keys and values for itself, 76 us as a tile; 40 tokens at 300 about 70
+// us either way; 16 tokens at 0, where a tile's launch is all there is, 48.6
+// against 50.6 us.  A prompt of 1000 tokens whose last 104 had gone to the
+// CUDA cores: 376 -> 231 us; 24 decode tokens and chunks of 300 and 205, with
+// 273 tokens on the CUDA cores: 487 -> 197 us.)
+bool planned(int T, int n_seq) {
+    if (!attn_prefill_tc_ok()) return false;
+    return decode_tc() ? T > kAttnDecodeMaxTokens || T - n_seq >= kAttnTileMinRows
+                       : T >= kAttnTile;
+}
 
-// Attention over the caches.  A call with 128 or more tokens: full prefill
-// tiles on the tensor cores, the rest on the CUDA-core kernel (one split);
-// a smaller call: the decode kernel on the tensor cores.  Per-split
-// partials, when there are several splits, are merged last.
+AttnPlan plan_at(const SaCall &c) {
+    return AttnPlan{at<AttnPlanHead>(c.ws, c.L.plan_head), at<int4>(c.ws, c.L.plan_tiles),
+                    at<int>(c.ws, c.L.plan_left)};
+}
+
+PlanArgs plan_args(const SaCall &c, const int32_t *seq, const int32_t *pos, int n_seq, int L) {
+    return PlanArgs{seq, pos, n_seq, L, planned(c.T, n_seq) ? plan_at(c) : AttnPlan{}};
+}
+
+// Whether a call wants the bf16 copy of its queries (one of the tensor-core
+// attention kernels reads it).
+bool wants_q16(int T, int n_seq) { return decode_tc() || planned(T, n_seq); }
+
+// Attention over the caches.  A planned call: its tiles on the tensor cores,
+// then its other tokens; any other call: every token by the decode kernel.
+// The CUDA-core kernel's per-split partials, when there are several splits,
+// are merged last.
 cudaError_t attend(const SaCall &c, const float *q, const int32_t *seq, const int32_t *pos,
                    int n_seq, int L, const void *kc, const void *vc, void *ctx,
                    const bf16 *q16 = nullptr) {
     const int Hq = c.d.n_heads, Hkv = c.d.n_kv_heads, G = Hq / Hkv;
     int ns = n_split_for(c.T, Hkv, L);
-    int *tile_ok = nullptr;
+    AttnPlan plan{};
     float *ml = at<float>(c.ws, c.L.part_ml), *acc = at<float>(c.ws, c.L.part_acc);
     bf16 *cp = static_cast<bf16 *>(ctx);
-    if (q16 && tc_attention(c.T)) {  // full prefill tiles on the tensor cores, the rest below
-        tile_ok = at<int>(c.ws, c.L.tile_ok);
-        cudaError_t e = launch_attn_prefill_tc(c.T, Hq, Hkv, n_seq, L, seq, pos, q16, kc, vc, ctx,
-                                               tile_ok, c.st);
+    if (q16 && planned(c.T, n_seq)) {
+        plan = plan_at(c);
+        cudaError_t e =
+            launch_attn_prefill_tc(c.T, Hq, Hkv, n_seq, L, plan, q16, kc, vc, ctx, c.st);
         if (e != cudaSuccess) return e;
         ns = 1;
-    } else if (q16 && decode_tc()) {
+    }
+    if (q16 && decode_tc())
         return launch_attn_decode_tc(c.T, Hq, Hkv, n_seq, L, seq, pos, q16, kc, vc, ctx,
                                      at<float>(c.ws, c.L.dec_part), at<int>(c.ws, c.L.dec_count),
-                                     c.st);
-    }
+                                     c.st, plan.head ? &plan : nullptr);
     const void *kern = nullptr;
     switch (G) {
         case 1: kern = (const void *)k_attn_partial<1>; break;
@@ -772,14 +913,13 @@ cudaError_t attend(const SaCall &c, const float *q, const int32_t *seq, const in
     int Hqv = Hq, Hkvv = Hkv, nsq = n_seq, Lv = L;
     const bf16 *kcp = static_cast<const bf16 *>(kc), *vcp = static_cast<const bf16 *>(vc);
     {
-        const int *tok = tile_ok;
         int n_tg = c.T * Hkv;
-        // (a prefill call usually leaves no token: one wave of CTAs that
-        // read the tile flags and find nothing to do; otherwise a block per
-        // item up to the grid's y limit, the kernel looping past it)
-        const int gy = std::min(n_tg, tile_ok ? 2 * device_info().sm_count : 65535);
+        // (a planned call usually leaves few tokens: one wave of CTAs;
+        // otherwise a block per item up to the grid's y limit, the kernel
+        // looping past it)
+        const int gy = std::min(n_tg, plan.head ? 2 * device_info().sm_count : 65535);
         void *args[] = {&Hqv, &Hkvv, &nsq, &Lv, &ns, &n_tg, &seq, &pos, &q, &kcp, &vcp, &ml,
-                        &acc, &cp, &tok};
+                        &acc, &cp, &plan};
         LaunchScope ls("attention", c.st);
         cudaError_t e = launch_pdl(kern, dim3(ns, gy), dim3(kAttnThreads), 0, c.st, args);
         if (e != cudaSuccess || ns == 1) return e;
@@ -872,17 +1012,19 @@ moe_status sa_forward_impl(const moe_sa_dims *dims, int32_t T, const int32_t *se
         int Tv = T, D = dims->d_model;
         const float *rc = resid;
         int32_t *off = at<int32_t>(ws, c.L.offsets);
-        void *args[] = {&Tv, &D, &rc, &xn, &eps, &off};
+        PlanArgs pa = plan_args(c, seq, pos, n_seq, max_len);
+        void *args[] = {&Tv, &D, &rc, &xn, &eps, &off, &pa};
+        const dim3 grid(T + (pa.plan.head ? 1 : 0));
         LaunchScope ls("sa_prenorm", c.st);
         const cudaError_t e =
             T >= kNormWideMinTokens
-                ? launch_pdl((const void *)k_sa_prenorm<kNormThreadsWide, kNormMaxVec>, dim3(T),
+                ? launch_pdl((const void *)k_sa_prenorm<kNormThreadsWide, kNormMaxVec>, grid,
                              dim3(kNormThreadsWide), 0, c.st, args)
-                : launch_pdl((const void *)k_sa_prenorm<kNormThreads, 4>, dim3(T),
+                : launch_pdl((const void *)k_sa_prenorm<kNormThreads, 4>, grid,
                              dim3(kNormThreads), 0, c.st, args);
         if (e != cudaSuccess) return MOE_ERR_CUDA;
     }
-    bf16 *q16 = wants_q16(T) ? at<bf16>(ws, c.L.q16) : nullptr;
+    bf16 *q16 = wants_q16(T, n_seq) ? at<bf16>(ws, c.L.q16) : nullptr;
     cudaError_t e = qkv_rope(c, xn, w_qkv, seq, pos, n_seq, max_len, q, k_cache, v_cache, q16);
     if (e == cudaSuccess) e = attend(c, q, seq, pos, n_seq, max_len, k_cache, v_cache, ctx, q16);
     if (e == cudaSuccess) e = out_proj(c, ctx, w_o, resid, xn_next, eps);
@@ -933,12 +1075,14 @@ moe_status moe_sa_attend(const moe_sa_dims *dims, int32_t T, const float *q, con
     // the same kernels as the whole block: the tensor-core attention
     // kernels, from a bf16 copy of the queries
     bf16 *q16 = nullptr;
-    if (wants_q16(T)) {
+    if (wants_q16(T, n_seq)) {
         q16 = at<bf16>(ws, c.L.q16);
+        int Tv = T;
+        PlanArgs pa = plan_args(c, seq, pos, n_seq, max_len);
         long long n4 = (long long)T * dims->n_heads * dims->head_dim / 4;
         const float *qc = q;
         int *dec_count = at<int>(ws, c.L.dec_count);
-        void *args[] = {&n4, &qc, &q16, &dec_count};
+        void *args[] = {&Tv, &n4, &qc, &q16, &dec_count, &pa};
         const int blocks = (int)std::min<long long>((n4 + 255) / 256, 4LL * device_info().sm_count);
         LaunchScope ls("q_bf16", c.st);
         cudaError_t e = launch_pdl((const void *)k_q_bf16, dim3(std::max(blocks, 1)), dim3(256), 0,

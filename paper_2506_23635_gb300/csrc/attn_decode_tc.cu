@@ -12,7 +12,7 @@
 //                       MN-major A operand), P_j K-major in shared memory
 //
 // with S^T and O^T in tensor memory (lane = position, resp. dim; column =
-// head).  Two schedules (template parameter SPLIT):
+// head).  Schedules (template parameter MODE):
 //
 //   shares   the position tiles (128 positions each) of every (token,
 //            key/value head), token by token, are one list; CTA b of G (one
@@ -29,6 +29,15 @@
 //            n_split first, then one at a time from a counter in the cluster's
 //            CTA 0, so a split whose share of the memory bandwidth runs ahead
 //            takes more.
+//   listed   shares of the tiles of the tokens that a plan lists (the tokens
+//            of a call that no prefill tile holds), 128 tokens after the
+//            other; with more than 128 a share's end moves to the nearest end
+//            of a (token, head), so that none is in two shares (there are 6 or
+//            more of them to a CTA then).  The CTAs start as the prefill
+//            attention ahead leaves them SMs: that kernel started after the
+//            queries and cache rows were complete, and its own results are not
+//            read here, so they wait for it only at their end (for the kernels
+//            that follow).
 //
 //   warp 0      TMA: a piece's bf16 query rows into one of four buffers, key
 //               and value tiles into three-stage rings (each 32 KB: two boxes
@@ -179,6 +188,8 @@ struct DecHeader {
     // position tiles of the tokens before it (entry T: of all of them)
     int seq[kDecMaxTokens], n[kDecMaxTokens];
     int before[kDecMaxTokens + 1];
+    int tok[kDecMaxTokens];  // listed: the token
+    int gave_up;             // listed: a wait ran out
 };
 static_assert(sizeof(DecHeader) <= kDecHdrBytes, "decode attention header");
 
@@ -413,18 +424,21 @@ __device__ __forceinline__ int dec_token(const int *before, int T, int Hkv, long
     return t;
 }
 
-// SPLIT: the n_split >= 2 CTAs of a cluster share one (token, key/value head);
-// otherwise n_split is 1 and every CTA has a share of all tiles.  (One kernel
-// that held both forms took 11.5-12.3 us where the cluster form alone takes
-// 10.6-12.0, one sequence of 300-2048 positions.)
-template <int G, bool SPLIT>
+// kDecSplits: the n_split >= 2 CTAs of a cluster share one (token, key/value
+// head); otherwise n_split is 1 and every CTA has a share of all tiles.  (One
+// kernel that held both forms took 11.5-12.3 us where the cluster form alone
+// takes 10.6-12.0, one sequence of 300-2048 positions.)
+enum : int { kDecShares = 0, kDecSplits = 1, kDecListed = 2 };
+
+template <int G, int MODE>
 __global__ void __launch_bounds__(kDecThreads, 1)
 k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, int T, int Hq, int Hkv, int n_seq, int L,
                  const int32_t *__restrict__ seq, const int32_t *__restrict__ pos,
                  bf16 *__restrict__ ctx, float *__restrict__ part, int *__restrict__ count,
-                 int n_split, unsigned *err) {
+                 int n_split, const AttnPlan plan, unsigned *err) {
     static_assert(G >= 1 && G <= kDecMaxG, "query heads per key/value head");
+    constexpr bool SPLIT = MODE == kDecSplits, LISTED = MODE == kDecListed;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -436,6 +450,14 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     // SMs this grid leaves free while the attention runs
     ptx::launch_dependents();
 
+    const int n_listed = LISTED ? __ldcg(&plan.head->n_left) : 0;
+    if (LISTED && n_listed == 0) {
+        ptx::grid_dependency_wait();
+        return;
+    }
+#pragma unroll 1
+    for (int t_base = 0; !LISTED || t_base < n_listed; t_base += kDecMaxTokens) {
+    if (LISTED) T = min(kDecMaxTokens, n_listed - t_base);
     // The producer warp sets up the barriers, finds the CTA's share and sends
     // its first tiles before the block-wide barrier.
     // the next tile to send: token, head, tile of its sequence, and the
@@ -465,6 +487,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         }
         return true;
     };
+    auto token = [&](int t) { return LISTED ? hd->tok[t] : t; };
     if (warp == 0) {
         // the tokens' sequences and positions are inputs of the call, complete
         // before it in stream order (no kernel of the library writes them):
@@ -475,10 +498,17 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = 4 * lane + i;
-            tok_seq[i] = t < T ? seq[t] : -1;
-            tok_n[i] = t < T ? pos[t] : -1;
+            int tok = t;
+            if (LISTED && t < T) hd->tok[t] = tok = __ldcg(plan.left + t_base + t);
+            tok_seq[i] = t < T ? seq[tok] : -1;
+            tok_n[i] = t < T ? pos[tok] : -1;
         }
         if (lane == 0) {
+            if (LISTED) {
+                hd->gave_up = 0;
+                if (t_base > 0)
+                    for (uint64_t *b = hd->k_full; b <= &hd->merge_full; ++b) ptx::mbar_inval(b);
+            }
             for (int b = 0; b < kDecStages; ++b) {
                 ptx::mbar_init(&hd->k_full[b], 1);
                 ptx::mbar_init(&hd->k_empty[b], 1);
@@ -556,7 +586,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 x = dec_start(W, cta + (lane & 1), n_cta);
                 const int t = dec_token(hd->before, T, Hkv, x);
                 const int ntx = hd->before[t + 1] - hd->before[t];
-                if (ntx <= kDecMaxWhole) {
+                if (ntx <= kDecMaxWhole || (LISTED && n_listed > kDecMaxTokens)) {
                     const int o =
                         (int)((unsigned)(x - (long long)hd->before[t] * Hkv) % (unsigned)ntx);
                     x += 2 * o < ntx ? -o : ntx - o;
@@ -577,7 +607,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // this one began: the first stages of them are loaded before the wait
         // for that kernel
         At a = at;
-        bool have = total > 0;
+        bool have = !LISTED && total > 0;
 #pragma unroll 1
         for (int j = 0; j < kDecStages && have; ++j) {
             const int sq = hd->seq[a.t];
@@ -604,7 +634,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             have = j + 1 < kDecStages && advance(a, j + 1, 0);
         }
     }
-    if (warp == 1) tmem_alloc(&hd->tmem_base, kDecTmemCols);
+    if (warp == 1 && (!LISTED || t_base == 0)) tmem_alloc(&hd->tmem_base, kDecTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -615,7 +645,8 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const uint32_t tmem = hd->tmem_base;
     const uint32_t sbase = ptx::smem_u32(smem);
     const bool any = hd->any != 0;  // the share has tiles
-    ptx::grid_dependency_wait();    // queries and new cache rows come from the previous kernel
+    // queries and new cache rows come from the previous kernel
+    if (!LISTED) ptx::grid_dependency_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -624,7 +655,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             if (!(early & 1)) ptx::mbar_arrive_expect_tx(&hd->k_full[0], kDecTile + kDecQ);
             for (int half = 0; half < 2; ++half)
                 ptx::tma_load_2d(smem + kDecOffQ + half * kDecNHalf, &tmQ, half * 64,
-                                 at.t * Hq + at.g * G, &hd->k_full[0], pol_q);
+                                 token(at.t) * Hq + at.g * G, &hd->k_full[0], pol_q);
         }
         if constexpr (SPLIT) cluster_wait();  // CTA 0's counter is initialised before the first take
         if (lane == 0) {
@@ -633,7 +664,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             DecDesc d;
             At nxt = at;
             bool have = total > 0;
-            bool more = have && advance(nxt, 1, 0);
+            bool more = have && advance(nxt, 1, 0), good = true;
             for (int j = 0;; ++j) {
                 const int b = j % kDecStages;
                 const uint32_t ph = ((j / kDecStages) & 1) ^ 1;
@@ -650,7 +681,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 const bool last = !more || (!SPLIT && at.tile == at.nt - 1);
                 if (first) {
                     ++piece;
-                    d.tg = at.t * Hkv + at.g;
+                    d.tg = token(at.t) * Hkv + at.g;
                     d.n = hd->n[at.t];
                     const bool whole = !SPLIT && at.tile == 0 && at.nt <= total - j;
                     d.b0 = d.parts = d.start = d.pad = 0;
@@ -667,14 +698,14 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                           (last ? kDecLast : 0);
                 const int row = (hd->seq[at.t] * Hkv + at.g) * L + at.tile * kDecPos;
                 const bool sent = j < kDecStages && ((early >> j) & 1);  // before the wait above
-                if (!dec_wait(&hd->k_empty[b], ph, err)) break;
+                if (!(good = dec_wait(&hd->k_empty[b], ph, err))) break;
                 if (!sent && j > 0)
                     ptx::mbar_arrive_expect_tx(&hd->k_full[b], kDecTile + (first ? kDecQ : 0u));
                 if (first && j > 0)
                     for (int half = 0; half < 2; ++half)
                         ptx::tma_load_2d(smem + kDecOffQ + (piece % kDecQBufs) * kDecQ +
                                              half * kDecNHalf,
-                                         &tmQ, half * 64, at.t * Hq + at.g * G, &hd->k_full[b],
+                                         &tmQ, half * 64, token(at.t) * Hq + at.g * G, &hd->k_full[b],
                                          pol_q);
                 if (!sent)
                     for (int half = 0; half < 2; ++half)
@@ -683,7 +714,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 k_issued = j + 1;
                 hd->desc[j % kDecRing] = d;
                 ptx::mbar_arrive(&hd->t_full[j % kDecRing]);
-                if (!dec_wait(&hd->v_empty[b], ph, err)) break;
+                if (!(good = dec_wait(&hd->v_empty[b], ph, err))) break;
                 if (!sent) {
                     ptx::mbar_arrive_expect_tx(&hd->v_full[b], kDecTile);
                     for (int half = 0; half < 2; ++half)
@@ -700,6 +731,13 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 dec_wait(&hd->k_full[j % kDecStages], (j / kDecStages) & 1, err);
             for (int j = std::max(0, v_issued - kDecStages); j < v_issued; ++j)
                 dec_wait(&hd->v_full[j % kDecStages], (j / kDecStages) & 1, err);
+            if (LISTED) {  // and the MMAs' last arrivals, before the barriers start anew
+                for (int j = std::max(0, k_issued - kDecStages); good && j < k_issued; ++j)
+                    good = dec_wait(&hd->k_empty[j % kDecStages], (j / kDecStages) & 1, err);
+                for (int j = std::max(0, v_issued - kDecStages); good && j < v_issued; ++j)
+                    good = dec_wait(&hd->v_empty[j % kDecStages], (j / kDecStages) & 1, err);
+                if (!good) hd->gave_up = 1;
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -746,7 +784,8 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 first = (fl1 & kDecFirst) != 0;
             }
             mma_commit(&hd->done);
-            dec_wait(&hd->done, 0, err);
+            good &= dec_wait(&hd->done, 0, err);
+            if (LISTED && !good) hd->gave_up = 1;
         }
         __syncwarp();
     } else {
@@ -910,6 +949,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             for (int h = 0; h < G; ++h)
                 Ls[h] = fin ? (hd->lsum[0][h] + hd->lsum[1][h]) + (hd->lsum[2][h] + hd->lsum[3][h])
                             : 0.f;
+            if (LISTED && !fin) hd->gave_up = 1;
             if constexpr (SPLIT) continue;  // (the share's only piece)
             if (flags & kDecWhole) {
                 bf16 *dst = dec_ctx<G>(ctx, tg, Hq, Hkv) + r;
@@ -1004,20 +1044,24 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem, kDecTmemCols);
+    if (!LISTED || hd->gave_up) break;
+    __syncthreads();  // (read by all before the next tokens' set-up)
+    }
+    if (warp == 1) tmem_dealloc(hd->tmem_base, kDecTmemCols);
+    if (LISTED) ptx::grid_dependency_wait();
 }
 
-template <bool SPLIT>
+template <int MODE>
 const void *dec_kernel(int G) {
     switch (G) {
-        case 1: return (const void *)k_attn_decode_tc<1, SPLIT>;
-        case 2: return (const void *)k_attn_decode_tc<2, SPLIT>;
-        case 3: return (const void *)k_attn_decode_tc<3, SPLIT>;
-        case 4: return (const void *)k_attn_decode_tc<4, SPLIT>;
-        case 5: return (const void *)k_attn_decode_tc<5, SPLIT>;
-        case 6: return (const void *)k_attn_decode_tc<6, SPLIT>;
-        case 7: return (const void *)k_attn_decode_tc<7, SPLIT>;
-        default: return (const void *)k_attn_decode_tc<8, SPLIT>;
+        case 1: return (const void *)k_attn_decode_tc<1, MODE>;
+        case 2: return (const void *)k_attn_decode_tc<2, MODE>;
+        case 3: return (const void *)k_attn_decode_tc<3, MODE>;
+        case 4: return (const void *)k_attn_decode_tc<4, MODE>;
+        case 5: return (const void *)k_attn_decode_tc<5, MODE>;
+        case 6: return (const void *)k_attn_decode_tc<6, MODE>;
+        case 7: return (const void *)k_attn_decode_tc<7, MODE>;
+        default: return (const void *)k_attn_decode_tc<8, MODE>;
     }
 }
 
@@ -1035,7 +1079,7 @@ const DecClusters &dec_clusters() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
     std::call_once(once[dev], [dev] {
-        const void *kern = (const void *)k_attn_decode_tc<1, true>;
+        const void *kern = (const void *)k_attn_decode_tc<1, kDecSplits>;
         const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kDecSmem) == cudaSuccess;
         for (int c = 2; c <= kDecMaxSplit; ++c) {
@@ -1084,9 +1128,9 @@ bool attn_decode_tc_ok() { return encode_fn() != nullptr; }
 cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
                                   const int32_t *pos, const void *q16, const void *k_cache,
                                   const void *v_cache, void *ctx, float *part, int *count,
-                                  cudaStream_t st) {
+                                  cudaStream_t st, const AttnPlan *plan) {
     const int G = Hq / Hkv;
-    if (G < 1 || G > kDecMaxG || G * Hkv != Hq || T < 1 || T > kDecMaxTokens)
+    if (G < 1 || G > kDecMaxG || G * Hkv != Hq || T < 1 || (!plan && T > kDecMaxTokens))
         return cudaErrorInvalidValue;
     CUtensorMap mq, mk, mv;
     const uint64_t rows = (uint64_t)n_seq * Hkv * L;
@@ -1098,15 +1142,19 @@ cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, cons
     int Tv = T, Hqv = Hq, Hkvv = Hkv, ns = n_seq, Lv = L;
     // few (token, key/value head)s: a cluster of CTAs for each; otherwise one
     // share of all tiles per SM
+    // (listed tokens are counted on the device: one CTA per SM)
     const int pairs = T * Hkv, sms = std::min(device_info().sm_count, kAttnDecodeMaxCtas);
     const int max_tiles = (L + kDecPos - 1) / kDecPos;
-    int n_split = dec_splits(pairs, max_tiles, sms);
-    const void *kern = n_split > 1 ? dec_kernel<true>(G) : dec_kernel<false>(G);
+    int n_split = plan ? 1 : dec_splits(pairs, max_tiles, sms);
+    AttnPlan pl = plan ? *plan : AttnPlan{};
+    const void *kern = plan          ? dec_kernel<kDecListed>(G)
+                       : n_split > 1 ? dec_kernel<kDecSplits>(G)
+                                     : dec_kernel<kDecShares>(G);
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
     if (e != cudaSuccess) return e;
     void *args[] = {&mq,  &mk,  &mv, &Tv,   &Hqv,   &Hkvv,    &ns, &Lv,
-                    &seq, &pos, &cp, &part, &count, &n_split, &err};
+                    &seq, &pos, &cp, &part, &count, &n_split, &pl, &err};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_split > 1 ? (unsigned)(n_split * pairs)
                                    : (unsigned)std::min<long long>((long long)pairs * max_tiles, sms));

@@ -1,14 +1,18 @@
 // Causal attention of prefill tiles on the tcgen05 tensor cores.
 //
-// A tile is 128 consecutive tokens of one call that are consecutive positions
-// p0 .. p0+127 of one sequence (a prefill chunk).  One CTA per (tile, pair of
-// query heads hA, hB = hA + 1 of one key/value head g), over cache positions
-// 0 .. p0+127 in key/value tiles of 128 positions; the two heads share every
-// key and value tile and every causal mask, so one copy stream feeds two
-// independent softmax chains that take turns on the tensor cores (a group
-// with an odd number of query heads leaves its last head alone in a CTA).
-// The grid runs every head pair of the last (longest) tile first, so the
-// short tiles fill the end of the launch.
+// A tile is up to 128 consecutive tokens of one call that are consecutive
+// positions p0 .. p0 + rows - 1 of one sequence (a prefill chunk, cut from its
+// first token on).  The tiles are found on the device (plan_attention, run by
+// a block of a kernel ahead) and listed by falling length.  A unit is a (tile,
+// pair of query heads hA, hB = hA + 1 of one key/value head g), over cache
+// positions 0 .. p0 + rows - 1 in key/value tiles of 128 positions; the two
+// heads share every key and value tile and every causal mask, so one copy
+// stream feeds two independent softmax chains that take turns on the tensor
+// cores (a group with an odd number of query heads leaves its last head alone
+// in a unit).  One CTA per SM takes units from a counter, the longest first.
+// A tile's missing rows cost what full ones cost: their queries are whatever
+// follows in memory, each row of the tensor core's output depends on its own
+// query only, and nothing of them is stored.
 //
 //   warp 0      TMA: both heads' bf16 query tiles once, then the key and
 //               the value tiles of positions [128j, 128j+128) into
@@ -46,9 +50,11 @@
 // MMAs): 108-110 us.
 //
 // Every wait is bounded (ptx.cuh) and sleeps on its barrier (suspend-time
-// hint) instead of spinning.  Tiles that do not satisfy the layout condition
-// record tile_ok = 0 and are left to the CUDA-core kernel.
+// hint) instead of spinning; a CTA one of whose waits gave up ends.
 #include <math.h>
+#include <stddef.h>
+
+#include <algorithm>
 
 #include "tc.cuh"
 
@@ -96,8 +102,11 @@ struct FaHeader {
     uint64_t o_full[kFaHeads];   // P_j V_j finished
     uint64_t done;
     uint32_t tmem_base;
-    int ok;
+    int next;    // the CTA's next unit
+    int gave_up; // a wait ran out
 };
+constexpr int kFaBars = (int)((offsetof(FaHeader, done) - offsetof(FaHeader, q_full)) / 8) + 1;
+constexpr int kFaBarP = (int)((offsetof(FaHeader, p_ready) - offsetof(FaHeader, q_full)) / 8);
 static_assert(sizeof(FaHeader) <= 256, "flash-attention header");
 
 // Wait for a barrier phase: a non-blocking test, then the bounded wait that
@@ -183,67 +192,59 @@ __device__ __forceinline__ void tmem_st_wait() {
 // files, so at most 168 registers a thread
 __global__ void __launch_bounds__(kFaThreads, 1)
 k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                  const __grid_constant__ CUtensorMap tmV, int T, int Hq, int Hkv, int n_seq, int L,
-                  const int32_t *__restrict__ seq, const int32_t *__restrict__ pos,
-                  bf16 *__restrict__ ctx, int *__restrict__ tile_ok, unsigned *err) {
+                  const __grid_constant__ CUtensorMap tmV, int Hq, int Hkv, int L,
+                  const AttnPlan plan, bf16 *__restrict__ ctx, unsigned *err) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     FaHeader *hd = reinterpret_cast<FaHeader *>(smem + kOffHdr);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = (T + kFa - 1) / kFa;
-    const int tile = n_tiles - 1 - (int)blockIdx.y;  // the longest tiles first
     const int G = Hq / Hkv, pairs = (G + 1) / 2;
-    const int g = (int)blockIdx.x / pairs, hp = (int)blockIdx.x - g * pairs;
-    const int h0 = g * G + 2 * hp;                // this CTA's first query head
-    const int nh = 2 * hp + 1 < G ? 2 : 1;        // and how many it holds
-    const int t0 = tile * kFa;
+    const uint32_t sbase = ptx::smem_u32(smem);
 
+    ptx::grid_dependency_wait();  // the plan, queries and caches come from earlier kernels
+    // the kernel for the tokens that no tile holds may take the SMs that this
+    // one leaves free
+    ptx::launch_dependents();
+    const int n_units = __ldcg(&plan.head->n_tiles) * Hkv * pairs;
+    int unit = (int)blockIdx.x;
+    if (unit >= n_units) return;
     if (threadIdx.x == 0) {
-        ptx::mbar_init(&hd->q_full, 1);
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(&hd->kv_full[b], 1);
-            ptx::mbar_init(&hd->kv_empty[b], 1);
-            ptx::mbar_init(&hd->v_full[b], 1);
-            ptx::mbar_init(&hd->v_empty[b], 1);
-        }
-        for (int x = 0; x < kFaHeads; ++x) {
-            ptx::mbar_init(&hd->s_full[x], 1);
-            ptx::mbar_init(&hd->p_ready[x], kFaWarpsPerHead);
-            ptx::mbar_init(&hd->o_full[x], 1);
-        }
-        ptx::mbar_init(&hd->done, 1);
-        ptx::fence_barrier_init();
+        hd->gave_up = 0;
         ptx::prefetch_tmap(&tmQ);
         ptx::prefetch_tmap(&tmK);
         ptx::prefetch_tmap(&tmV);
-        hd->ok = 1;
     }
     if (warp == 1) tmem_alloc(&hd->tmem_base, kFaTmemCols);
-    ptx::grid_dependency_wait();  // queries and caches come from the previous kernel
-    __syncthreads();
-    // the tile qualifies if its 128 tokens exist and are positions p0..p0+127
-    // of one sequence inside the cache
-    const int sq = seq[min(t0, T - 1)], p0 = pos[min(t0, T - 1)];
-    if (threadIdx.x < kFa) {
-        const int t = t0 + threadIdx.x;
-        const bool good = t < T && seq[t] == sq && pos[t] == p0 + (int)threadIdx.x && sq >= 0 &&
-                          sq < n_seq && p0 >= 0 && p0 + kFa <= L;
-        if (!good) hd->ok = 0;
+
+#pragma unroll 1
+    for (bool again = false;; again = true) {
+    if (threadIdx.x == 0) {
+        uint64_t *bars = &hd->q_full;  // all of them, one after the other
+        if (again)
+            for (int i = 0; i < kFaBars; ++i) ptx::mbar_inval(bars + i);
+        for (int i = 0; i < kFaBars; ++i)
+            ptx::mbar_init(bars + i, i >= kFaBarP && i < kFaBarP + kFaHeads ? kFaWarpsPerHead : 1);
+        ptx::fence_barrier_init();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = hd->tmem_base;
-    const bool ok = hd->ok != 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) tile_ok[tile] = ok ? 1 : 0;
-    const int n_kv = ok ? (p0 + kFa - 1) / kFa + 1 : 0;  // key/value tiles 0 .. n_kv-1
-    const uint32_t sbase = ptx::smem_u32(smem);
+    const int tile = unit / (Hkv * pairs), gp = unit - tile * Hkv * pairs;
+    const int g = gp / pairs, hp = gp - g * pairs;
+    const int h0 = g * G + 2 * hp;                // the unit's first query head
+    const int nh = 2 * hp + 1 < G ? 2 : 1;        // and how many it holds
+    const int4 td = __ldcg(&plan.tiles[tile]);
+    const int t0 = td.x, rows = td.y, p0 = td.z, sq = td.w;
+    const int n_kv = (p0 + rows - 1) / kFa + 1;   // key/value tiles 0 .. n_kv-1
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        if (lane == 0 && ok) {
+        if (lane == 0) {
+            const int taken = atomicAdd(&plan.head->next, 1);  // (used at the end)
             const uint64_t pol = ptx::policy_evict_last();
+            bool good = true;
             ptx::mbar_arrive_expect_tx(&hd->q_full, (uint32_t)nh * kTileBytes);
             for (int x = 0; x < nh; ++x)
                 for (int half = 0; half < 2; ++half)
@@ -253,13 +254,13 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             int issued = 0, v_issued = 0;
             for (int j = 0; j < n_kv; ++j) {
                 const int b = j & 1;
-                if (!fa_wait(&hd->kv_empty[b], ((j >> 1) & 1) ^ 1, err)) break;
+                if (!(good = fa_wait(&hd->kv_empty[b], ((j >> 1) & 1) ^ 1, err))) break;
                 ptx::mbar_arrive_expect_tx(&hd->kv_full[b], kTileBytes);
                 for (int half = 0; half < 2; ++half)
                     ptx::tma_load_2d(smem + kOffK + b * kTileBytes + half * kHalfBytes, &tmK,
                                      half * 64, row0 + j * kFa, &hd->kv_full[b], pol);
                 issued = j + 1;
-                if (!fa_wait(&hd->v_empty[b], ((j >> 1) & 1) ^ 1, err)) break;
+                if (!(good = fa_wait(&hd->v_empty[b], ((j >> 1) & 1) ^ 1, err))) break;
                 ptx::mbar_arrive_expect_tx(&hd->v_full[b], kTileBytes);
                 for (int half = 0; half < 2; ++half)
                     ptx::tma_load_2d(smem + kOffV + b * kTileBytes + half * kHalfBytes, &tmV,
@@ -267,15 +268,22 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 v_issued = j + 1;
             }
             // let loads still in flight land before the block can exit
-            fa_wait(&hd->q_full, 0, err);
+            good &= fa_wait(&hd->q_full, 0, err);
             for (int j = (issued > 2 ? issued - 2 : 0); j < issued; ++j)
-                fa_wait(&hd->kv_full[j & 1], (j >> 1) & 1, err);
+                good &= fa_wait(&hd->kv_full[j & 1], (j >> 1) & 1, err);
             for (int j = (v_issued > 2 ? v_issued - 2 : 0); j < v_issued; ++j)
-                fa_wait(&hd->v_full[j & 1], (j >> 1) & 1, err);
+                good &= fa_wait(&hd->v_full[j & 1], (j >> 1) & 1, err);
+            // and the MMAs' last arrivals, before the barriers start anew
+            for (int j = (issued > 2 ? issued - 2 : 0); good && j < issued; ++j)
+                good = fa_wait(&hd->kv_empty[j & 1], (j >> 1) & 1, err);
+            for (int j = (v_issued > 2 ? v_issued - 2 : 0); good && j < v_issued; ++j)
+                good = fa_wait(&hd->v_empty[j & 1], (j >> 1) & 1, err);
+            hd->next = (int)gridDim.x + taken;
+            if (!good) hd->gave_up = 1;
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && ok) {
+        if (lane == 0) {
             bool good = fa_wait(&hd->q_full, 0, err) && fa_wait(&hd->kv_full[0], 0, err);
             if (good) {
                 tc_fence_after();
@@ -312,16 +320,17 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
             }
             mma_commit(&hd->done);
-            fa_wait(&hd->done, 0, err);
+            good &= fa_wait(&hd->done, 0, err);
+            if (!good) hd->gave_up = 1;
         }
         __syncwarp();
-    } else if (ok && (warp - 2) / kFaWarpsPerHead < nh) {
+    } else if ((warp - 2) / kFaWarpsPerHead < nh) {
         // ------------------------------------------------------------ softmax
         const int x = (warp - 2) / kFaWarpsPerHead;  // head h0 + x of the CTA
         const int q = warp & 3;                      // tensor-memory lane quarter
         const int r = q * 32 + lane;                 // query row of the tile
         const int qpos = p0 + r;
-        const int last = p0 + kFa - 1;               // the tile's last query position
+        const int last = p0 + rows - 1;              // the tile's last query position
         const float sl2 = 1.4426950408889634f / sqrtf((float)kHeadDimFa);
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const uint32_t s_col = tmem + lane_base + kColS + (uint32_t)x * kFa;
@@ -417,8 +426,8 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (lane == 0) ptx::mbar_arrive(&hd->p_ready[x]);
             l = l * corr + ((sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y));
         }
-        bool fin = good && n_kv > 0;
-        if (fin) fin = fa_wait(&hd->o_full[x], (n_kv - 1) & 1, err);
+        const bool fin = good && fa_wait(&hd->o_full[x], (n_kv - 1) & 1, err);
+        if (!fin) hd->gave_up = 1;
         if (__all_sync(0xffffffffu, fin)) {
             tc_fence_after();
             const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -428,6 +437,7 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 float vv[32];
                 tmem_ld32(o_col + c, vv);
                 tmem_ld_wait();
+                if (r >= rows) continue;
 #pragma unroll
                 for (int i = 0; i < 32; i += 8) {
                     uint32_t w[4];
@@ -445,16 +455,19 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem, kFaTmemCols);
+    unit = hd->next;
+    if (unit >= n_units || hd->gave_up) break;
+    }
+    if (warp == 1) tmem_dealloc(hd->tmem_base, kFaTmemCols);
 }
 
 }  // namespace
 
 bool attn_prefill_tc_ok() { return encode_fn() != nullptr; }
 
-cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
-                                   const int32_t *pos, const void *q16, const void *k_cache,
-                                   const void *v_cache, void *ctx, int *tile_ok, cudaStream_t st) {
+cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, const AttnPlan &plan,
+                                   const void *q16, const void *k_cache, const void *v_cache,
+                                   void *ctx, cudaStream_t st) {
     CUtensorMap mq, mk, mv;
     const uint64_t rows = (uint64_t)n_seq * Hkv * L;
     if (!make_map(&mq, q16, (uint64_t)T, (uint64_t)Hq * 128, kFa) ||
@@ -466,12 +479,15 @@ cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, con
     if (e != cudaSuccess) return e;
     unsigned *err = device_info().err;
     bf16 *cp = static_cast<bf16 *>(ctx);
-    void *args[] = {&mq, &mk, &mv, &T, &Hq, &Hkv, &n_seq, &L, &seq, &pos, &cp, &tile_ok, &err};
-    // a CTA per (pair of query heads of one key/value head, tile)
+    AttnPlan pl = plan;
+    void *args[] = {&mq, &mk, &mv, &Hq, &Hkv, &L, &pl, &cp, &err};
+    // one CTA per SM, or per unit of the most tiles that T tokens can make
     const int pairs = (Hq / Hkv + 1) / 2;
+    const long long most = (long long)Hkv * pairs * (T / kAttnTileMinRows);
     LaunchScope ls("attention_tc", st);
-    return launch_pdl(kern, dim3(Hkv * pairs, (T + kFa - 1) / kFa), dim3(kFaThreads), kFaSmem, st,
-                      args);
+    return launch_pdl(kern,
+                      dim3((unsigned)std::max(1LL, std::min<long long>(most, device_info().sm_count))),
+                      dim3(kFaThreads), kFaSmem, st, args);
 }
 
 }  // namespace moe

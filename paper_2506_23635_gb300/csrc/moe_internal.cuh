@@ -263,22 +263,39 @@ constexpr int kRowsMaxParts = 4;
 int gemm_rows_parts(int Kdim, int Nw);
 cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const void *w, int parts,
                                 float *y, cudaStream_t st, const char *name = nullptr);
-// Causal attention of prefill tiles on the tensor cores (attn_tc.cu): every
-// 128-token tile of the call whose tokens are positions p0..p0+127 of one
-// sequence; tile_ok[i] = 1 for the tiles it handled (the others are left to
-// the CUDA-core kernel).  q16 [T, Hq*128] bf16 queries (rotated, unscaled),
-// caches [n_seq, Hkv, L, 128] bf16, head_dim 128.
-constexpr int kAttnTcTile = 128;
+// How the tokens of an attention call are shared between the kernels, found on
+// the device (plan_attention in attn.cu): the tiles of the tensor-core prefill
+// attention, longest first, and the tokens that none of them holds.
+constexpr int kAttnTile = 128;  // tokens of a tile at most
+// and at least: fewer consecutive tokens are attended one by one (a tile costs
+// its (head pair)s ~2.75 us of an SM for each 128 cache positions whatever its
+// rows, a token its key/value heads ~1 us: DBRX's heads break even at ~8-10)
+constexpr int kAttnTileMinRows = 16;
+struct AttnPlanHead {
+    int n_tiles, n_left;
+    int next;  // units taken from the tiles beyond each CTA's first
+    int pad;
+};
+struct AttnPlan {
+    AttnPlanHead *head;
+    int4 *tiles;  // first token, tokens, position of the first, sequence
+    int *left;    // tokens in ascending order
+};
+// Causal attention of the plan's tiles on the tensor cores (attn_tc.cu).  q16
+// [T, Hq*128] bf16 queries (rotated, unscaled), caches [n_seq, Hkv, L, 128]
+// bf16, head_dim 128.
 bool attn_prefill_tc_ok();
-cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
-                                   const int32_t *pos, const void *q16, const void *k_cache,
-                                   const void *v_cache, void *ctx, int *tile_ok, cudaStream_t st);
+cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, const AttnPlan &plan,
+                                   const void *q16, const void *k_cache, const void *v_cache,
+                                   void *ctx, cudaStream_t st);
 // Decode attention on the tensor cores (attn_decode_tc.cu): every token of a
 // call of up to kAttnDecodeMaxTokens over positions 0..pos[t] of its
 // sequence; ctx written.  Queries as above; query heads per key/value head
 // <= 8.  part: kAttnDecodePartFloats floats for the results of (token,
 // key/value head)s that several CTAs share; count: kAttnDecodeMaxCtas ints,
-// zero at the start (the kernel that writes q16 zeroes them).
+// zero at the start (the kernel that writes q16 zeroes them).  With a plan,
+// only its tokens that no tile holds, any number of them; the launch ahead is
+// then the plan's prefill attention, which this one overlaps.
 constexpr int kAttnDecodeMaxTokens = 128;
 constexpr int kAttnDecodeMaxCtas = 160;
 constexpr size_t kAttnDecodePartFloats = (size_t)2 * kAttnDecodeMaxCtas * 8 * (128 + 2);
@@ -286,7 +303,7 @@ bool attn_decode_tc_ok();
 cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
                                   const int32_t *pos, const void *q16, const void *k_cache,
                                   const void *v_cache, void *ctx, float *part, int *count,
-                                  cudaStream_t st);
+                                  cudaStream_t st, const AttnPlan *plan = nullptr);
 
 // name: the profiling name of the launch (default "gemm_down_tc").  y_tail
 // (optional, [T*K, D]): the stream-K schedule's second output; the result is

@@ -537,3 +537,53 @@ def test_decode_shares_of_tiles(Hq, Hkv, n_dec, chunk, L):
                  dev(vc, "bf16"), eps=EPS)
     assert m.get_last_error() == 0
     assert_parity(to_numpy(resid) - x, want - x, "bf16", "mixed call below 128 tokens")
+
+
+# (Hq, Hkv, max_len, runs): runs of consecutive positions in the order of the
+# call, (sequence, first position, tokens); -1: one token each of that many
+# sequences.  Tiles of 16 tokens and more are cut from a run's first token,
+# shorter ones are listed: runs one short of a tile, a tile, one over and one
+# short of 16 over it; the smallest tile; two runs of one sequence; a call of
+# 40 tokens; 300 listed tokens (three batches of them) around a tile; an odd
+# group of query heads; a sequence past 256 key/value tiles beside short ones.
+RAGGED = [
+    (6, 1, 700, [(0, 37, 127), (-1, 0, 5), (1, 0, 129), (2, 130, 128), (3, 1, 143), (4, 600, 16),
+                 (5, 600, 15), (1, 129, 77)]),
+    (12, 2, 300, [(0, 250, 40)]),
+    (4, 2, 200, [(-1, 0, 170), (0, 20, 33), (-1, 0, 130)]),
+    (3, 1, 400, [(0, 0, 300), (1, 3, 200), (-1, 0, 3)]),
+    (2, 1, 33100, [(0, 33000, 90), (1, 5, 20), (2, 128, 64), (-1, 0, 4)]),
+]
+
+
+@pytest.mark.parametrize("Hq,Hkv,L,runs", RAGGED, ids=lambda v: str(v)[:24])
+def test_ragged_tiles_and_listed_tokens(Hq, Hkv, L, runs):
+    """Calls whose prompts start and end anywhere, decode tokens between them,
+    over caches that hold NaN past each sequence's last position of the call."""
+    m = moe()
+    rng = np.random.default_rng(L + Hq)
+    shape = gen.AttnShape(Hq * 128, Hq, Hkv, 128, 10000.0, "bf16")
+    seq, pos, n_seq = [], [], 1 + max(r[0] for r in runs)
+    for s, p0, n in runs:
+        if s >= 0:
+            seq += [s] * n
+            pos += range(p0, p0 + n)
+        else:
+            seq += range(n_seq, n_seq + n)
+            pos += rng.integers(0, min(L, 400), size=n).tolist()
+            n_seq += n
+    seq, pos = np.array(seq, np.int32), np.array(pos, np.int32)
+    T = seq.size
+    kc, vc = (a.copy() for a in gen.host_kv_cache(shape, n_seq, L, 83))
+    nan = gen.store(np.full(1, np.nan), "bf16")[0]
+    for s in range(n_seq):
+        end = int(pos[seq == s].max(initial=-1)) + 1
+        kc[s, :, end:] = nan
+        vc[s, :, end:] = nan
+    q = rng.normal(size=(T, Hq, 128)).astype(np.float32) * 4
+    ctx = m.sa_attend(_sa(m, shape), torch.from_numpy(q).cuda(), torch.from_numpy(seq).cuda(),
+                      torch.from_numpy(pos).cuda(), dev(kc, "bf16"), dev(vc, "bf16"))
+    assert m.get_last_error() == 0
+    want = oracle.attention(oracle.round_bf16(q.astype(np.float64)), gen.to_f64(kc, "bf16"),
+                            gen.to_f64(vc, "bf16"), seq, pos)
+    assert_parity(to_numpy(ctx), want.reshape(T, Hq * 128), "bf16", "ragged attention ctx", True)
