@@ -50,6 +50,8 @@ constexpr int kSplitPositions = 128;  // cache positions per split (a 32-positio
 constexpr int kMaxSplit = 64;
 constexpr int kMaxSplitCtas = 4096;   // bound on T * Hkv * splits (sizes the workspace)
 constexpr int kMaxSaTokens = 65536;
+static_assert(kMaxSaTokens <= (kAttnDecodeCounts - kAttnDecodeMaxCtas) * kAttnDecodeMaxTokens,
+              "a counter for every 128 tokens");
 
 // Most position splits a call of T tokens may use (the workspace holds this many).
 int split_cap(int T, int Hkv) {
@@ -275,7 +277,7 @@ k_sa_setup(int T, int32_t *offsets) {
 // The decode attention's counters start at zero (threads of one block).
 __device__ __forceinline__ void zero_dec_count(int *count) {
     if (count)
-        for (int i = threadIdx.x; i < kAttnDecodeMaxCtas; i += blockDim.x) count[i] = 0;
+        for (int i = threadIdx.x; i < kAttnDecodeCounts; i += blockDim.x) count[i] = 0;
 }
 
 // qkv [T, (Hq + 2 Hkv) 128] fp32 (the sum of n_part partial projections
@@ -719,7 +721,8 @@ k_residual_prenorm(int T, int D, int n_part, float *__restrict__ resid, const fl
 // ---- host ------------------------------------------------------------------------
 
 struct SaWs {
-    size_t offsets, xn, qkv, q, q16, plan_head, plan_tiles, plan_left, part_ml, part_acc, dec_count, dec_part, ctx, total;
+    size_t offsets, xn, qkv, q, q16, plan_head, plan_tiles, plan_left, part_ml, part_acc,
+        dec_count, dec_part, ctx, total;
 };
 
 SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
@@ -742,7 +745,7 @@ SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
     L.plan_left = o; o += up((size_t)T * 4);
     L.part_ml = o; o += up(splits * 2 * 4);
     L.part_acc = o; o += up(splits * kHeadDim * 4);
-    L.dec_count = o; o += up(kAttnDecodeMaxCtas * 4);
+    L.dec_count = o; o += up(kAttnDecodeCounts * 4);
     L.dec_part = o; o += up(kAttnDecodePartFloats * 4);
     L.ctx = o; o += up((size_t)T * nq * 2);
     L.total = o;
@@ -848,18 +851,22 @@ bool decode_tc() {
     return !off && attn_decode_tc_ok();
 }
 
-// Whether a call's tokens are sorted into prefill tiles and the rest.  A call
-// with hardly more tokens than the caches have sequences is a decode step:
-// every token goes to the decode kernel, which takes any.  (The attention block
-// of DBRX: 127 tokens from position 512 on 107 us one by one, each streaming
-// its keys and values for itself, 76 us as a tile; 40 tokens at 300 about 70
-// us either way; 16 tokens at 0, where a tile's launch is all there is, 48.6
-// against 50.6 us.  A prompt of 1000 tokens whose last 104 had gone to the
+// Whether a call's tokens are sorted into prefill tiles and the rest.  A small
+// call with hardly more tokens than the caches have sequences is a decode
+// step: every token goes to the decode kernel, which takes any, and the launch
+// of the other is saved.  (The attention block of DBRX: 127 tokens from
+// position 512 on 107 us one by one, each streaming its keys and values for
+// itself, 76 us as a tile; 100 tokens at 0 72 and 70 us; 40 tokens at 300, and
+// 30 tokens beside 40 decode tokens, the same either way; 16 tokens at 0 48.6
+// against 50.6 us, four runs of 9 at 600 beside 40 decode tokens 100 against
+// 104 us.  A prompt of 1000 tokens whose last 104 had gone to the
 // CUDA cores: 376 -> 231 us; 24 decode tokens and chunks of 300 and 205, with
 // 273 tokens on the CUDA cores: 487 -> 197 us.)
+constexpr int kPlanMinTokens = 48;  // beyond one for each sequence
+
 bool planned(int T, int n_seq) {
     if (!attn_prefill_tc_ok()) return false;
-    return decode_tc() ? T > kAttnDecodeMaxTokens || T - n_seq >= kAttnTileMinRows
+    return decode_tc() ? T > kAttnDecodeMaxTokens || T - n_seq >= kPlanMinTokens
                        : T >= kAttnTile;
 }
 

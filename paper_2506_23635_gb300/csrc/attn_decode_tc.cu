@@ -20,6 +20,13 @@
 //            W tiles, so every SM streams the same number of bytes whatever
 //            the sequences' lengths.  A share is a run of pieces: the end of
 //            one (token, head)'s tiles, whole ones, the start of another's.
+//            Where there are many (token, head)s to a CTA, it takes them whole,
+//            longest first and one after the other from a counter: parts and
+//            their merges cost more than the uneven ends (attention block at
+//            48 sequences of 512-2048 positions and a chunk of 8: 97 us with
+//            a CTA for each (token, head), 102 in equal shares, 91 so; up to
+//            4096 positions 139 and 125; taking the next one at the start of
+//            its predecessor, in the call's order, 147).
 //            (One CTA per (token, head) before: 88 of 152 SMs with 11
 //            sequences, all waiting for the longest; 1488-4096 positions, 118
 //            MB of keys and values: 42.2 us before, 30.6 us, of which ~8 us are
@@ -29,11 +36,10 @@
 //            n_split first, then one at a time from a counter in the cluster's
 //            CTA 0, so a split whose share of the memory bandwidth runs ahead
 //            takes more.
-//   listed   shares of the tiles of the tokens that a plan lists (the tokens
-//            of a call that no prefill tile holds), 128 tokens after the
-//            other; with more than 128 a share's end moves to the nearest end
-//            of a (token, head), so that none is in two shares (there are 6 or
-//            more of them to a CTA then).  The CTAs start as the prefill
+//   listed   the same for the tokens that a plan lists (the tokens of a call
+//            that no prefill tile holds), 128 tokens after the other (none of
+//            more than 128 is in two shares: there are 6 or more (token,
+//            head)s to a CTA then).  The CTAs start as the prefill
 //            attention ahead leaves them SMs: that kernel started after the
 //            queries and cache rows were complete, and its own results are not
 //            read here, so they wait for it only at their end (for the kernels
@@ -150,21 +156,26 @@ struct DecDesc {
     int tg;       // token * Hkv + key/value head
     int n;        // positions the token attends to (0: outside the cache)
     int flags;    // kDecFirst, kDecLast: of its piece; kDecWhole: the piece is the
-                  // whole (token, head); from bit 4: the query buffer
-    int b0, parts;  // not whole: the first CTA with a piece of it, and how many have one
+                  // whole (token, head), kDecEnd: of its share; from bit 4: the query buffer
+    int b0, parts;  // not whole: the first share with a piece of it, and how many have one
     int start;      // not whole: this piece is its start
-    int pad;
+    int share;
 };
 // a part's slot in the workspace: 8 rows of O^T, 8 pairs (base, sum)
 constexpr int kDecSlot = kDecMaxG * (128 + 2);
-static_assert(2 * kAttnDecodeMaxCtas * kDecSlot <= (int)kAttnDecodePartFloats, "two slots a CTA");
+static_assert(2 * kAttnDecodeMaxCtas * kDecSlot <= (int)kAttnDecodePartFloats,
+              "two slots a share");
 // shares of fewer tiles than this leave SMs out: two tiles' copies are in
 // flight together and cost little more than one's, a part to merge 2-3 us
 constexpr int kDecMinTiles = 2;
 // a share's end inside a (token, head) of at most this many tiles moves to the
 // nearer end of it
 constexpr int kDecMaxWhole = 4;
-enum : int { kDecFirst = 1, kDecLast = 2, kDecWhole = 4, kDecQShift = 4 };
+// from this many (token, head)s for each CTA on they are taken whole (32
+// tokens of DBRX, 1.7, up to 4096 positions: 102 us in equal shares, 112 with
+// a CTA each)
+constexpr int kDecWholeMin = 2;
+enum : int { kDecFirst = 1, kDecLast = 2, kDecWhole = 4, kDecEnd = 8, kDecQShift = 4 };
 
 struct DecHeader {
     uint64_t k_full[kDecStages], k_empty[kDecStages];  // key tile j in stage j % 3
@@ -179,7 +190,6 @@ struct DecHeader {
     uint32_t tmem_base;
     uint32_t next_tile;              // the cluster's tile counter (in CTA 0)
     int last;                        // this CTA counted last on its first (1), last (2) piece
-    int any;                         // the CTA's share has tiles
     alignas(16) DecDesc desc[kDecRing];
     float red[4][kDecMaxG];     // the warps' tile maxima
     float lsum[4][kDecMaxG];    // the warps' row sums at the end
@@ -188,7 +198,8 @@ struct DecHeader {
     // position tiles of the tokens before it (entry T: of all of them)
     int seq[kDecMaxTokens], n[kDecMaxTokens];
     int before[kDecMaxTokens + 1];
-    int tok[kDecMaxTokens];  // listed: the token
+    int tok[kDecMaxTokens];    // listed: the token
+    int order[kDecMaxTokens];  // taken whole: the tokens by falling length
     int gave_up;             // listed: a wait ran out
 };
 static_assert(sizeof(DecHeader) <= kDecHdrBytes, "decode attention header");
@@ -465,10 +476,13 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     struct At {
         int t, g, tile, nt;
     } at = {0, 0, 0, 1};
-    long long W = 0, lo = 0;
-    int total = 0, n_cta = 1, early = 0;
+    long long lo = 0;  // the share's first tile
+    long long W = 0;
+    int n_share = 1;
+    bool whole_only = false;  // the shares are the (token, head)s
+    int cur = cta, total = 0, early = 0;  // the share, its tiles
     const uint64_t pol_kv = ptx::policy_evict_first();  // key and value tiles are read once
-    // the tile after a, this CTA's j-th; false: there is none.  A split's
+    // the tile after a, its share's j-th; false: there is none.  A split's
     // first kDecStages tiles are fixed (c, c + n_split, ...); `taken` is then
     // the next one from the cluster's counter
     auto advance = [&](At &a, int j, int taken) -> bool {
@@ -488,6 +502,40 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         return true;
     };
     auto token = [&](int t) { return LISTED ? hd->tok[t] : t; };
+    // the next (token, head) that no CTA has taken (the first ones are the
+    // CTAs' own, unless the CTAs start at different times)
+    auto take = [&]() {
+        return atomicAdd(&count[kAttnDecodeMaxCtas + t_base / kDecMaxTokens], 1) +
+               (LISTED ? 0 : (int)gridDim.x);
+    };
+    // where share c starts (c - 1 ends): moved to the nearer end of a (token,
+    // head) of few tiles
+    auto share_end = [&](int c) -> long long {
+        if (c >= n_share) return W;
+        const long long x = dec_start(W, c, n_share);
+        const int t = dec_token(hd->before, T, Hkv, x);
+        const int ntx = hd->before[t + 1] - hd->before[t];
+        if (ntx > kDecMaxWhole) return x;
+        const int o = (int)((unsigned)(x - (long long)hd->before[t] * Hkv) % (unsigned)ntx);
+        return x + (2 * o < ntx ? -o : ntx - o);
+    };
+    // (token, head) c of those taken whole, longest first
+    auto find_whole = [&](At &a, int c) {
+        total = 0;
+        if (c >= n_share) return;
+        a.t = hd->order[c / Hkv];
+        a.g = c % Hkv;
+        a.tile = 0;
+        a.nt = total = hd->before[a.t + 1] - hd->before[a.t];
+    };
+    // the share's first tile: lo
+    auto find = [&](At &a) {
+        a.t = dec_token(hd->before, T, Hkv, lo);
+        a.nt = hd->before[a.t + 1] - hd->before[a.t];
+        const long long in_t = lo - (long long)hd->before[a.t] * Hkv;
+        a.g = in_t < (1 << 30) ? (int)((unsigned)in_t / (unsigned)a.nt) : (int)(in_t / a.nt);
+        a.tile = (int)(in_t - (long long)a.g * a.nt);
+    };
     if (warp == 0) {
         // the tokens' sequences and positions are inputs of the call, complete
         // before it in stream order (no kernel of the library writes them):
@@ -578,29 +626,39 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             if (lane == 31) hd->before[kDecMaxTokens] = run;
             __syncwarp();
             W = (long long)hd->before[kDecMaxTokens] * Hkv;
-            n_cta = (int)min((long long)gridDim.x,
-                             max(1LL, W < (1 << 24) ? (unsigned)W / (unsigned)kDecMinTiles
-                                                    : W / kDecMinTiles));
-            long long x = W;  // even lanes: the share's start, odd lanes: its end
-            if (cta + (lane & 1) < n_cta) {
-                x = dec_start(W, cta + (lane & 1), n_cta);
-                const int t = dec_token(hd->before, T, Hkv, x);
-                const int ntx = hd->before[t + 1] - hd->before[t];
-                if (ntx <= kDecMaxWhole || (LISTED && n_listed > kDecMaxTokens)) {
-                    const int o =
-                        (int)((unsigned)(x - (long long)hd->before[t] * Hkv) % (unsigned)ntx);
-                    x += 2 * o < ntx ? -o : ntx - o;
+            whole_only = T * Hkv >= kDecWholeMin * (int)gridDim.x ||
+                         (LISTED && n_listed > kDecMaxTokens);
+            n_share = whole_only ? T * Hkv
+                                 : (int)min((long long)gridDim.x,
+                                            max(1LL, W < (1 << 24)
+                                                         ? (unsigned)W / (unsigned)kDecMinTiles
+                                                         : W / kDecMinTiles));
+            if (whole_only) {
+                // the tokens by falling length, ties in their order: each
+                // lane counts those ahead of its four
+                int rank[4] = {0, 0, 0, 0};
+                int b0 = 0;
+                for (int u = 0; u < T; ++u) {
+                    const int b1 = hd->before[u + 1], nu = b1 - b0;
+                    b0 = b1;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        rank[i] += nu > nt[i] || (nu == nt[i] && u < 4 * lane + i) ? 1 : 0;
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (4 * lane + i < T) hd->order[rank[i]] = 4 * lane + i;
+                __syncwarp();
+                if (LISTED) cur = __shfl_sync(0xffffffffu, lane == 0 ? take() : 0, 0);
+                find_whole(at, cur);
+            } else {
+                // even lanes: the share's start, odd lanes: its end
+                const long long x = share_end(cur + (lane & 1));
+                lo = __shfl_sync(0xffffffffu, x, 0);
+                total = (int)(__shfl_sync(0xffffffffu, x, 1) - lo);
+                find(at);
             }
-            lo = __shfl_sync(0xffffffffu, x, 0);
-            total = (int)(__shfl_sync(0xffffffffu, x, 1) - lo);
-            at.t = dec_token(hd->before, T, Hkv, lo);
-            at.nt = hd->before[at.t + 1] - hd->before[at.t];
-            const long long in_t = lo - (long long)hd->before[at.t] * Hkv;
-            at.g = in_t < (1 << 30) ? (int)((unsigned)in_t / (unsigned)at.nt) : (int)(in_t / at.nt);
-            at.tile = (int)(in_t - (long long)at.g * at.nt);
         }
-        if (lane == 0) hd->any = total > 0 ? 1 : 0;
         // key and value tiles that no token of this call writes into (all of
         // the sequence's positions in them lie before the call's first one)
         // hold what earlier calls left, complete before the kernel ahead of
@@ -644,14 +702,13 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if constexpr (SPLIT) cluster_arrive_release();
     const uint32_t tmem = hd->tmem_base;
     const uint32_t sbase = ptx::smem_u32(smem);
-    const bool any = hd->any != 0;  // the share has tiles
     // queries and new cache rows come from the previous kernel
     if (!LISTED) ptx::grid_dependency_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         const uint64_t pol_q = ptx::policy_evict_normal();
-        if (lane == 0 && any) {  // the first piece's query rows
+        if (!LISTED && lane == 0 && total > 0) {  // the first piece's query rows
             if (!(early & 1)) ptx::mbar_arrive_expect_tx(&hd->k_full[0], kDecTile + kDecQ);
             for (int half = 0; half < 2; ++half)
                 ptx::tma_load_2d(smem + kDecOffQ + half * kDecNHalf, &tmQ, half * 64,
@@ -662,8 +719,36 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             const uint32_t counter = ptx::map_rank(ptx::smem_u32(&hd->next_tile), 0u);
             int piece = -1, k_issued = 0, v_issued = 0, taken = 0;
             DecDesc d;
-            At nxt = at;
+            // (a (token, head)'s successor is taken two tiles before its end:
+            // the counter's answer is there in time, and the CTAs that are
+            // done first take the next ones)
+            int share = n_share;
+            int jj = 0;  // tiles of the share before this one
+            auto next_share = [&]() {
+                cur = share;
+                find_whole(at, cur);
+                jj = 0;
+                return total > 0;
+            };
+            // values of tile v_issued: sent after the keys of the tile that
+            // follows, so that their stage is free again soon after they land
+            // (their P is formed while they are on the way)
+            int v_row = 0;
+            bool v_sent = false;
+            auto send_v = [&]() -> bool {
+                const int b = v_issued % kDecStages;
+                if (!dec_wait(&hd->v_empty[b], ((v_issued / kDecStages) & 1) ^ 1, err)) return false;
+                if (!v_sent) {
+                    ptx::mbar_arrive_expect_tx(&hd->v_full[b], kDecTile);
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffV + b * kDecTile + half * kDecHalf, &tmV,
+                                         half * 64, v_row, &hd->v_full[b], pol_kv);
+                }
+                ++v_issued;
+                return true;
+            };
             bool have = total > 0;
+            At nxt = at;
             bool more = have && advance(nxt, 1, 0), good = true;
             for (int j = 0;; ++j) {
                 const int b = j % kDecStages;
@@ -671,37 +756,40 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 if (!have) {
                     hd->desc[j % kDecRing].tile = -1;
                     ptx::mbar_arrive(&hd->t_full[j % kDecRing]);
+                    if (j > 0) good = send_v();
                     break;
                 }
                 // (taken two tiles ahead: the counter's round trip runs while
                 // a stage frees)
                 if (SPLIT && more && j + 2 >= kDecStages)
                     taken = kDecStages * n_split + (int)dec_take(counter);
-                const bool first = j == 0 || (!SPLIT && at.tile == 0);
+                if (!SPLIT && whole_only && at.tile == std::max(0, at.nt - 3)) share = take();
+                const bool first = jj == 0 || (!SPLIT && at.tile == 0);
                 const bool last = !more || (!SPLIT && at.tile == at.nt - 1);
                 if (first) {
                     ++piece;
                     d.tg = token(at.t) * Hkv + at.g;
                     d.n = hd->n[at.t];
-                    const bool whole = !SPLIT && at.tile == 0 && at.nt <= total - j;
-                    d.b0 = d.parts = d.start = d.pad = 0;
+                    const bool whole = !SPLIT && at.tile == 0 && at.nt <= total - jj;
+                    d.b0 = d.parts = d.start = 0;
+                    d.share = cur;
                     if (!whole && !SPLIT) {
-                        const long long f0 = lo + j - at.tile;  // the (token, head)'s first tile
-                        d.b0 = dec_owner(f0, W, n_cta);
-                        d.parts = dec_owner(f0 + at.nt - 1, W, n_cta) - d.b0 + 1;
+                        const long long f0 = lo + jj - at.tile;  // the (token, head)'s first tile
+                        d.b0 = dec_owner(f0, W, n_share);
+                        d.parts = dec_owner(f0 + at.nt - 1, W, n_share) - d.b0 + 1;
                         d.start = at.tile == 0 ? 1 : 0;
                     }
                     d.flags = (whole ? kDecWhole : 0) | ((piece % kDecQBufs) << kDecQShift);
                 }
                 d.tile = at.tile;
-                d.flags = (d.flags & ~(kDecFirst | kDecLast)) | (first ? kDecFirst : 0) |
-                          (last ? kDecLast : 0);
+                d.flags = (d.flags & ~(kDecFirst | kDecLast | kDecEnd)) | (first ? kDecFirst : 0) |
+                          (last ? kDecLast : 0) | (more ? 0 : kDecEnd);
                 const int row = (hd->seq[at.t] * Hkv + at.g) * L + at.tile * kDecPos;
                 const bool sent = j < kDecStages && ((early >> j) & 1);  // before the wait above
                 if (!(good = dec_wait(&hd->k_empty[b], ph, err))) break;
-                if (!sent && j > 0)
+                if (!sent && (LISTED || j > 0))
                     ptx::mbar_arrive_expect_tx(&hd->k_full[b], kDecTile + (first ? kDecQ : 0u));
-                if (first && j > 0)
+                if (first && (LISTED || j > 0))
                     for (int half = 0; half < 2; ++half)
                         ptx::tma_load_2d(smem + kDecOffQ + (piece % kDecQBufs) * kDecQ +
                                              half * kDecNHalf,
@@ -714,17 +802,17 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 k_issued = j + 1;
                 hd->desc[j % kDecRing] = d;
                 ptx::mbar_arrive(&hd->t_full[j % kDecRing]);
-                if (!(good = dec_wait(&hd->v_empty[b], ph, err))) break;
-                if (!sent) {
-                    ptx::mbar_arrive_expect_tx(&hd->v_full[b], kDecTile);
-                    for (int half = 0; half < 2; ++half)
-                        ptx::tma_load_2d(smem + kDecOffV + b * kDecTile + half * kDecHalf, &tmV,
-                                         half * 64, row, &hd->v_full[b], pol_kv);
-                }
-                v_issued = j + 1;
+                if (j > 0 && !(good = send_v())) break;
+                v_row = row;
+                v_sent = sent;
                 at = nxt;
                 have = more;
-                more = more && advance(nxt, j + 2, taken);
+                ++jj;
+                if (!SPLIT && !have) {
+                    have = whole_only && next_share();
+                    nxt = at;
+                }
+                more = have && advance(nxt, SPLIT ? j + 2 : jj + 1, taken);
             }
             // copies still in flight land before the block can exit
             for (int j = std::max(0, k_issued - kDecStages); j < k_issued; ++j)
@@ -742,16 +830,18 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && any) {
-            bool good = dec_wait(&hd->t_full[0], 0, err) && dec_wait(&hd->k_full[0], 0, err);
-            if (good) {
+        if (lane == 0) {
+            bool good = dec_wait(&hd->t_full[0], 0, err);
+            const bool any = good && hd->desc[0].tile >= 0;
+            good = good && (!any || dec_wait(&hd->k_full[0], 0, err));
+            if (good && any) {
                 tc_fence_after();
                 dec_issue_qk(tmem + kDecColS, sbase + kDecOffK, sbase + kDecOffQ);
                 mma_commit(&hd->s_full[0]);
                 mma_commit(&hd->k_empty[0]);
             }
             bool first = true;  // tile j is its piece's first
-            for (int j = 0; good; ++j) {
+            for (int j = 0; good && any; ++j) {
                 // is there a tile j + 1 (published by the producer)?
                 const int r1 = (j + 1) % kDecRing;
                 if (!(good = dec_wait(&hd->t_full[r1], ((j + 1) / kDecRing) & 1, err))) break;
@@ -820,18 +910,16 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         // head) of which other CTAs hold parts too (parts > 0): which, the
         // first CTA with a part, how many
         int pend_tg[2], pend_b0[2], pend_parts[2] = {0, 0};
-        bool good = any;  // (an empty share has nothing to wait for)
-        for (int j = 0; any; ++j) {
+        bool good = true;
+        for (int j = 0;; ++j) {
             const int b = j & 1;
             good = good && dec_wait(&hd->t_full[j % kDecRing], (j / kDecRing) & 1, err);
             // (lane 0's reading steers the warp: its loop stays converged)
             const DecDesc *dj = &hd->desc[j % kDecRing];
             const int tile = __shfl_sync(0xffffffffu, good ? dj->tile : -1, 0);
             if (tile < 0) break;
-            const int n = __shfl_sync(0xffffffffu, dj->n, 0);
-            const int flags = __shfl_sync(0xffffffffu, dj->flags, 0);
-            const int tg = __shfl_sync(0xffffffffu, dj->tg, 0);
-            const int b0 = dj->b0, parts = dj->parts, start = dj->start;
+            const int n = dj->n, flags = dj->flags, tg = dj->tg;  // (one value for the warp)
+            const int b0 = dj->b0, parts = dj->parts, start = dj->start, share = dj->share;
             if (flags & kDecFirst) {
 #pragma unroll
                 for (int h = 0; h < G; ++h) {
@@ -955,20 +1043,42 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 bf16 *dst = dec_ctx<G>(ctx, tg, Hq, Hkv) + r;
 #pragma unroll
                 for (int h = 0; h < G; ++h) dst[h * 128] = dec_mean(o[h], Ls[h]);
-                continue;
-            }
-            // a part: its slot holds G rows of O^T, then G pairs (base, sum)
-            float *mine = part + (size_t)(2 * cta + start) * kDecSlot;
+            } else {
+                // a part: its slot holds G rows of O^T, then G pairs (base, sum)
+                float *mine = part + (size_t)(2 * share + start) * kDecSlot;
 #pragma unroll
-            for (int h = 0; h < G; ++h) {
-                mine[h * 128 + r] = o[h];
-                if (r == 0)
-                    *reinterpret_cast<float2 *>(mine + kDecMaxG * 128 + 2 * h) =
-                        make_float2(fin ? base[h] : -INFINITY, Ls[h]);
+                for (int h = 0; h < G; ++h) {
+                    mine[h * 128 + r] = o[h];
+                    if (r == 0)
+                        *reinterpret_cast<float2 *>(mine + kDecMaxG * 128 + 2 * h) =
+                            make_float2(fin ? base[h] : -INFINITY, Ls[h]);
+                }
+                // (start 0: the share begins inside the (token, head))
+                if (start) pend_tg[1] = tg, pend_b0[1] = b0, pend_parts[1] = parts;
+                else pend_tg[0] = tg, pend_b0[0] = b0, pend_parts[0] = parts;
             }
-            // (start 0: the share begins inside the (token, head))
-            if (start) pend_tg[1] = tg, pend_b0[1] = b0, pend_parts[1] = parts;
-            else pend_tg[0] = tg, pend_b0[0] = b0, pend_parts[0] = parts;
+            if (!(flags & kDecEnd) || (pend_parts[0] == 0 && pend_parts[1] == 0)) continue;
+            // the share is done: its parts are counted, and the CTA that
+            // counts last on a (token, head) finds every part of it stored
+            ptx::named_bar_sync(1, 128);
+            if (r == 0) {
+                __threadfence();  // the warps' stores (ordered by the barrier) before the counts
+                int last = 0;
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (pend_parts[i] > 0 &&
+                        atomicAdd(&count[pend_b0[i]], 1) == pend_parts[i] - 1)
+                        last |= 1 << i;
+                hd->last = last;
+                __threadfence();  // the counts before the loads of the other parts
+            }
+            ptx::named_bar_sync(1, 128);
+#pragma unroll 1
+            for (int i = 0; i < 2; ++i)
+                if ((hd->last >> i) & 1)
+                    dec_merge<G>(part, pend_b0[i], pend_parts[i], r,
+                                 dec_ctx<G>(ctx, pend_tg[i], Hq, Hkv) + r);
+            pend_parts[0] = pend_parts[1] = 0;
         }
         if constexpr (SPLIT) {
             // every split sends its part of head h to the CTA that owns it,
@@ -1016,27 +1126,6 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 }
                 dst[h * 128] = dec_mean(A, S);
             }
-        } else if (pend_parts[0] > 0 || pend_parts[1] > 0) {
-            // count this share's parts; the CTA that counts last on a (token,
-            // head) finds every part of it stored
-            ptx::named_bar_sync(1, 128);
-            if (r == 0) {
-                __threadfence();  // the warps' stores (ordered by the barrier) before the counts
-                int last = 0;
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    if (pend_parts[i] > 0 &&
-                        atomicAdd(&count[pend_b0[i]], 1) == pend_parts[i] - 1)
-                        last |= 1 << i;
-                hd->last = last;
-                __threadfence();  // the counts before the loads of the other parts
-            }
-            ptx::named_bar_sync(1, 128);
-#pragma unroll 1
-            for (int i = 0; i < 2; ++i)
-                if ((hd->last >> i) & 1)
-                    dec_merge<G>(part, pend_b0[i], pend_parts[i], r,
-                                 dec_ctx<G>(ctx, pend_tg[i], Hq, Hkv) + r);
         }
     }
     // (the aligned wait of every thread: the others waited at their start)

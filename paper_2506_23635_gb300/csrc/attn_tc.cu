@@ -242,7 +242,6 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            const int taken = atomicAdd(&plan.head->next, 1);  // (used at the end)
             const uint64_t pol = ptx::policy_evict_last();
             bool good = true;
             ptx::mbar_arrive_expect_tx(&hd->q_full, (uint32_t)nh * kTileBytes);
@@ -267,6 +266,11 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                                      half * 64, row0 + j * kFa, &hd->v_full[b], pol);
                 v_issued = j + 1;
             }
+            // the next unit: taken near this one's end, the counter's answer
+            // due once the last MMAs have finished (taken at the unit's start,
+            // the CTAs with the longest first units drew second ones as early
+            // as the others: 1536 tokens at 512, 82 us instead of 70)
+            const int taken = atomicAdd(&plan.head->next, 1);
             // let loads still in flight land before the block can exit
             good &= fa_wait(&hd->q_full, 0, err);
             for (int j = (issued > 2 ? issued - 2 : 0); j < issued; ++j)

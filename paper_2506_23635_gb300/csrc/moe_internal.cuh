@@ -292,12 +292,15 @@ cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, con
 // call of up to kAttnDecodeMaxTokens over positions 0..pos[t] of its
 // sequence; ctx written.  Queries as above; query heads per key/value head
 // <= 8.  part: kAttnDecodePartFloats floats for the results of (token,
-// key/value head)s that several CTAs share; count: kAttnDecodeMaxCtas ints,
+// key/value head)s that several CTAs share; count: kAttnDecodeCounts ints,
 // zero at the start (the kernel that writes q16 zeroes them).  With a plan,
 // only its tokens that no tile holds, any number of them; the launch ahead is
 // then the plan's prefill attention, which this one overlaps.
 constexpr int kAttnDecodeMaxTokens = 128;
 constexpr int kAttnDecodeMaxCtas = 160;
+// a counter of finished parts for each CTA, one of (token, head)s taken for
+// every 128 listed tokens of the largest call
+constexpr int kAttnDecodeCounts = kAttnDecodeMaxCtas + 65536 / kAttnDecodeMaxTokens;
 constexpr size_t kAttnDecodePartFloats = (size_t)2 * kAttnDecodeMaxCtas * 8 * (128 + 2);
 bool attn_decode_tc_ok();
 cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, const int32_t *seq,
