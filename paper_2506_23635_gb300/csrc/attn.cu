@@ -15,7 +15,7 @@
 //                  it lets the projection launch at once (the projection's
 //                  weight loads do not depend on it);
 //   projection     W_qkv . x: the tcgen05 kernel with the weights as the M
-//                  operand (split reduction) for up to 64 tokens, the grouped
+//                  operand (split reduction) for up to 768 tokens, the grouped
 //                  tcgen05 GEMM with E = 1 beyond (fp32 out);
 //   k_rope_cache   rotary embedding of q and k (angles formed and reduced in
 //                  fp64, evaluated in fp32), k and v written to the cache in
@@ -281,7 +281,8 @@ __device__ __forceinline__ void zero_dec_count(int *count) {
 }
 
 // qkv [T, (Hq + 2 Hkv) 128] fp32 (the sum of n_part partial projections
-// part_stride floats apart) -> q [T, Hq, 128] fp32 (rotated); rotated keys
+// part_stride floats apart) -> q [T, Hq, 128] rotated, in fp32 and in bf16
+// (either may be left out); rotated keys
 // and the values to the caches [n_seq, Hkv, L, 128] in bf16.  A block holds
 // kRopeRows head rows of one token, 64 threads each: thread i turns the pair
 // (i, i + 64) of a query or key head, or copies two value elements.
@@ -359,9 +360,11 @@ k_rope_cache(int T, int Hq, int Hkv, int n_seq, int L, RopeRates rates,
         const float cs = cs_s[u][i], sn = sn_s[u][i];
         const float x0 = a * cs - b * sn, x1 = b * cs + a * sn;
         if (hr < Hq) {
-            float *qo = q + (size_t)t * nq + (size_t)hr * kHeadDim;
-            qo[i] = x0;
-            qo[i + H2] = x1;
+            if (q) {
+                float *qo = q + (size_t)t * nq + (size_t)hr * kHeadDim;
+                qo[i] = x0;
+                qo[i + H2] = x1;
+            }
             if (q16) {  // the tensor-core attention's copy
                 bf16 *qh = q16 + (size_t)t * nq + (size_t)hr * kHeadDim;
                 qh[i] = __float2bfloat16_rn(x0);
@@ -736,8 +739,10 @@ SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
     L.xn = o; o += up((size_t)T * d.d_model * 2);
     // projection outputs (partial sums of a split reduction for up to
     // kRowsMaxTokens tokens): qkv first, later the output projection's rows
-    const size_t parts = T <= kRowsMaxTokens ? kRowsMaxParts : 1;
-    L.qkv = o; o += up(parts * T * std::max(nr, (size_t)d.d_model) * 4);
+    // (as many rows as any smaller call needs, too)
+    const size_t part_rows =
+        std::max<size_t>(T, (size_t)kRowsMaxParts * std::min<int64_t>(T, kRowsMaxTokens));
+    L.qkv = o; o += up(part_rows * std::max(nr, (size_t)d.d_model) * 4);
     L.q = o; o += up((size_t)T * nq * 4);
     L.q16 = o; o += up((size_t)T * nq * 2);
     L.plan_head = o; o += up(sizeof(AttnPlanHead));
@@ -815,7 +820,7 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
     cudaError_t e;
     int n_part = 1;
     if (c.T <= kRowsMaxTokens) {
-        n_part = gemm_rows_parts(c.d.d_model, c.nr());
+        n_part = gemm_rows_parts(c.T, c.d.d_model, c.nr());
         e = launch_gemm_rows_tc(c.T, c.d.d_model, c.nr(), xn, w_qkv, n_part, qkv, c.st,
                                 "qkv_rows_tc");
     } else {
@@ -949,7 +954,7 @@ cudaError_t out_proj(const SaCall &c, const void *ctx, const void *w_o, float *r
     int n_part = 1;
     cudaError_t e;
     if (c.T <= kRowsMaxTokens) {
-        n_part = gemm_rows_parts(c.nq(), c.d.d_model);
+        n_part = gemm_rows_parts(c.T, c.nq(), c.d.d_model);
         e = launch_gemm_rows_tc(c.T, c.nq(), c.d.d_model, ctx, w_o, n_part, y, c.st, "o_rows_tc");
     } else {
         e = launch_gemm_down_tc(pd, c.T, ctx, offsets, w_o, y, c.st, "o_gemm_tc");
@@ -1032,7 +1037,9 @@ moe_status sa_forward_impl(const moe_sa_dims *dims, int32_t T, const int32_t *se
         if (e != cudaSuccess) return MOE_ERR_CUDA;
     }
     bf16 *q16 = wants_q16(T, n_seq) ? at<bf16>(ws, c.L.q16) : nullptr;
-    cudaError_t e = qkv_rope(c, xn, w_qkv, seq, pos, n_seq, max_len, q, k_cache, v_cache, q16);
+    // (only the CUDA-core attention reads the fp32 queries)
+    cudaError_t e = qkv_rope(c, xn, w_qkv, seq, pos, n_seq, max_len, decode_tc() ? nullptr : q,
+                             k_cache, v_cache, q16);
     if (e == cudaSuccess) e = attend(c, q, seq, pos, n_seq, max_len, k_cache, v_cache, ctx, q16);
     if (e == cudaSuccess) e = out_proj(c, ctx, w_o, resid, xn_next, eps);
     return cuda_status(e);

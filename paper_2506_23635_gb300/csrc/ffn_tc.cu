@@ -368,12 +368,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 
 // ---- one weight matrix against a few token rows (weights as the M operand) -------
 //
-// y[j, n] = x[j, :] . W[n, :] for j < T <= 128 tokens and the Nw rows of one
-// matrix W [Nw, Kdim].  A decode batch fills few of the 128 slot rows of the
+// y[j, n] = x[j, :] . W[n, :] for j < T <= 768 tokens, in near-equal runs of at
+// most 256 (gridDim.z), and the Nw rows of one matrix W [Nw, Kdim].  A decode
+// batch fills few of the 128 slot rows of the
 // MMA above, and a single matrix has few 256-row tiles; here the weights are
 // the A operand instead (128 rows per tile) and the tokens the B operand
-// (NTOK = 16, 32, 64 or 128 columns), so every stage is 16 KB of weights
-// plus NTOK x 128 B of tokens and 6-12 stages stay in flight.
+// (NTOK = 16, 32, 64, 128, 160, 192, 224 or 256 columns), so every stage is 16 KB of
+// weights plus NTOK x 128 B of tokens and 4-12 stages stay in flight.
 // Loaded HBM latency is ~3.5 us, so streaming at the HBM rate needs ~25 MB in
 // flight: the reduction is split over gridDim.y CTAs per tile (split z writes
 // its partial sums to y_out + z*T*Nw; the caller adds the parts in order).
@@ -389,11 +390,11 @@ struct SwapCfg {
             ? (int)((227 * 1024 - 1024 - kTcHeaderBytes) / kStageBytes)
             : 12;
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kTcHeaderBytes;
-    static constexpr uint32_t kTmemCols = NTOK < 32 ? 32 : NTOK;
+    static constexpr uint32_t kTmemCols = NTOK < 32 ? 32 : NTOK > 128 ? 256 : NTOK;
     // kind::f16: bf16 A and B, fp32 D, both K-major, N = NTOK, M = 128
     static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
                                        ((uint32_t)(NTOK >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-    static_assert(NTOK % 16 == 0 && NTOK >= 16 && NTOK <= 128, "token columns");
+    static_assert(NTOK % 16 == 0 && NTOK >= 16 && NTOK <= 256, "token columns");
     static_assert(kStageBytes % 1024 == 0, "stages stay 1024-byte aligned");
     static_assert(kStages >= 4 && kStages <= kMaxSwapStages, "stages");
     static_assert((kTmemCols & (kTmemCols - 1)) == 0, "tensor memory is allocated in powers of two");
@@ -423,7 +424,11 @@ k_gemm_swap(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     const int kb0 = (int)((long long)nk_all * blockIdx.y / gridDim.y);
     const int nk = (int)((long long)nk_all * (blockIdx.y + 1) / gridDim.y) - kb0;
     const int n0 = blockIdx.x * BM;  // first weight row of this CTA's tile
-    y_out += (size_t)blockIdx.y * T * Nw;
+    // the run of tokens of this CTA: T / gridDim.z of them
+    const int t0 = (int)((long long)T * blockIdx.z / gridDim.z);
+    const int t1 = (int)((long long)T * (blockIdx.z + 1) / gridDim.z);
+    y_out += (size_t)blockIdx.y * T * Nw + (size_t)t0 * Nw;
+    T = t1 - t0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -455,7 +460,7 @@ k_gemm_swap(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
             }
             ptx::grid_dependency_wait();  // the token rows come from the previous kernel
             for (int kb = 0; kb < early; ++kb)
-                ptx::tma_load_2d(smem + kb * C::kStageBytes + C::kStageW, &tmX, (kb0 + kb) * BK, 0,
+                ptx::tma_load_2d(smem + kb * C::kStageBytes + C::kStageW, &tmX, (kb0 + kb) * BK, t0,
                                  &hd->full[kb], pol_x);
             int issued = early;
             for (int kb = early; kb < nk; ++kb) {
@@ -464,7 +469,7 @@ k_gemm_swap(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
                 unsigned char *st = smem + s * C::kStageBytes;
                 ptx::mbar_arrive_expect_tx(&hd->full[s], C::kStageBytes);
                 ptx::tma_load_2d(st, &tmW, (kb0 + kb) * BK, n0, &hd->full[s], pol_w);
-                ptx::tma_load_2d(st + C::kStageW, &tmX, (kb0 + kb) * BK, 0, &hd->full[s], pol_x);
+                ptx::tma_load_2d(st + C::kStageW, &tmX, (kb0 + kb) * BK, t0, &hd->full[s], pol_x);
                 issued = kb + 1;
             }
             // let loads still in flight land before the block can exit
@@ -617,7 +622,7 @@ cudaError_t launch_swap(const CUtensorMap &w, const CUtensorMap &x, int T, int K
     CUtensorMap mw = w, mx = x;
     void *args[] = {&mw, &mx, &T, &Kdim, &Nw, &y, &err};
     LaunchScope ls(name ? name : "gemm_rows_tc", st);
-    return launch_pdl(kern, dim3((Nw + BM - 1) / BM, parts), dim3(kThreadsTc), C::kSmem, st,
+    return launch_pdl(kern, dim3((Nw + BM - 1) / BM, parts, (T + 255) / 256), dim3(kThreadsTc), C::kSmem, st,
                       args);
 }
 
@@ -675,8 +680,8 @@ cudaError_t launch_gemm_down_tc(const moe_dims &d, int T, const void *h, const i
                                         y_sorted, st, name, y_tail);
 }
 
-int gemm_rows_parts(int Kdim, int Nw) {
-    const int tiles = (Nw + BM - 1) / BM, nk = (Kdim + BK - 1) / BK;
+int gemm_rows_parts(int T, int Kdim, int Nw) {
+    const int tiles = (Nw + BM - 1) / BM * ((T + 255) / 256), nk = (Kdim + BK - 1) / BK;
     const int by_sms = std::max(1, device_info().sm_count / std::max(1, tiles));
     return std::max(1, std::min({kRowsMaxParts, by_sms, nk}));
 }
@@ -685,8 +690,16 @@ cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const vo
                                 float *y, cudaStream_t st, const char *name) {
     if (T < 1 || T > kRowsMaxTokens || parts < 1 || parts > kRowsMaxParts)
         return cudaErrorInvalidValue;
-    const int ntok = (T + 15) / 16 * 16;
-    const uint32_t xrows = ntok <= 16 ? 16 : ntok <= 32 ? 32 : ntok <= 64 ? 64 : 128;
+    const int runs = (T + 255) / 256;  // of at most 256 tokens, near-equal
+    const int ntok = ((T + runs - 1) / runs + 15) / 16 * 16;
+    const uint32_t xrows = ntok <= 16    ? 16
+                           : ntok <= 32  ? 32
+                           : ntok <= 64  ? 64
+                           : ntok <= 128 ? 128
+                           : ntok <= 160 ? 160
+                           : ntok <= 192 ? 192
+                           : ntok <= 224 ? 224
+                                         : 256;
     CUtensorMap mw, mx;
     if (!make_map(&mw, w, (uint64_t)Nw, (uint64_t)Kdim, BM) ||
         !make_map(&mx, x, (uint64_t)T, (uint64_t)Kdim, xrows))
@@ -694,7 +707,11 @@ cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const vo
     if (xrows == 16) return launch_swap<16>(mw, mx, T, Kdim, Nw, parts, y, st, name);
     if (xrows == 32) return launch_swap<32>(mw, mx, T, Kdim, Nw, parts, y, st, name);
     if (xrows == 64) return launch_swap<64>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    return launch_swap<128>(mw, mx, T, Kdim, Nw, parts, y, st, name);
+    if (xrows == 128) return launch_swap<128>(mw, mx, T, Kdim, Nw, parts, y, st, name);
+    if (xrows == 160) return launch_swap<160>(mw, mx, T, Kdim, Nw, parts, y, st, name);
+    if (xrows == 192) return launch_swap<192>(mw, mx, T, Kdim, Nw, parts, y, st, name);
+    if (xrows == 224) return launch_swap<224>(mw, mx, T, Kdim, Nw, parts, y, st, name);
+    return launch_swap<256>(mw, mx, T, Kdim, Nw, parts, y, st, name);
 }
 
 }  // namespace moe

@@ -258,9 +258,13 @@ cudaError_t launch_gemm_up_tc(const moe_dims &d, int T, const void *x_sorted,
 // reduction split into `parts` (<= kRowsMaxParts) shares whose partial sums
 // land in y + p*T*Nw for p < parts (the caller adds them in order).
 // gemm_rows_parts: the split that keeps the SMs streaming for this shape.
-constexpr int kRowsMaxTokens = 128;
+// (the last size that the CTA-pair GEMM does not beat: attention block of DBRX,
+// two projections, on this kernel and on that: 130 tokens 70 and 99 us, 256: 82
+// and 109, 400: 107 and 129, 512: 126 and 142, 600: 149 and 162, 768: 176 and
+// 177, 1000: 230 and 219, 1200: 282 and 260)
+constexpr int kRowsMaxTokens = 768;
 constexpr int kRowsMaxParts = 4;
-int gemm_rows_parts(int Kdim, int Nw);
+int gemm_rows_parts(int T, int Kdim, int Nw);
 cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const void *w, int parts,
                                 float *y, cudaStream_t st, const char *name = nullptr);
 // How the tokens of an attention call are shared between the kernels, found on

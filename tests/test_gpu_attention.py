@@ -587,3 +587,38 @@ def test_ragged_tiles_and_listed_tokens(Hq, Hkv, L, runs):
     want = oracle.attention(oracle.round_bf16(q.astype(np.float64)), gen.to_f64(kc, "bf16"),
                             gen.to_f64(vc, "bf16"), seq, pos)
     assert_parity(to_numpy(ctx), want.reshape(T, Hq * 128), "bf16", "ragged attention ctx", True)
+
+
+# (D, Hq, Hkv, tokens): the projections of calls above 128 tokens: one token
+# more, each width of a token run (160, 192, 224 and 256), one token over a run
+# of 256 and over two, the last size of this kernel and the first of the pair
+# GEMM, output widths that end inside a weight tile.
+PROJ = [(768, 3, 1, 129), (328, 12, 4, 180), (512, 2, 1, 211), (1536, 12, 4, 256),
+        (2560, 16, 2, 257), (384, 6, 1, 513), (1024, 6, 1, 768), (1000, 6, 1, 769)]
+
+
+@pytest.mark.parametrize("D,Hq,Hkv,T", PROJ, ids=lambda v: str(v))
+def test_projections_of_many_tokens(D, Hq, Hkv, T):
+    """The whole block on one prompt against the oracle."""
+    m = moe()
+    rng = np.random.default_rng(D + T)
+    shape = gen.AttnShape(D, Hq, Hkv, 128, 10000.0, "bf16")
+    w_qkv, w_o = gen.host_attn_weights(shape, 91)
+    kc, vc = gen.host_kv_cache(shape, 2, T + 5, 91)
+    seq, pos = np.ones(T, np.int32), np.arange(3, T + 3, dtype=np.int32)
+    x = rng.normal(size=(T, D)).astype(np.float32)
+    want, _, _ = oracle.sa_forward(x.astype(np.float64), w_qkv, w_o, "bf16", Hq, Hkv,
+                                   shape.rope_base, EPS, seq, pos, gen.to_f64(kc, "bf16"),
+                                   gen.to_f64(vc, "bf16"))
+    resid = torch.from_numpy(x).cuda()
+    m.sa_forward(_sa(m, shape), resid, dev(w_qkv, "bf16"), dev(w_o, "bf16"),
+                 torch.from_numpy(seq).cuda(), torch.from_numpy(pos).cuda(), dev(kc, "bf16"),
+                 dev(vc, "bf16"), eps=EPS)
+    assert m.get_last_error() == 0
+    # the first positions average few values and are several times as large as
+    # the last ones (0.44 against an RMS of 0.09 over 256 rows); the bf16
+    # roundings of a row's probabilities and context are relative to its own
+    # values, so each row is held to the bound on its own RMS
+    scale = 1.0 / np.sqrt(np.mean((want - x) ** 2, axis=1, keepdims=True))
+    assert_parity((to_numpy(resid) - x) * scale, (want - x) * scale, "bf16",
+                  "attention block")
