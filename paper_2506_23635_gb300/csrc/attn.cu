@@ -15,7 +15,7 @@
 //                  it lets the projection launch at once (the projection's
 //                  weight loads do not depend on it);
 //   projection     W_qkv . x: the tcgen05 kernel with the weights as the M
-//                  operand (split reduction) for up to 768 tokens, the grouped
+//                  operand (split reduction) for up to 640 tokens, the grouped
 //                  tcgen05 GEMM with E = 1 beyond (fp32 out);
 //   k_rope_cache   rotary embedding of q and k (angles formed and reduced in
 //                  fp64, evaluated in fp32), k and v written to the cache in

@@ -368,7 +368,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 
 // ---- one weight matrix against a few token rows (weights as the M operand) -------
 //
-// y[j, n] = x[j, :] . W[n, :] for j < T <= 768 tokens, in near-equal runs of at
+// y[j, n] = x[j, :] . W[n, :] for j < T <= 640 tokens, in near-equal runs of at
 // most 256 (gridDim.z), and the Nw rows of one matrix W [Nw, Kdim].  A decode
 // batch fills few of the 128 slot rows of the
 // MMA above, and a single matrix has few 256-row tiles; here the weights are
@@ -510,15 +510,25 @@ k_gemm_swap(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         } else if (ptx::mbar_wait(&hd->tfull, 0, err)) {
             tc_fence_after();
             const uint32_t base = tmem + ((uint32_t)(q * 32) << 16);
+            // whole chunks of 32 tokens without a bound on each, 32-bit offsets
+            // (a 64-bit product and two bounds for every store cost 1-2 us
+            // of the attention block's two projections at 256 tokens and more)
+            float *yc = y_out + n;
+            const uint32_t row = (uint32_t)Nw;
+            const int rows = n < Nw ? min(NTOK, T) : 0;
 #pragma unroll 1
-            for (int c = 0; c < NTOK; c += 32) {
+            for (int c = 0; c < NTOK; c += 32, yc += (size_t)32 * row) {
                 float v[32];
                 tmem_ld32(base + c, v);
                 tmem_ld_wait();
-                if (n < Nw) {
+                const int left = rows - c;
+                if (left >= 32) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) yc[j * row] = v[j];
+                } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        if (c + j < NTOK && c + j < T) y_out[(size_t)(c + j) * Nw + n] = v[j];
+                        if (j < left) yc[j * row] = v[j];
                 }
             }
         }

@@ -408,9 +408,12 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                 const int p = q & 1;
                 const bool is_a = (q < 2) != (a_mode == 2);
                 const int f = (t.wt * CG + (int)rank) * C::kOutPerCta + p * 32 + lane;
-                const bool f_ok = f < Nw;
+                const bool f_ok = f < Nw && !dead;
+                // (addresses and bounds as in DOWN below)
+                const uint32_t row = (uint32_t)Nw;
+                bf16 *hc = h_out + (j0 + (is_a ? 0 : 16)) * Nw + f;
 #pragma unroll 1
-                for (int c = 0; c < t.n; c += 32, ++chunk) {
+                for (int c = 0; c < t.n; c += 32, ++chunk, hc += (size_t)32 * row) {
                     float v[32];
                     if (!dead) {
                         tmem_ld32(base + c, v);
@@ -426,30 +429,47 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 #pragma unroll
                     for (int i = 0; i < 16; ++i) mine[i * 32 + lane] = is_a ? v[16 + i] : v[i];
                     ptx::named_bar_sync(1 + p, 64);
-                    const int col0 = c + (is_a ? 0 : 16);
+                    const int left = f_ok ? t.cnt - c - (is_a ? 0 : 16) : 0;
+                    bf16 hv[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float o = theirs[i * 32 + lane];
-                        const float hv = is_a ? silu(v[i]) * o : silu(o) * v[16 + i];
-                        const int col = col0 + i;
-                        if (!dead && f_ok && col < t.cnt)
-                            h_out[(j0 + col) * Nw + f] = __float2bfloat16_rn(hv);
+                        hv[i] = __float2bfloat16_rn(is_a ? silu(v[i]) * o : silu(o) * v[16 + i]);
+                    }
+                    if (left >= 16) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) hc[i * row] = hv[i];
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (i < left) hc[i * row] = hv[i];
                     }
                 }
             } else {
                 const int dcol = (t.wt * CG + (int)rank) * C::kOutPerCta + q * 32 + lane;
                 const bool d_ok = dcol < Nw && !dead;
+                // whole chunks of 32 slots without a bound on each, 32-bit
+                // offsets from the chunk's first row: an expert of 1024 hidden
+                // units gives the MMAs 16 stages a tile, and with a 64-bit
+                // product and a bound for every store the four warps took 2.4
+                // times as long as those (12,000 slots: 206 us)
+                float *yc = y_out + j0 * Nw + dcol;
+                const uint32_t row = (uint32_t)Nw;
 #pragma unroll 1
-                for (int c = 0; c < t.n; c += 32) {
+                for (int c = 0; c < t.n; c += 32, yc += (size_t)32 * row) {
                     float v[32];
                     if (!dead) {
                         tmem_ld32(base + c, v);
                         tmem_ld_wait();
                     }
-                    if (d_ok) {
+                    const int left = t.cnt - c;
+                    if (d_ok && left >= 32) {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) yc[i * row] = v[i];
+                    } else if (d_ok) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i)
-                            if (c + i < t.cnt) y_out[(j0 + c + i) * Nw + dcol] = v[i];
+                            if (i < left) yc[i * row] = v[i];
                     }
                 }
             }

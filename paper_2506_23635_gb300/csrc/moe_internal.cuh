@@ -259,10 +259,9 @@ cudaError_t launch_gemm_up_tc(const moe_dims &d, int T, const void *x_sorted,
 // land in y + p*T*Nw for p < parts (the caller adds them in order).
 // gemm_rows_parts: the split that keeps the SMs streaming for this shape.
 // (the last size that the CTA-pair GEMM does not beat: attention block of DBRX,
-// two projections, on this kernel and on that: 130 tokens 70 and 99 us, 256: 82
-// and 109, 400: 107 and 129, 512: 126 and 142, 600: 149 and 162, 768: 176 and
-// 177, 1000: 230 and 219, 1200: 282 and 260)
-constexpr int kRowsMaxTokens = 768;
+// two projections, on this kernel and on that: 300 tokens 94 and 106 us, 400:
+// 105 and 115, 512: 125 and 127, 600: 148 and 152, 700: 170 and 161)
+constexpr int kRowsMaxTokens = 640;
 constexpr int kRowsMaxParts = 4;
 int gemm_rows_parts(int T, int Kdim, int Nw);
 cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const void *w, int parts,

@@ -594,7 +594,7 @@ def test_ragged_tiles_and_listed_tokens(Hq, Hkv, L, runs):
 # of 256 and over two, the last size of this kernel and the first of the pair
 # GEMM, output widths that end inside a weight tile.
 PROJ = [(768, 3, 1, 129), (328, 12, 4, 180), (512, 2, 1, 211), (1536, 12, 4, 256),
-        (2560, 16, 2, 257), (384, 6, 1, 513), (1024, 6, 1, 768), (1000, 6, 1, 769)]
+        (2560, 16, 2, 257), (384, 6, 1, 513), (1024, 6, 1, 640), (1000, 6, 1, 641)]
 
 
 @pytest.mark.parametrize("D,Hq,Hkv,T", PROJ, ids=lambda v: str(v))
