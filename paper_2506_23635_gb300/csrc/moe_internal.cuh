@@ -335,14 +335,12 @@ cudaError_t launch_gemm_down_wm(const moe_dims &d, int T, const void *h, const i
                                 const void *w2, float *y_sorted, cudaStream_t st,
                                 const char *name);
 
-// Router logits of batches of 128 or more tokens on the tensor cores
-// (route_tc.cu), E <= 16, bf16: partial logits of ksplit shares of d in
-// `scratch` (route_tc_scratch_bytes), then top-k and gates as moe_route.
+// Router of larger batches on the tensor cores (route_tc.cu), E <= 16, bf16:
+// logits, top-k and gates as moe_route.
+constexpr int kRouteTcMinTokens = 128;
 bool route_tc_ok(const moe_dims &d, int T);
-size_t route_tc_scratch_bytes(const moe_dims &d, int T);
 cudaError_t launch_route_tc(const moe_dims &d, int T, const void *x, const void *wr,
-                            float *logits, int32_t *idx, float *gate, float *scratch,
-                            cudaStream_t st);
+                            float *logits, int32_t *idx, float *gate, cudaStream_t st);
 
 // Bulk-copy pipelined decode kernels (ffn_stream.cu), bf16 only, up to
 // kStreamMaxSlots slots; the GLU hidden vectors h are bf16.  Batches of at

@@ -434,3 +434,49 @@ def test_size_extremes(case):
     gi, _, _ = m.route(d, x, w_r)
     assert np.array_equal(gi.cpu().numpy()[toks], idx)
     assert_parity(to_numpy(out)[toks], want, dt, f"extremes {case}")
+
+
+@pytest.mark.parametrize("S,E,K", [(1024, 16, 4), (1026, 16, 2), (1032, 3, 1), (8192, 256, 8),
+                                   (12004, 16, 4), (65536, 16, 4), (65540, 16, 4), (9000, 200, 1)])
+def test_dispatch_sizes(S, E, K):
+    """Stable order, counts and offsets at the ends of the dispatch kernels'
+    ranges (one CTA, a cluster of 8 with ragged and full shares, the general
+    kernel), one expert unused; entries outside [0, E) are left out."""
+    m = moe()
+    rng = np.random.default_rng(S + E)
+    idx = rng.integers(0, E, size=S).astype(np.int32)
+    idx[idx == E // 2] = 0
+    d = m.dims(64, 64, E, K, torch.bfloat16)
+    got = [a.cpu().numpy() for a in m.dispatch(d, torch.from_numpy(idx.reshape(-1, K)).cuda())]
+    assert m.get_last_error() == 0
+    perm = np.argsort(idx, kind="stable")
+    inv = np.empty(S, np.int64)
+    inv[perm] = np.arange(S)
+    counts = np.bincount(idx, minlength=E)
+    for g, w in zip(got, (counts, np.concatenate([[0], np.cumsum(counts)]), perm, inv)):
+        assert np.array_equal(g, w)
+
+
+@pytest.mark.parametrize("T,D,E,K", [(128, 8, 4, 2), (129, 520, 16, 4), (300, 6144, 16, 4),
+                                     (257, 40000, 5, 5), (1000, 72, 1, 1)])
+def test_route_many_tokens(T, D, E, K):
+    """The tensor-core router (128 tokens and more): shares of d with no block
+    and with ragged ones, two ring stages, a last tile of one token; logits and
+    gates against fp64, as close as 32-bit sums are."""
+    m = moe()
+    g = torch.Generator().manual_seed(T + D)
+    x = torch.randn(T, D, generator=g).bfloat16()
+    w = (torch.randn(D, E, generator=g) * 0.02).bfloat16()
+    d = m.dims(D, 64, E, K, torch.bfloat16)
+    idx, gate, logits = m.route(d, x.cuda(), w.cuda(), want_logits=True)
+    assert m.get_last_error() == 0
+    want = x.double() @ w.double()
+    # D products of magnitude |x w| summed in fp32: sqrt(D) roundings of 2^-24
+    # of the running sum (at most the sum's own scale) with a factor of 8
+    tol = 8 * D ** 0.5 * 2.0 ** -24 * 0.02 * D ** 0.5
+    assert float((logits.cpu().double() - want).abs().max()) <= tol
+    l64 = logits.cpu().double()
+    order = l64.sort(dim=1, descending=True, stable=True).indices[:, :K]
+    assert torch.equal(idx.cpu().long(), order)
+    p = l64.gather(1, order).softmax(dim=1)
+    assert float((gate.cpu().double() - p).abs().max()) <= 1e-6
