@@ -480,3 +480,22 @@ def test_route_many_tokens(T, D, E, K):
     assert torch.equal(idx.cpu().long(), order)
     p = l64.gather(1, order).softmax(dim=1)
     assert float((gate.cpu().double() - p).abs().max()) <= 1e-6
+
+
+@pytest.mark.parametrize("case", [(8, 8, 1, 1, 1), (72, 40, 3, 2, 9), (200, 64, 5, 5, 64), (600, 72, 2, 1, 33),
+                                  (1304, 64, 8, 3, 64), (64, 128, 40, 2, 30)],
+                         ids=lambda c: "D{}F{}E{}K{}T{}".format(*c))
+def test_fp32_down_projection_splits(case):
+    """fp32 layers whose output rows are taken by one, two, four and eight
+    warps (few rows, few experts, more experts than warps), a last block with
+    missing rows, a residual added once."""
+    m = moe()
+    D, F, E, K, T = case
+    L = _host((D, F, E, K, T, "f32"), seed=31)
+    d = _dims(m, L.shape)
+    x, w_r, w1, v1, w2 = _devlayer(L)
+    res = torch.randn(T, D, generator=torch.Generator().manual_seed(D)).cuda()
+    want, _, _ = oracle.layer_tokens(L.x, L.w_r, L.w1, L.v1, L.w2, "f32", K)
+    out = m.layer_forward(d, x, w_r, w1, v1, w2, residual=res)
+    assert m.get_last_error() == 0
+    assert_parity(to_numpy(out), want + to_numpy(res), "f32", f"fp32 layer {case}")
