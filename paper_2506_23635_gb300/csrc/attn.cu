@@ -824,7 +824,7 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
         e = launch_gemm_rows_tc(c.T, c.d.d_model, c.nr(), xn, w_qkv, n_part, qkv, c.st,
                                 "qkv_rows_tc");
     } else {
-        e = launch_gemm_down_tc(pd, c.T, xn, offsets, w_qkv, qkv, c.st, "qkv_gemm_tc");
+        e = launch_gemm_down_wm(pd, c.T, xn, offsets, w_qkv, qkv, c.st, "qkv_gemm_tc");
     }
     if (e != cudaSuccess) return e;
     long long pstride = (long long)c.T * c.nr();
@@ -957,7 +957,7 @@ cudaError_t out_proj(const SaCall &c, const void *ctx, const void *w_o, float *r
         n_part = gemm_rows_parts(c.T, c.nq(), c.d.d_model);
         e = launch_gemm_rows_tc(c.T, c.nq(), c.d.d_model, ctx, w_o, n_part, y, c.st, "o_rows_tc");
     } else {
-        e = launch_gemm_down_tc(pd, c.T, ctx, offsets, w_o, y, c.st, "o_gemm_tc");
+        e = launch_gemm_down_wm(pd, c.T, ctx, offsets, w_o, y, c.st, "o_gemm_tc");
     }
     if (e != cudaSuccess) return e;
     if (xn_next) {

@@ -313,7 +313,10 @@ cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, cons
 
 // name: the profiling name of the launch (default "gemm_down_tc").  y_tail
 // (optional, [T*K, D]): the stream-K schedule's second output; the result is
-// then y_sorted + y_tail.
+// then y_sorted + y_tail.  The 128-slot-tile kernels of both projections read
+// the offsets before their dependency wait: the launch ahead of the up
+// projection is launch_gather_rows, that ahead of the down projection the up
+// projection, and either lets the next one launch after its own wait.
 cudaError_t launch_gemm_down_tc(const moe_dims &d, int T, const void *h, const int32_t *offsets,
                                 const void *w2, float *y_sorted, cudaStream_t st,
                                 const char *name = nullptr, float *y_tail = nullptr);
