@@ -428,7 +428,7 @@ static_assert(sizeof(SwapHeader) <= kTcHeaderBytes, "swap kernel header too larg
 template <int NTOK>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 k_gemm_swap(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-            int T, int Kdim, int Nw, float *__restrict__ y_out, unsigned *err) {
+            int T, int Kdim, int Nw, int add, float *__restrict__ y_out, unsigned *err) {
     using C = SwapCfg<NTOK>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
@@ -538,6 +538,13 @@ k_gemm_swap(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
                 tmem_ld32(base + c, v);
                 tmem_ld_wait();
                 const int left = rows - c;
+                if (add) {
+                    float o[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) o[j] = j < left ? yc[j * row] : 0.f;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] += o[j];
+                }
                 if (left >= 32) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) yc[j * row] = v[j];
@@ -639,7 +646,7 @@ uint32_t a_box_rows(int T) {
 
 template <int NTOK>
 cudaError_t launch_swap(const CUtensorMap &w, const CUtensorMap &x, int T, int Kdim, int Nw,
-                        int parts, float *y, cudaStream_t st, const char *name) {
+                        int parts, float *y, cudaStream_t st, const char *name, bool add) {
     using C = SwapCfg<NTOK>;
     const void *kern = (const void *)k_gemm_swap<NTOK>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -647,7 +654,8 @@ cudaError_t launch_swap(const CUtensorMap &w, const CUtensorMap &x, int T, int K
     if (e != cudaSuccess) return e;
     unsigned *err = device_info().err;
     CUtensorMap mw = w, mx = x;
-    void *args[] = {&mw, &mx, &T, &Kdim, &Nw, &y, &err};
+    int addv = add ? 1 : 0;
+    void *args[] = {&mw, &mx, &T, &Kdim, &Nw, &addv, &y, &err};
     LaunchScope ls(name ? name : "gemm_rows_tc", st);
     return launch_pdl(kern, dim3((Nw + BM - 1) / BM, parts, (T + 255) / 256), dim3(kThreadsTc), C::kSmem, st,
                       args);
@@ -714,8 +722,8 @@ int gemm_rows_parts(int T, int Kdim, int Nw) {
 }
 
 cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const void *w, int parts,
-                                float *y, cudaStream_t st, const char *name) {
-    if (T < 1 || T > kRowsMaxTokens || parts < 1 || parts > kRowsMaxParts)
+                                float *y, cudaStream_t st, const char *name, bool add) {
+    if (T < 1 || T > kRowsMaxTokens || parts < 1 || parts > kRowsMaxParts || (add && parts > 1))
         return cudaErrorInvalidValue;
     const int runs = (T + 255) / 256;  // of at most 256 tokens, near-equal
     const int ntok = ((T + runs - 1) / runs + 15) / 16 * 16;
@@ -731,14 +739,14 @@ cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const vo
     if (!make_map(&mw, w, (uint64_t)Nw, (uint64_t)Kdim, BM) ||
         !make_map(&mx, x, (uint64_t)T, (uint64_t)Kdim, xrows))
         return cudaErrorInvalidValue;
-    if (xrows == 16) return launch_swap<16>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    if (xrows == 32) return launch_swap<32>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    if (xrows == 64) return launch_swap<64>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    if (xrows == 128) return launch_swap<128>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    if (xrows == 160) return launch_swap<160>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    if (xrows == 192) return launch_swap<192>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    if (xrows == 224) return launch_swap<224>(mw, mx, T, Kdim, Nw, parts, y, st, name);
-    return launch_swap<256>(mw, mx, T, Kdim, Nw, parts, y, st, name);
+    if (xrows == 16) return launch_swap<16>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    if (xrows == 32) return launch_swap<32>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    if (xrows == 64) return launch_swap<64>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    if (xrows == 128) return launch_swap<128>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    if (xrows == 160) return launch_swap<160>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    if (xrows == 192) return launch_swap<192>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    if (xrows == 224) return launch_swap<224>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
+    return launch_swap<256>(mw, mx, T, Kdim, Nw, parts, y, st, name, add);
 }
 
 }  // namespace moe

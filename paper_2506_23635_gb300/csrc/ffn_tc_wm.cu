@@ -235,14 +235,14 @@ template <int MODE, int CG>
 __global__ void __launch_bounds__(kWmThreads, 1)
 k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
           const __grid_constant__ SlotMaps tmB, int a_mode, const int32_t *__restrict__ offsets,
-          int E, int S, int Kdim, int Nw, bf16 *__restrict__ h_out, float *__restrict__ y_out,
-          unsigned *err) {
+          int E, int S, int Kdim, int Nw, int add, bf16 *__restrict__ h_out,
+          float *__restrict__ y_out, unsigned *err) {
     // DOWN: tmA0 = W2 [E*D, F] (128-row box).  UP, a_mode 0: tmA0 = W1 and
     // tmA1 = V1, [E*F, D] each (64-row boxes); a_mode 1 / 2: tmA0 = both as
     // one 3-D tensor [2][E*F][D] (box 64 rows x 2), W1 first (1) or V1
     // first (2).  tmB: the sorted slot rows [S, Kdim] (x_sorted for UP, h
     // for DOWN).  Kdim: reduction length; Nw: output width
-    // (F for UP, D for DOWN).
+    // (F for UP, D for DOWN).  add (DOWN): the result is added to y_out.
     using C = WmCfg<MODE, CG>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
@@ -463,6 +463,13 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                         tmem_ld_wait();
                     }
                     const int left = t.cnt - c;
+                    if (add && d_ok) {
+                        float o[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) o[i] = i < left ? yc[i * row] : 0.f;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] += o[i];
+                    }
                     if (d_ok && left >= 32) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) yc[i * row] = v[i];
@@ -497,13 +504,15 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
 template <int MODE, int CG>
 cudaError_t launch_wm_cg(const CUtensorMap &a0, const CUtensorMap &a1, const SlotMaps &b,
                          int a_mode, const int32_t *offsets, int E, int S, int Kdim, int Nw,
-                         bf16 *h, float *y, int grid, cudaStream_t st, const char *name) {
+                         int add, bf16 *h, float *y, int grid, cudaStream_t st,
+                         const char *name) {
     using C = WmCfg<MODE, CG>;
     const void *kern = (const void *)k_gemm_wm<MODE, CG>;
     unsigned *err = device_info().err;
     CUtensorMap m0 = a0, m1 = a1;
     SlotMaps mb = b;
-    void *args[] = {&m0, &m1, &mb, &a_mode, &offsets, &E, &S, &Kdim, &Nw, &h, &y, &err};
+    void *args[] = {&m0, &m1, &mb, &a_mode, &offsets, &E, &S, &Kdim, &Nw, &add, &h,
+                    &y, &err};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kWmThreads);
@@ -575,19 +584,19 @@ bool single_cta_forced() {
 
 template <int MODE>
 cudaError_t launch_wm(const CUtensorMap (&a)[2], const void *slots, int a_mode,
-                      const int32_t *offsets, int E, int S, int Kdim, int Nw, bf16 *h, float *y,
-                      cudaStream_t st, const char *name) {
+                      const int32_t *offsets, int E, int S, int Kdim, int Nw, int add, bf16 *h,
+                      float *y, cudaStream_t st, const char *name) {
     const int pairs = single_cta_forced() ? 0 : wm_pairs<MODE>();
     SlotMaps b;
     if (!slot_maps(b, slots, S, Kdim, pairs > 0 ? 8 : 16)) return cudaErrorInvalidValue;
     if (pairs > 0)
-        return launch_wm_cg<MODE, 2>(a[0], a[1], b, a_mode, offsets, E, S, Kdim, Nw, h, y,
+        return launch_wm_cg<MODE, 2>(a[0], a[1], b, a_mode, offsets, E, S, Kdim, Nw, add, h, y,
                                      2 * pairs, st, name);
     const void *kern = (const void *)k_gemm_wm<MODE, 1>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)WmCfg<MODE, 1>::kSmem);
     if (e != cudaSuccess) return e;
-    return launch_wm_cg<MODE, 1>(a[0], a[1], b, a_mode, offsets, E, S, Kdim, Nw, h, y,
+    return launch_wm_cg<MODE, 1>(a[0], a[1], b, a_mode, offsets, E, S, Kdim, Nw, add, h, y,
                                  device_info().sm_count, st, name);
 }
 
@@ -631,18 +640,18 @@ cudaError_t launch_gemm_up_wm(const moe_dims &d, int T, const void *x_sorted,
             return cudaErrorInvalidValue;
         a_mode = 0;
     }
-    return launch_wm<kWmUp>(a, x_sorted, a_mode, offsets, E, S, D, F, static_cast<bf16 *>(h), nullptr, st,
+    return launch_wm<kWmUp>(a, x_sorted, a_mode, offsets, E, S, D, F, 0, static_cast<bf16 *>(h), nullptr, st,
                             "gemm_up_glu_tc");
 }
 
 cudaError_t launch_gemm_down_wm(const moe_dims &d, int T, const void *h, const int32_t *offsets,
                                 const void *w2, float *y_sorted, cudaStream_t st,
-                                const char *name) {
+                                const char *name, bool add) {
     const int S = T * d.top_k, D = d.d_model, F = d.ffn_hidden, E = d.n_experts;
     CUtensorMap a[2];
     if (!make_map(&a[0], w2, (uint64_t)E * D, (uint64_t)F, 128)) return cudaErrorInvalidValue;
     a[1] = a[0];
-    return launch_wm<kWmDown>(a, h, 0, offsets, E, S, F, D, nullptr, y_sorted, st,
+    return launch_wm<kWmDown>(a, h, 0, offsets, E, S, F, D, add ? 1 : 0, nullptr, y_sorted, st,
                               name ? name : "gemm_down_tc");
 }
 

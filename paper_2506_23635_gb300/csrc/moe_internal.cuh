@@ -264,8 +264,10 @@ cudaError_t launch_gemm_up_tc(const moe_dims &d, int T, const void *x_sorted,
 constexpr int kRowsMaxTokens = 640;
 constexpr int kRowsMaxParts = 4;
 int gemm_rows_parts(int T, int Kdim, int Nw);
+// add (one part): the result is added to y.
 cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const void *w, int parts,
-                                float *y, cudaStream_t st, const char *name = nullptr);
+                                float *y, cudaStream_t st, const char *name = nullptr,
+                                bool add = false);
 // How the tokens of an attention call are shared between the kernels, found on
 // the device (plan_attention in attn.cu): the tiles of the tensor-core prefill
 // attention, longest first, and the tokens that none of them holds.
@@ -336,7 +338,7 @@ cudaError_t launch_gemm_up_wm(const moe_dims &d, int T, const void *x_sorted,
                               cudaStream_t st);
 cudaError_t launch_gemm_down_wm(const moe_dims &d, int T, const void *h, const int32_t *offsets,
                                 const void *w2, float *y_sorted, cudaStream_t st,
-                                const char *name);
+                                const char *name, bool add = false);
 
 // Router of larger batches on the tensor cores (route_tc.cu), E <= 16, bf16:
 // logits, top-k and gates as moe_route.
