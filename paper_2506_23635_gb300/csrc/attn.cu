@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kRopeThreads)
 k_rope_cache(int T, int Hq, int Hkv, int n_seq, int L, RopeRates rates,
              const int32_t *__restrict__ seq, const int32_t *__restrict__ pos,
              const float *__restrict__ qkv, int n_part, long long part_stride,
-             float *__restrict__ q, bf16 *__restrict__ q16, bf16 *__restrict__ kc,
+             const ProjSplit split, float *__restrict__ q, bf16 *__restrict__ q16, bf16 *__restrict__ kc,
              bf16 *__restrict__ vc, int *__restrict__ dec_count, unsigned *err) {
     // the tensor-core attention, one CTA per SM on the SMs that this grid
     // leaves free, may launch now and set itself up while this kernel runs
@@ -322,13 +322,24 @@ k_rope_cache(int T, int Hq, int Hkv, int n_seq, int L, RopeRates rates,
     // in flight while the angles are formed), the projection's partial sums
     // added in order
     const bool row_ok = hr < Hq + 2 * Hkv;
+    // n_part 0: as many parts as the projection's split left each (row, token)
+    __shared__ int np_s[kRopeTokens][kRopeRows];
+    if (n_part == 0) {
+        if (threadIdx.x < kRopeTokens * kRopeRows) {
+            const int u = threadIdx.x / kRopeRows, r = threadIdx.x % kRopeRows;
+            np_s[u][r] = split.parts(T, min(tb + u, T - 1),
+                                     min((int)blockIdx.x * kRopeRows + r, Hq + 2 * Hkv - 1) * kHeadDim);
+        }
+        __syncthreads();
+    }
     float2 av[kRopeTokens], bv[kRopeTokens];
 #pragma unroll
     for (int u = 0; u < kRopeTokens; ++u) {
         av[u] = bv[u] = make_float2(0.f, 0.f);
         if (row_ok && u < nt) {
             const float *row = qkv + (size_t)(tb + u) * (nq + 2 * nkv) + (size_t)hr * kHeadDim + i;
-            for (int k = 0; k < n_part; ++k) {
+            const int np = n_part > 0 ? n_part : np_s[u][threadIdx.x / 32];
+            for (int k = 0; k < np; ++k) {
                 const float2 a = *reinterpret_cast<const float2 *>(row + k * part_stride);
                 const float2 b = *reinterpret_cast<const float2 *>(row + k * part_stride + H2);
                 av[u].x += a.x;
@@ -758,7 +769,8 @@ SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
     // kRowsMaxTokens tokens): qkv first, later the output projection's rows
     // (as many rows as any smaller call needs, too)
     const size_t part_rows =
-        std::max<size_t>(T, (size_t)kRowsMaxParts * std::min<int64_t>(T, kRowsMaxTokens));
+        std::max({(size_t)T, (size_t)kRowsMaxParts * std::min<int64_t>(T, kRowsMaxTokens),
+                  (size_t)2 * std::min<int64_t>(T, kProjSplitMaxTokens)});
     L.qkv = o; o += up(part_rows * std::max(nr, (size_t)d.d_model) * 4);
     L.q = o; o += up((size_t)T * nq * 4);
     L.q16 = o; o += up((size_t)T * nq * 2);
@@ -836,7 +848,11 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
     float *qkv = at<float>(c.ws, c.L.qkv);
     cudaError_t e;
     int n_part = 1;
-    if (c.T <= kRowsMaxTokens) {
+    ProjSplit split{};
+    if (proj_split(c.T, c.d.d_model, c.nr(), &split)) {
+        n_part = 0;
+        e = launch_proj_wm(c.T, c.d.d_model, c.nr(), xn, w_qkv, qkv, split, c.st, "qkv_gemm_tc");
+    } else if (c.T <= kRowsMaxTokens) {
         n_part = gemm_rows_parts(c.T, c.d.d_model, c.nr());
         e = launch_gemm_rows_tc(c.T, c.d.d_model, c.nr(), xn, w_qkv, n_part, qkv, c.st,
                                 "qkv_rows_tc");
@@ -855,7 +871,7 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
     int Tv = c.T;
     int *dec_count = q16 ? at<int>(c.ws, c.L.dec_count) : nullptr;
     void *args[] = {&Tv,     &Hq,      &Hkv, &ns,  &Lv,  &rates, &seq, &pos,
-                    &qkvc,   &n_part,  &pstride, &q, &q16, &kcp, &vcp, &dec_count, &err};
+                    &qkvc,   &n_part,  &pstride, &split, &q, &q16, &kcp, &vcp, &dec_count, &err};
     LaunchScope ls("rope_cache", c.st);
     const int rows = Hq + 2 * Hkv;
     return launch_pdl((const void *)k_rope_cache,

@@ -11,6 +11,10 @@
 //   UP   (GLU):  h[j, f] = SiLU(x_j . W1[e,f,:]) * (x_j . V1[e,f,:])   -> bf16
 //   DOWN:        y[j, d] = h[j, :] . W2[e,d,:]                          -> fp32
 //
+//   PROJ         y = x . W^T of one matrix (the attention block's projection),
+//                as DOWN with one expert, each CTA pair an equal share of all
+//                (unit, k-block)s (ProjSplit): y in one or two parts
+//
 // A unit of work is (expert e, weight tile, slot tile).
 //  * Weight tile: 128 A rows per CTA.  UP: 64 rows of W1 and the same 64
 //    rows of V1 (one 3-D copy over the two tensors when their distance
@@ -70,7 +74,7 @@ constexpr int kWmMaxStages = 8;
 constexpr size_t kWmHeaderBytes = 2048;
 constexpr uint32_t kWmTmemCols = 512;  // two 256-column accumulators
 
-enum WmMode { kWmUp = 0, kWmDown = 1 };
+enum WmMode { kWmUp = 0, kWmDown = 1, kWmProj = 2 };
 
 template <int MODE, int CG>
 struct WmCfg {
@@ -194,6 +198,48 @@ __device__ __forceinline__ bool wm_item(const int *tprefix, const int32_t *offse
     return true;
 }
 
+// The items of pair (or CTA) `pair`: tile, the k-blocks [kb0, kb1) of it, and
+// (PROJ) which part of the result they give.
+template <int MODE>
+struct WmItems {
+    const int *tprefix;
+    const int32_t *offsets;
+    int E, S, n_units, pair, n_pairs, gran, nk;
+    ProjSplit split;
+    int i = 0, pos = 0, end = 0;
+    __device__ __forceinline__ void start() {
+        if (MODE == kWmProj) {
+            const int W = n_units * nk;
+            pos = W * pair / n_pairs;
+            end = W * (pair + 1) / n_pairs;
+        }
+    }
+    __device__ __forceinline__ bool next(WmTile &t, int &kb0, int &kb1, int &part) {
+        if (MODE == kWmProj) {
+            if (pos >= end) return false;
+            const int u = pos / nk;
+            kb0 = pos - u * nk;
+            kb1 = min(nk, kb0 + end - pos);
+            pos += kb1 - kb0;
+            part = pair - split.owner(u * nk);
+            t.e = 0;
+            t.wt = u / split.nst;
+            const int st = u - t.wt * split.nst;
+            t.s0 = split.run_start(S, st);
+            t.cnt = split.run_start(S, st + 1) - t.s0;
+            t.n = (t.cnt + gran - 1) / gran * gran;
+            return true;
+        }
+        kb0 = 0;
+        kb1 = nk;
+        part = 0;
+        do {
+            if (!wm_item(tprefix, offsets, E, n_units, pair, n_pairs, i++, gran, t)) return false;
+        } while (t.cnt == 0);
+        return true;
+    }
+};
+
 // A tensor copy that completes on the mbarrier at cluster address `bar` --
 // this CTA's or, in a CTA pair, the peer's (cta_group::2).
 template <int CG>
@@ -236,7 +282,7 @@ __global__ void __launch_bounds__(kWmThreads, 1)
 k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
           const __grid_constant__ SlotMaps tmB, int a_mode, const int32_t *__restrict__ offsets,
           int E, int S, int Kdim, int Nw, int add, bf16 *__restrict__ h_out,
-          float *__restrict__ y_out, unsigned *err) {
+          float *__restrict__ y_out, const ProjSplit split, unsigned *err) {
     // DOWN: tmA0 = W2 [E*D, F] (128-row box).  UP, a_mode 0: tmA0 = W1 and
     // tmA1 = V1, [E*F, D] each (64-row boxes); a_mode 1 / 2: tmA0 = both as
     // one 3-D tensor [2][E*F][D] (box 64 rows x 2), W1 first (1) or V1
@@ -277,14 +323,23 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         if (CG == 2) tmem_alloc_pair(&hd->tmem_base, kWmTmemCols);
         else tmem_alloc(&hd->tmem_base, kWmTmemCols);
     }
-    ptx::grid_dependency_wait();  // offsets and the slot rows come from earlier kernels
-    if (warp == 2) wm_prefix(offsets, E, S, nwt, hd->tprefix, err);
+    // offsets and the slot rows come from earlier kernels (PROJ: no offsets,
+    // and the weights of the first stages are loaded before the wait)
+    if (MODE != kWmProj) {
+        ptx::grid_dependency_wait();
+        if (warp == 2) wm_prefix(offsets, E, S, nwt, hd->tprefix, err);
+    }
     tc_fence_before();
     if (CG == 2) ptx::cluster_sync_all();  // barriers initialised in both CTAs
     else __syncthreads();
     tc_fence_after();
     const uint32_t tmem = hd->tmem_base;
-    const int n_units = hd->tprefix[E];
+    WmItems<MODE> items{hd->tprefix, offsets, E, S,
+                        MODE == kWmProj ? nwt * split.nst : hd->tprefix[E], unit0, ustride,
+                        C::kGran, nk, split};
+    items.start();
+    WmTile t;
+    int kb0, kb1, part;
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -296,16 +351,32 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
             const uint64_t pol_x = ptx::policy_evict_last();
             uint32_t it = 0;
             bool ok = true;
-            WmTile t;
-            for (int i = 0; ok && wm_item(hd->tprefix, offsets, E, n_units, unit0, ustride, i,
-                                          C::kGran, t);
-                 ++i) {
-                if (t.cnt == 0) continue;
+            // PROJ: how many stages of the first item have their weights sent
+            // before the slot rows may be read
+            uint32_t early = 0;
+            if (MODE == kWmProj) {
+                WmItems<MODE> peek = items;
+                if (peek.next(t, kb0, kb1, part)) {
+                    const int arow = (t.wt * CG + (int)rank) * C::kOutPerCta;
+                    early = (uint32_t)min(kStages, kb1 - kb0);
+                    for (uint32_t s = 0; s < early; ++s) {
+                        uint64_t *fb = &hd->full[s];
+                        const uint32_t fbc = CG == 2 ? ptx::map_rank(ptx::smem_u32(fb), 0) : 0u;
+                        if (issuer)
+                            ptx::mbar_arrive_expect_tx(
+                                fb, (kStageA + (uint32_t)(t.n / CG) * (kWmBK * 2)) * CG);
+                        wm_tma<CG>(smem + s * kStageBytes, &tmA0, (kb0 + (int)s) * kWmBK, arow, fb,
+                                   fbc, pol_w);
+                    }
+                }
+                ptx::grid_dependency_wait();
+            }
+            while (ok && items.next(t, kb0, kb1, part)) {
                 const uint32_t rows_b = (uint32_t)(t.n / CG);  // a multiple of 16, <= kRowsB
                 const int brow = t.s0 + (int)(rank * rows_b);
                 const int arow = t.e * Nw + (t.wt * CG + (int)rank) * C::kOutPerCta;
 
-                for (int kb = 0; kb < nk; ++kb, ++it) {
+                for (int kb = kb0; kb < kb1; ++kb, ++it) {
                     const uint32_t s = it % kStages, ph = (it / kStages) & 1;
                     if (!(ok = ptx::mbar_wait_hint(&hd->empty[s], ph ^ 1, err))) break;
                     unsigned char *sa = smem + s * kStageBytes;
@@ -314,8 +385,11 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                     uint64_t *fb = &hd->full[s];
                     const uint32_t fbc = CG == 2 ? ptx::map_rank(ptx::smem_u32(fb), 0) : 0u;
                     // the even CTA expects the bytes of both CTAs of the pair
-                    if (issuer) ptx::mbar_arrive_expect_tx(fb, (kStageA + rows_b * (kWmBK * 2)) * CG);
-                    if (MODE == kWmUp && a_mode != 0) {
+                    if (issuer && (MODE != kWmProj || it >= early))
+                        ptx::mbar_arrive_expect_tx(fb, (kStageA + rows_b * (kWmBK * 2)) * CG);
+                    if (MODE == kWmProj && it < early) {
+                        // (the weights are on the way)
+                    } else if (MODE == kWmUp && a_mode != 0) {
                         wm_tma3<CG>(sa, &tmA0, kx, arow, fb, fbc, pol_w);
                     } else {
                         wm_tma<CG>(sa, &tmA0, kx, arow, fb, fbc, pol_w);
@@ -340,11 +414,7 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
             if (lane == 0) {
                 uint32_t it = 0, tl = 0;
                 bool ok = true;
-                WmTile t;
-                for (int i = 0; ok && wm_item(hd->tprefix, offsets, E, n_units, unit0, ustride,
-                                              i, C::kGran, t);
-                     ++i) {
-                    if (t.cnt == 0) continue;
+                while (ok && items.next(t, kb0, kb1, part)) {
                     const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
                     ++tl;
                     // released by both CTAs' epilogues
@@ -354,7 +424,7 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                     tc_fence_after();
                     const uint32_t d_tmem = tmem + acc * 256;
                     const uint32_t idesc = C::kIdescBase | ((uint32_t)(t.n >> 3) << 17);
-                    for (int kb = 0; kb < nk; ++kb, ++it) {
+                    for (int kb = kb0; kb < kb1; ++kb, ++it) {
                         const uint32_t s = it % kStages, ph = (it / kStages) & 1;
                         if (!(ok = ptx::mbar_wait_hint(&hd->full[s], ph, err))) break;
                         tc_fence_after();
@@ -362,7 +432,7 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                         const uint64_t adesc = smem_desc(sa), bdesc = smem_desc(sa + kStageA);
 #pragma unroll
                         for (int kk = 0; kk < kWmBK / 16; ++kk) {
-                            const uint32_t accum = (kb | kk) != 0 ? 1u : 0u;
+                            const uint32_t accum = (kb != kb0 || kk != 0) ? 1u : 0u;
                             if (CG == 2)
                                 mma_bf16_pair(d_tmem, adesc + 2 * kk, bdesc + 2 * kk, idesc, accum);
                             else
@@ -391,10 +461,8 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
         uint32_t tl = 0, chunk = 0;
         const uint32_t tempty_issuer0 =
             CG == 2 ? ptx::map_rank(ptx::smem_u32(&hd->tempty[0]), 0) : 0u;
-        WmTile t;
-        for (int i = 0; wm_item(hd->tprefix, offsets, E, n_units, unit0, ustride, i, C::kGran, t);
-             ++i) {
-            if (t.cnt == 0) continue;
+        if (MODE == kWmProj) ptx::grid_dependency_wait();  // (y's last readers)
+        while (items.next(t, kb0, kb1, part)) {
             const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
             ++tl;
             if (!dead && !ptx::mbar_wait_hint(&hd->tfull[acc], aph, err)) dead = true;
@@ -454,6 +522,7 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                 // product and a bound for every store the four warps took 2.4
                 // times as long as those (12,000 slots: 206 us)
                 float *yc = y_out + j0 * Nw + dcol;
+                if (MODE == kWmProj) yc += (size_t)part * S * Nw;
                 const uint32_t row = (uint32_t)Nw;
 #pragma unroll 1
                 for (int c = 0; c < t.n; c += 32, yc += (size_t)32 * row) {
@@ -463,7 +532,7 @@ k_gemm_wm(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUte
                         tmem_ld_wait();
                     }
                     const int left = t.cnt - c;
-                    if (add && d_ok) {
+                    if (MODE == kWmDown && add && d_ok) {
                         float o[32];
 #pragma unroll
                         for (int i = 0; i < 32; ++i) o[i] = i < left ? yc[i * row] : 0.f;
@@ -505,14 +574,14 @@ template <int MODE, int CG>
 cudaError_t launch_wm_cg(const CUtensorMap &a0, const CUtensorMap &a1, const SlotMaps &b,
                          int a_mode, const int32_t *offsets, int E, int S, int Kdim, int Nw,
                          int add, bf16 *h, float *y, int grid, cudaStream_t st,
-                         const char *name) {
+                         const char *name, ProjSplit split = ProjSplit{}) {
     using C = WmCfg<MODE, CG>;
     const void *kern = (const void *)k_gemm_wm<MODE, CG>;
     unsigned *err = device_info().err;
     CUtensorMap m0 = a0, m1 = a1;
     SlotMaps mb = b;
     void *args[] = {&m0, &m1, &mb, &a_mode, &offsets, &E, &S, &Kdim, &Nw, &add, &h,
-                    &y, &err};
+                    &y, &split, &err};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kWmThreads);
@@ -623,6 +692,35 @@ bool weight_pair_map(CUtensorMap *m, const void *w1, const void *v1, uint64_t ro
 }
 
 }  // namespace
+
+bool proj_split(int T, int Kdim, int Nw, ProjSplit *split) {
+    ProjSplit s{0, (Kdim + 63) / 64, (Nw + 255) / 256, (T + 255) / 256};
+    const int u = s.nwt * s.nst;
+    if (T < kProjSplitMinTokens || T > kProjSplitMaxTokens || u > ProjSplit::kMaxUnits ||
+        encode_fn() == nullptr || single_cta_forced())
+        return false;
+    s.pairs = std::min(wm_pairs<kWmProj>(), ProjSplit::kMaxPairs);
+    // not where a unit would be cut in more than two parts, nor where full
+    // rounds of whole units leave less than a quarter idle: there the runs of a
+    // weight tile, in step, share it in L2, and out of step do not (attention
+    // block of DBRX, equal shares against the kernel otherwise taken: 96 units
+    // on 76 pairs, 63% busy: 600 tokens 143 -> 136 us, 768: 161 -> 156; 160, 70%:
+    // 1200: 240 -> 229; 128, 84%: 1000: 197 -> 208; 256, 84%: 2048: 374 -> 404)
+    const int rounds = (u + s.pairs - 1) / std::max(1, s.pairs);
+    if (s.pairs < 1 || u < s.pairs || 4 * u >= 3 * rounds * s.pairs) return false;
+    *split = s;
+    return true;
+}
+
+cudaError_t launch_proj_wm(int T, int Kdim, int Nw, const void *x, const void *w, float *y,
+                           const ProjSplit &split, cudaStream_t st, const char *name) {
+    CUtensorMap a;
+    SlotMaps b;
+    if (!make_map(&a, w, (uint64_t)Nw, (uint64_t)Kdim, 128) || !slot_maps(b, x, T, Kdim, 8))
+        return cudaErrorInvalidValue;
+    return launch_wm_cg<kWmProj, 2>(a, a, b, 0, nullptr, 1, T, Kdim, Nw, 0, nullptr, y,
+                                    2 * split.pairs, st, name, split);
+}
 
 cudaError_t launch_gemm_up_wm(const moe_dims &d, int T, const void *x_sorted,
                               const int32_t *offsets, const void *w1, const void *v1, void *h,

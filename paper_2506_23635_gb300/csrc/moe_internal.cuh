@@ -333,6 +333,34 @@ constexpr int kWmMinTokens = 65;
 inline bool use_wm(const moe_dims &d, int T) {
     return T >= kWmMinTokens && (long long)T * d.top_k >= 128LL * d.n_experts;
 }
+// One weight matrix against many token rows (ffn_tc_wm.cu): y = x . w^T in fp32,
+// its units (256 weight rows x a run of up to 256 tokens) x k-blocks shared out
+// evenly, CTA pair p taking the blocks [W p / P, W (p + 1) / P) of all W, at
+// least a unit each: a unit that two pairs have a piece of comes in two parts,
+// which the caller adds in order: part k of it lies at y + k T Nw.
+struct ProjSplit {
+    static constexpr int kMaxPairs = 80;
+    static constexpr int kMaxUnits = 640;
+    int pairs, nk, nwt, nst;  // k-blocks of a unit, weight tiles, token runs
+    __host__ __device__ int owner(int block) const {
+        return ((block + 1) * pairs - 1) / (nwt * nst * nk);
+    }
+    __host__ __device__ int run_start(int T, int st) const {
+        return (int)((long long)st * T / nst);
+    }
+    // parts of output row n (of Nw) of token t
+    __host__ __device__ int parts(int T, int t, int n) const {
+        const int st = ((t + 1) * nst - 1) / T;  // the run that holds t
+        const int first = ((n >> 8) * nst + st) * nk;
+        return owner(first + nk - 1) - owner(first) + 1;
+    }
+};
+constexpr int kProjSplitMinTokens = 257;
+constexpr int kProjSplitMaxTokens = 2048;
+bool proj_split(int T, int Kdim, int Nw, ProjSplit *split);
+cudaError_t launch_proj_wm(int T, int Kdim, int Nw, const void *x, const void *w, float *y,
+                           const ProjSplit &split, cudaStream_t st, const char *name);
+
 cudaError_t launch_gemm_up_wm(const moe_dims &d, int T, const void *x_sorted,
                               const int32_t *offsets, const void *w1, const void *v1, void *h,
                               cudaStream_t st);

@@ -592,9 +592,11 @@ def test_ragged_tiles_and_listed_tokens(Hq, Hkv, L, runs):
 # (D, Hq, Hkv, tokens): the projections of calls above 128 tokens: one token
 # more, each width of a token run (160, 192, 224 and 256), one token over a run
 # of 256 and over two, the last size of this kernel and the first of the pair
-# GEMM, output widths that end inside a weight tile.
+# GEMM, output widths that end inside a weight tile; last, 84, 96 and 160 units
+# for the pairs (equal shares, units in two parts).
 PROJ = [(768, 3, 1, 129), (328, 12, 4, 180), (512, 2, 1, 211), (1536, 12, 4, 256),
-        (2560, 16, 2, 257), (384, 6, 1, 513), (1024, 6, 1, 640), (1000, 6, 1, 641)]
+        (2560, 16, 2, 257), (384, 6, 1, 513), (1024, 6, 1, 640), (1000, 6, 1, 641),
+        (328, 40, 8, 530), (512, 48, 8, 768), (264, 48, 8, 1100)]
 
 
 @pytest.mark.parametrize("D,Hq,Hkv,T", PROJ, ids=lambda v: str(v))
