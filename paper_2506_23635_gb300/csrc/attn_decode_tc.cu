@@ -175,6 +175,13 @@ constexpr int kDecMaxWhole = 4;
 // tokens of DBRX, 1.7, up to 4096 positions: 102 us in equal shares, 112 with
 // a CTA each)
 constexpr int kDecWholeMin = 2;
+// listed tokens: taken whole unless the longest has more tiles than twice an
+// equal share and this many.  The CTAs start one by one as the prefill
+// attention leaves them SMs, and an equal share that starts late ends late
+// (attention block of DBRX, a chunk of 200 beside decode tokens of 512-2048
+// positions, equal shares and taken whole: 2 tokens 75 and 79 us, 4: 90 and 80,
+// 8: 93 and 81, 16: 100 and 85, 24: 109 and 89)
+constexpr int kDecListedSlack = 12;
 enum : int { kDecFirst = 1, kDecLast = 2, kDecWhole = 4, kDecEnd = 8, kDecQShift = 4 };
 
 struct DecHeader {
@@ -626,8 +633,14 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             if (lane == 31) hd->before[kDecMaxTokens] = run;
             __syncwarp();
             W = (long long)hd->before[kDecMaxTokens] * Hkv;
-            whole_only = T * Hkv >= kDecWholeMin * (int)gridDim.x ||
-                         (LISTED && n_listed > kDecMaxTokens);
+            if (LISTED) {
+                const int longest = __reduce_max_sync(
+                    0xffffffffu, max(max(nt[0], nt[1]), max(nt[2], nt[3])));
+                whole_only = n_listed > kDecMaxTokens ||
+                             longest <= 2 * W / (int)gridDim.x + kDecListedSlack;
+            } else {
+                whole_only = T * Hkv >= kDecWholeMin * (int)gridDim.x;
+            }
             n_share = whole_only ? T * Hkv
                                  : (int)min((long long)gridDim.x,
                                             max(1LL, W < (1 << 24)

@@ -545,7 +545,8 @@ def test_decode_shares_of_tiles(Hq, Hkv, n_dec, chunk, L):
 # shorter ones are listed: runs one short of a tile, a tile, one over and one
 # short of 16 over it; the smallest tile; two runs of one sequence; a call of
 # 60 tokens; 300 listed tokens (three batches of them) around a tile; an odd
-# group of query heads; a sequence past 256 key/value tiles beside short ones.
+# group of query heads; a sequence past 256 key/value tiles beside short ones;
+# few listed tokens far on (equal shares).
 RAGGED = [
     (6, 1, 700, [(0, 37, 127), (-1, 0, 5), (1, 0, 129), (2, 130, 128), (3, 1, 143), (4, 600, 16),
                  (5, 600, 15), (1, 129, 77)]),
@@ -553,6 +554,7 @@ RAGGED = [
     (4, 2, 200, [(-1, 0, 170), (0, 20, 33), (-1, 0, 130)]),
     (3, 1, 400, [(0, 0, 300), (1, 3, 200), (-1, 0, 3)]),
     (2, 1, 33100, [(0, 33000, 90), (1, 5, 20), (2, 128, 64), (-1, 0, 4)]),
+    (6, 1, 2600, [(0, 2500, 3), (1, 100, 60), (2, 2590, 1)]),
 ]
 
 
