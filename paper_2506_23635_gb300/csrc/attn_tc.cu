@@ -9,10 +9,11 @@
 // heads share every key and value tile and every causal mask, so one copy
 // stream feeds two independent softmax chains that take turns on the tensor
 // cores (a group with an odd number of query heads leaves its last head alone
-// in a unit).  One CTA per SM takes units from a counter, the longest first.
-// A tile's missing rows cost what full ones cost: their queries are whatever
-// follows in memory, each row of the tensor core's output depends on its own
-// query only, and nothing of them is stored.
+// in a unit, and few tiles give every head a unit of its own).  One CTA per SM
+// takes units from a counter, the longest first.  A tile's missing rows cost
+// what full ones cost: their queries are whatever follows in memory, each row
+// of the tensor core's output depends on its own query only, and nothing of
+// them is stored.
 //
 //   warp 0      TMA: both heads' bf16 query tiles once, then the key and
 //               the value tiles of positions [128j, 128j+128) into
@@ -206,7 +207,15 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // the kernel for the tokens that no tile holds may take the SMs that this
     // one leaves free
     ptx::launch_dependents();
-    const int n_units = __ldcg(&plan.head->n_tiles) * Hkv * pairs;
+    // two heads a unit; one where even so every SM has little more than a unit
+    // and nothing else runs on the SMs that stay free: the longest unit is then
+    // shorter (attention block of DBRX, 300 tokens at 512: 104.8 -> 101.8 us,
+    // 512 at 0: 122.5 -> 120.8; beside 24 decode tokens 89 -> 95, 700 tokens
+    // 150 -> 155, which so keep two)
+    const int n_tiles = __ldcg(&plan.head->n_tiles), n_left = __ldcg(&plan.head->n_left);
+    const bool single = n_left == 0 && 3 * n_tiles * Hq <= 4 * (int)gridDim.x;
+    const int per = single ? G : pairs;  // units of a (tile, key/value head)
+    const int n_units = n_tiles * Hkv * per;
     int unit = (int)blockIdx.x;
     if (unit >= n_units) return;
     if (threadIdx.x == 0) {
@@ -231,10 +240,10 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = hd->tmem_base;
-    const int tile = unit / (Hkv * pairs), gp = unit - tile * Hkv * pairs;
-    const int g = gp / pairs, hp = gp - g * pairs;
-    const int h0 = g * G + 2 * hp;                // the unit's first query head
-    const int nh = 2 * hp + 1 < G ? 2 : 1;        // and how many it holds
+    const int tile = unit / (Hkv * per), gp = unit - tile * Hkv * per;
+    const int g = gp / per, hp = gp - g * per;
+    const int h0 = g * G + (single ? hp : 2 * hp);         // the unit's first query head
+    const int nh = !single && 2 * hp + 1 < G ? 2 : 1;      // and how many it holds
     const int4 td = __ldcg(&plan.tiles[tile]);
     const int t0 = td.x, rows = td.y, p0 = td.z, sq = td.w;
     const int n_kv = (p0 + rows - 1) / kFa + 1;   // key/value tiles 0 .. n_kv-1
@@ -486,8 +495,7 @@ cudaError_t launch_attn_prefill_tc(int T, int Hq, int Hkv, int n_seq, int L, con
     AttnPlan pl = plan;
     void *args[] = {&mq, &mk, &mv, &Hq, &Hkv, &L, &pl, &cp, &err};
     // one CTA per SM, or per unit of the most tiles that T tokens can make
-    const int pairs = (Hq / Hkv + 1) / 2;
-    const long long most = (long long)Hkv * pairs * (T / kAttnTileMinRows);
+    const long long most = (long long)Hq * (T / kAttnTileMinRows);
     LaunchScope ls("attention_tc", st);
     return launch_pdl(kern,
                       dim3((unsigned)std::max(1LL, std::min<long long>(most, device_info().sm_count))),

@@ -13,11 +13,11 @@
 //   accumulators in turn (the tensor core truncates when it adds to an
 //   accumulator: chains of 3 roundings instead of 48 at d_model 6144; relative
 //   error of the logits against 64 bits 0.80e-7, with four accumulators
-//   1.84e-7, k_route 0.87e-7).  Four warps read their 32 tokens' rows from tensor memory
-//   and store the share's partial logits into the shared memory of the CTA
-//   that finishes the token, 16 tokens each: a warp per token adds the shares
-//   in order and runs select_topk (ties to the lower index, NaN ranked as
-//   -inf; one thread per token was slower).
+//   1.84e-7, k_route 0.87e-7).  Four warps read their 32 tokens' rows from
+//   tensor memory and store the share's partial logits into the shared memory
+//   of the CTA that finishes the token, 16 tokens each: half a warp per token
+//   adds the shares (in 64 bits) and selects the top-k (ties to the lower
+//   index, NaN ranked as -inf).
 // Bound by latency (one kernel after the other, event pairs): 128-600 tokens
 // 16 us, 2048 tokens 24 us with x in HBM (17.5 + 10.7 us as two kernels, the
 // second for the top-k), 3000 tokens 18-23 us (k_route, which re-reads W_r from
