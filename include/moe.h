@@ -36,6 +36,10 @@
  *     the same time on the GPU need workspaces of their own.
  *   - Calls are asynchronous on `stream` and never synchronise with the host
  *     (except moe_get_last_error and moe_profile_read).
+ *   - Inputs, weights included, are read in stream order: once everything
+ *     ahead of the call on `stream` has completed, also where that ends in a
+ *     kernel that lets the next launch start before it ends (programmatic
+ *     stream serialisation).
  *   - Arguments are validated before anything is launched; on a validation
  *     error nothing is written and the status says why.
  *   - T == 0 is valid and launches nothing (moe_dispatch still writes zero

@@ -248,12 +248,12 @@ k_route_dispatch_small(int T, int D, int E, int K, const TX *__restrict__ x,
             ptx::fence_barrier_init();
         }
         __syncthreads();
-        // W_r does not come from the previous kernel: its copy starts before
-        // the dependency wait, and the next kernel may launch at once (its
-        // CTAs take the other SMs and wait for this one on the device)
-        stage_router_issue<TW>(wsm, wr, (uint32_t)((size_t)D * E * sizeof(TW)), &bar);
+        // the next kernel may launch at once (its CTAs take the other SMs and
+        // wait for this one on the device); x and W_r may come from the
+        // previous one
         ptx::launch_dependents();
-        ptx::grid_dependency_wait();  // x may come from the previous kernel
+        ptx::grid_dependency_wait();
+        stage_router_issue<TW>(wsm, wr, (uint32_t)((size_t)D * E * sizeof(TW)), &bar);
         const bool ok = ptx::mbar_wait(&bar, 0, err);
         // a wait that gave up (recorded in err) ends the whole block, never part of it
         if (!__syncthreads_and(ok)) return;
@@ -312,8 +312,7 @@ k_route_dispatch_small(int T, int D, int E, int K, const TX *__restrict__ x,
 
 // ---------------------------------------------------------------------------
 // Route and dispatch of a decode batch (T <= 64, T*K <= 256) in one launch of
-// a cluster of kClusterCtas CTAs.  CTA r bulk-copies rows [d0_r, d1_r) of W_r
-// (before waiting for the previous kernel: the router is a weight) and the
+// a cluster of kClusterCtas CTAs.  CTA r bulk-copies rows [d0_r, d1_r) of W_r and the
 // same columns of every token row of x into its shared memory, and computes
 // the partial logits of every token over that slice of d.  After a cluster
 // barrier, token t is finished by one warp of CTA t mod kClusterCtas: it adds
@@ -381,6 +380,7 @@ k_route_dispatch_cluster(int T, int D, int E, int K, const TX *__restrict__ x,
         ptx::fence_barrier_init();
     }
     __syncthreads();
+    ptx::grid_dependency_wait();  // x and W_r may come from the previous kernel
     if (tid == 0 && dn > 0) {
         const uint32_t bytes = (uint32_t)((size_t)dn * E * sizeof(TW));
         const uint64_t pol = ptx::policy_evict_last();
@@ -391,7 +391,6 @@ k_route_dispatch_cluster(int T, int D, int E, int K, const TX *__restrict__ x,
                           reinterpret_cast<const unsigned char *>(wr + (size_t)d0 * E) + o,
                           min(kChunk, bytes - o), &bar[0], pol);
     }
-    ptx::grid_dependency_wait();  // x may come from the previous kernel
     if (warp == 0 && dn > 0) {
         // one bulk copy per token row: dn elements from column d0 (16-byte
         // aligned because D and d0 are multiples of 8)

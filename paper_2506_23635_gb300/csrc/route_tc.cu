@@ -6,8 +6,7 @@
 // k_route_tc: the 8 CTAs of a cluster take the 128 tokens of a tile, CTA r the
 //   r-th of 8 equal shares of the 64-column blocks of d.  Its slice of W_r is
 //   written by the threads, transposed, into shared memory in the 128-byte
-//   swizzled K-major layout (16 expert rows per 64-column panel) -- before
-//   the dependency wait, as W_r comes from no earlier kernel; the token rows
+//   swizzled K-major layout (16 expert rows per 64-column panel); the token rows
 //   arrive by TMA, all of a share in flight where the SM has room; one lane
 //   issues tcgen05.mma (M = 128 tokens, N = 16 experts, K = 16) into 16
 //   accumulators in turn (the tensor core truncates when it adds to an
@@ -140,8 +139,9 @@ k_route_tc(const __grid_constant__ CUtensorMap tmX, int T, int D, int E, int K, 
         }
         ptx::mbar_init(&hd->done, 1);
         ptx::fence_barrier_init();
-        // the token rows may come from the previous kernel; the first stages
-        // of them are on the way while W_r is laid out
+        // the token rows may come from the previous kernel (so may W_r, whose
+        // layout below waits too); the first stages of them are on the way
+        // while W_r is laid out
         ptx::grid_dependency_wait();
         const uint64_t pol = ptx::policy_evict_normal();
         for (int i = 0; i < min(n_stage, nkb); ++i) {
@@ -152,6 +152,7 @@ k_route_tc(const __grid_constant__ CUtensorMap tmX, int T, int D, int E, int K, 
     }
     __syncwarp();
     if (warp == 1) tmem_alloc(&hd->tmem, kRtTmemCols);
+    ptx::grid_dependency_wait();
     // W_r^T slice: panel i holds d = (kb0 + i) * 64 + c, c < 64; row e of the
     // panel is expert e (zero past E or past D)
     const bool vec = E == 16;  // a router row is 32 B: two 16-byte loads
@@ -188,7 +189,6 @@ k_route_tc(const __grid_constant__ CUtensorMap tmX, int T, int D, int E, int K, 
     const uint32_t tmem = hd->tmem;
     // every CTA of the cluster has started before the others store to it
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    ptx::grid_dependency_wait();
 
     if (warp == 0) {
         if (lane == 0) {
