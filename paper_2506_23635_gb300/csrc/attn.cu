@@ -12,8 +12,8 @@
 //   k_sa_prenorm   RMSNorm0 of the fp32 residual -> bf16 rows; block 0 also
 //                  writes the trivial dispatch of a one-"expert" projection
 //                  (offsets {0, T}), for the grouped GEMM of prefill batches;
-//                  it lets the projection launch at once (the projection's
-//                  weight loads do not depend on it);
+//                  it lets the projection launch once its own wait is over (the
+//                  projection's weight loads do not depend on it);
 //   projection     W_qkv . x: the tcgen05 kernel with the weights as the M
 //                  operand (split reduction) for up to 640 tokens, the grouped
 //                  tcgen05 GEMM with E = 1 beyond (fp32 out);
@@ -216,10 +216,11 @@ template <int NT, int VEC>
 __global__ void __launch_bounds__(NT)
 k_sa_prenorm(int T, int D, const float *__restrict__ resid, bf16 *__restrict__ xn, float eps,
              int32_t *offsets, const PlanArgs pa) {
-    // the projection after this kernel may start now: its weight loads do
-    // not depend on anything here
-    ptx::launch_dependents();
     ptx::grid_dependency_wait();
+    // the projection after this kernel may start now: its weight loads do not
+    // depend on anything here, and what is ahead of the call, which may have
+    // written the weights, is complete (so only after the wait)
+    ptx::launch_dependents();
     __shared__ float red[NT / 32];
     int t = blockIdx.x;
     if (pa.plan.head) {  // block 0 makes the attention's plan

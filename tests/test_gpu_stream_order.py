@@ -81,3 +81,44 @@ def test_layer_router_weight_written_just_ahead(T):
     w2 = (torch.randn(E, D, F, generator=g) * 0.02).bfloat16().cuda()
     ws, out = m.alloc_workspace(d, T), torch.empty(T, D, dtype=torch.bfloat16, device="cuda")
     _check(m, wr, lambda: [m.layer_forward(d, x, wr.weight(D, E), w1, v1, w2, out=out, ws=ws)])
+
+
+@pytest.mark.parametrize("D,Hq,Hkv,T", [(256, 2, 1, 3), (256, 2, 1, 150), (328, 12, 4, 400),
+                                        (328, 40, 8, 530), (256, 2, 1, 700)])
+def test_projection_weight_written_just_ahead(D, Hq, Hkv, T):
+    """The attention block's W_qkv, on each kernel that takes it: the
+    weights-as-M kernel of one run of tokens and of two, the pair GEMM in equal
+    shares of the (unit, k-block)s and in whole units."""
+    m = moe()
+    g = torch.Generator().manual_seed(T)
+    wr = Writer(m, (Hq + 2 * Hkv) * 128 * D)
+    a = m.sa_dims(D, Hq, Hkv, 128, 10000.0)
+    x = torch.randn(T, D, generator=g).cuda()
+    w_o = (torch.randn(D, Hq * 128, generator=g) * 0.02).bfloat16().cuda()
+    seq = torch.zeros(T, dtype=torch.int32, device="cuda")
+    pos = torch.arange(T, dtype=torch.int32, device="cuda")
+    kc = torch.empty(1, Hkv, T, 128, dtype=torch.bfloat16, device="cuda")
+    vc, out = torch.empty_like(kc), torch.empty_like(x)
+    ws = torch.empty(m.sa_workspace_size(a, T), dtype=torch.uint8, device="cuda")
+    w_qkv = wr.weight((Hq + 2 * Hkv) * 128, D)
+
+    def block():
+        m.sa_forward(a, out, w_qkv, w_o, seq, pos, kc, vc, ws=ws)
+        return [out, kc, vc]
+
+    wr.write()
+    torch.cuda.synchronize()
+    out.copy_(x)
+    want = [t.clone() for t in block()]
+    for _ in range(5):
+        wr.vc.zero_()
+        out.copy_(x)
+        torch.cuda.synchronize()
+        wr.write()
+        got = block()
+        torch.cuda.synchronize()
+        # (the caches hold the projection itself; the block's sums over
+        # positions may take their parts in another order)
+        assert torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+        assert float((got[0] - want[0]).norm()) <= 1e-2 * float((want[0] - x).norm())
+    assert m.get_last_error() == 0
