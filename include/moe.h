@@ -338,7 +338,10 @@ int32_t moe_profile_read(moe_kernel_stat *stats, int32_t max_stats);
  *     RMSNorm0 as in moe_prenorm (no learned scale).
  * Storage: the normalised input, the rotated queries (as the attention
  * reads them), the cached keys and values and the attention output ctx are
- * bf16; projections accumulate in fp32; the residual stream is fp32.
+ * bf16; projections accumulate in fp32; the residual stream is fp32.  Scores
+ * and sums are fp32; probabilities enter the product with V in two bf16 terms
+ * (16 bits of each; on the CUDA cores they are fp32), but in one in a prefill
+ * tile of 128 tokens that starts at a multiple of 128 of the call's tokens.
  *
  * Layouts (row-major): w_qkv [(Hq + 2 Hkv) dh, D] bf16 -- the query rows,
  * then the key rows, then the value rows; w_o [D, Hq dh] bf16; k_cache and

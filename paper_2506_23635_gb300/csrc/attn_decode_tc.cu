@@ -7,9 +7,12 @@
 //
 //   S^T = K_j Q^T       M = 128 positions, N = 16 (the G heads, zero-
 //                       padded), K = 128 dims; K_j and Q both K-major
-//   O^T += V_j^T P_j^T  M = 128 dims, N = 16 heads, K = 128 positions; V_j
+//   O^T += V_j^T P_j^T  M = 128 dims, N = 16, K = 128 positions; V_j
 //                       as it lies in the cache (dims contiguous: an
-//                       MN-major A operand), P_j K-major in shared memory
+//                       MN-major A operand), P_j K-major in shared memory:
+//                       rows h the heads' probabilities rounded to bf16, rows
+//                       8 + h the rounded rests, whose columns of O^T are
+//                       added at the end of a piece
 //
 // with S^T and O^T in tensor memory (lane = position, resp. dim; column =
 // head).  Schedules (template parameter MODE):
@@ -60,8 +63,8 @@
 //               shared memory), the base-2 exponent of the 1/sqrt(128)-
 //               scaled scores against a per-head base that moves only when
 //               the maximum passes it by more than 8 (then O^T is rescaled
-//               in tensor memory, each thread its dim's row), bf16
-//               probabilities written into P_j (rows = heads, positions
+//               in tensor memory, each thread its dim's row), both terms
+//               of the probabilities written into P_j (positions
 //               contiguous, 128-byte swizzle), rows of V_j past the
 //               sequence's last position zeroed (0 * NaN is NaN; those cache
 //               rows may hold anything).
@@ -87,9 +90,10 @@
 // the call's own positions do not depend on it and are loaded at once (0.5-1.5
 // us of the attention block at 1-11 sequences).
 //
-// Numerics as the prefill flash attention: bf16 queries and probabilities,
-// fp32 scores and accumulation; the row sum takes the probabilities as
-// stored.  Every wait is bounded (ptx.cuh); once one gives up the thread
+// Numerics: bf16 queries, fp32 scores and accumulation, probabilities in two
+// bf16 terms (2^-17 of each at most unaccounted for: the padding rows of N hold
+// the second, so it costs no MMA and no time that could be measured); the row
+// sum takes the probabilities as stored.  Every wait is bounded (ptx.cuh); once one gives up the thread
 // skips the later waits and the kernel ends.
 #include <math.h>
 
@@ -894,15 +898,12 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     } else {
         // ------------------------------------------------------------ softmax
         {
-            // probability rows G..15 of both buffers stay zero (the MMA's
-            // padding heads; no thread writes them later, and each thread's
-            // proxy fence before it releases P_0 covers its zeros)
-            constexpr int kPadRow = G * 8;  // 16-byte chunks before row G of a half
-            constexpr int kPad = 16 * 8 - kPadRow;
-            for (int i = threadIdx.x - 64; i < 4 * kPad; i += 128) {
-                uint4 *half = reinterpret_cast<uint4 *>(smem + kDecOffP) + (i / kPad) * (kDecNHalf / 16);
-                half[kPadRow + i % kPad] = make_uint4(0u, 0u, 0u, 0u);
-            }
+            // probability rows G..7 and 8 + G..15 of both buffers stay zero
+            // (the MMA's padding heads; no thread writes them later, and each
+            // thread's proxy fence before it releases P_0 covers its zeros)
+            for (int i = threadIdx.x - 64; i < 2 * (int)(kDecP / 16); i += 128)
+                if ((i / 8) % 8 >= G)  // (16-byte chunk i, eight to a row)
+                    reinterpret_cast<uint4 *>(smem + kDecOffP)[i] = make_uint4(0u, 0u, 0u, 0u);
         }
         const int qd = warp & 3;       // tensor-memory lane quarter
         const int r = qd * 32 + lane;  // position of the tile; dim of O^T
@@ -988,11 +989,14 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll
             for (int h = 0; h < G; ++h) {
                 const float pv = valid ? dec_exp2(x[h] - base[h]) : 0.f;
-                const bf16 pq = __float2bfloat16_rn(pv);
-                if (good)
-                    *reinterpret_cast<bf16 *>(pb + swizzle_offset((uint32_t)h,
-                                                                  (uint32_t)(r & 63))) = pq;
-                l[h] = fmaf(l[h], corr[h], __bfloat162float(pq));
+                const bf16 p1 = __float2bfloat16_rn(pv);
+                const bf16 p2 = __float2bfloat16_rn(pv - __bfloat162float(p1));
+                if (good) {
+                    unsigned char *row = pb + swizzle_offset((uint32_t)h, (uint32_t)(r & 63));
+                    *reinterpret_cast<bf16 *>(row) = p1;
+                    *reinterpret_cast<bf16 *>(row + 8 * 128) = p2;  // (rows 8 apart swizzle alike)
+                }
+                l[h] = fmaf(l[h], corr[h], __bfloat162float(p1) + __bfloat162float(p2));
             }
             // a value tile that runs past the sequence's last position: its
             // rows there are zeroed before P_j V_j reads them
@@ -1019,7 +1023,10 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     tmem_ld16(tmem + lane_base + kDecColO, so);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int h = 0; h < G; ++h) so[h] *= corr[h];
+                    for (int h = 0; h < G; ++h) {
+                        so[h] *= corr[h];
+                        so[8 + h] *= corr[h];
+                    }
                     tmem_st16(tmem + lane_base + kDecColO, so);
                 }
             }
@@ -1045,6 +1052,8 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 tmem_ld16(tmem + lane_base + kDecColO, o);
                 tmem_ld_wait();
                 tc_fence_before();
+#pragma unroll
+                for (int h = 0; h < G; ++h) o[h] += o[8 + h];
             }
 #pragma unroll
             for (int h = 0; h < G; ++h)

@@ -40,6 +40,19 @@
 //               may hold anything, and 0 * NaN is NaN) before its P_j is
 //               announced, which comes before either head's P_j V_j.
 //
+// Probabilities: a tile of 128 rows that starts at a multiple of 128 of the
+// call's tokens takes them in bf16.  Any other tile holds tokens whose
+// probabilities the CUDA-core kernel would keep in fp32: here they are two bf16
+// terms (the rounded value and the rounded rest, which leave 2^-17 of it at most),
+// for every 32 positions 16 columns of the first and 16 of the second over
+// the scores, and P V is two products.  Error of the attention block against 64
+// bits, on the CUDA cores, in one term, in two: chunks of 300 and 205 beside
+// 24 decode tokens 5.12e-3, 5.18e-3, 5.06e-3 (full tiles there are in two terms
+// too); 200 decode tokens (attn_decode_tc.cu) 4.43e-3, 4.55e-3, 4.43e-3.  The
+// second term costs: this kernel at 1000 tokens 32 -> 39 us (170 us for the last
+// 104 of them on the CUDA cores), 104 tokens at position 896 26.6 -> 31.0, 2048
+// tokens (none in two terms) 81.8 -> 83.9.
+//
 // At 2048 tokens (48 query heads): 94-100 us, against 108-113 us for one head
 // per CTA with eight softmax warps (two threads per row and a row-max
 // exchange).  By clock stamps a key/value tile takes ~5250 cycles for the two
@@ -157,17 +170,24 @@ __device__ __forceinline__ void issue_qk(uint32_t d_tmem, uint32_t q_smem, uint3
 // O (+)= P V: P [128 queries, 128 positions] in tensor memory (row r in lane
 // r, two positions per 32-bit column), V [128 positions, 128 dims] as stored
 // (MN-major); K = 16 positions (8 columns of P) per instruction.  The first
-// key/value tile overwrites O, the later ones add to it.
+// key/value tile overwrites O, the later ones add to it.  One term of P: the
+// first 64 columns.  TWO: of every 32 columns 16 hold the first term of 32
+// positions and 16 the second.
+template <bool TWO>
 __device__ __forceinline__ void issue_pv(uint32_t d_tmem, uint32_t p_tmem, uint32_t v_smem,
                                          bool accumulate) {
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
         const uint64_t bd = smem_desc_mn(v_smem + ks * 16 * 128);
-        const uint32_t acc = (accumulate || ks != 0) ? 1u : 0u;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "r"(p_tmem + ks * 8), "l"(bd), "r"(kFaIdescVmn), "r"(acc));
+#pragma unroll
+        for (int term = 0; term < (TWO ? 2 : 1); ++term) {
+            const uint32_t acc = (accumulate || (ks | term) != 0) ? 1u : 0u;
+            const uint32_t col = TWO ? (ks >> 1) * 32 + term * 16 + (ks & 1) * 8 : ks * 8;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+                "r"(p_tmem + col), "l"(bd), "r"(kFaIdescVmn), "r"(acc));
+        }
     }
 }
 
@@ -187,6 +207,254 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32
 
 __device__ __forceinline__ void tmem_st_wait() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// The MMA issuer's part of a unit: nh heads over n_kv key/value tiles.  TWO:
+// probabilities in two terms.  False: a wait gave up.
+template <bool TWO>
+__device__ __forceinline__ bool fa_issue(FaHeader *hd, uint32_t sbase, uint32_t tmem, int n_kv,
+                                         int nh, unsigned *err) {
+    bool good = fa_wait(&hd->q_full, 0, err) && fa_wait(&hd->kv_full[0], 0, err);
+    if (good) {
+        tc_fence_after();
+        for (int x = 0; x < nh; ++x) {
+            issue_qk(tmem + kColS + x * kFa, sbase + kOffQ + x * kTileBytes, sbase + kOffK);
+            mma_commit(&hd->s_full[x]);
+        }
+        mma_commit(&hd->kv_empty[0]);  // key tile 0 read once these finish
+    }
+    for (int j = 0; j < n_kv && good; ++j) {
+        const int b = j & 1;
+        if (!(good = fa_wait(&hd->v_full[b], (j >> 1) & 1, err))) break;
+        for (int x = 0; x < nh && good; ++x) {
+            // O += P_j V_j once the head's softmax warps have written P_j
+            if (!(good = fa_wait(&hd->p_ready[x], j & 1, err))) break;
+            tc_fence_after();
+            issue_pv<TWO>(tmem + kColO + x * kFa, tmem + kColS + x * kFa,
+                          sbase + kOffV + b * kTileBytes, j != 0);
+            mma_commit(&hd->o_full[x]);
+            if (x == nh - 1) mma_commit(&hd->v_empty[b]);  // value tile j read by both
+            if (j + 1 < n_kv) {
+                // S_{j+1} replaces P_j: only after P_j V_j has finished
+                const int b1 = (j + 1) & 1;
+                if (!(good = fa_wait(&hd->o_full[x], j & 1, err))) break;
+                // (head B follows head A, which has waited for key tile j+1)
+                if (x == 0 && !(good = fa_wait(&hd->kv_full[b1], ((j + 1) >> 1) & 1, err)))
+                    break;
+                tc_fence_after();
+                issue_qk(tmem + kColS + x * kFa, sbase + kOffQ + x * kTileBytes,
+                         sbase + kOffK + b1 * kTileBytes);
+                mma_commit(&hd->s_full[x]);
+                if (x == nh - 1) mma_commit(&hd->kv_empty[b1]);
+            }
+        }
+    }
+    return good;
+}
+
+// One row's softmax over a unit's key/value tiles: thread r of head x's four
+// warps; l: the row sum relative to the exponent base it ends with.
+__device__ __forceinline__ bool fa_softmax(FaHeader *hd, unsigned char *smem, uint32_t s_col,
+                                           uint32_t o_col, int n_kv, int p0, int rows, int r, int x,
+                                           float &l, unsigned *err) {
+    const int lane = threadIdx.x & 31;
+    const int qpos = p0 + r;
+    const int last = p0 + rows - 1;              // the tile's last query position
+    const float sl2 = 1.4426950408889634f / sqrtf((float)kHeadDimFa);
+    // m: the exponent base of the row (scaled scores), which may trail the
+    // row maximum by up to kFaRescale; l: the row sum relative to it
+    float m = -INFINITY;
+    l = 0.f;
+    bool good = true;
+    for (int j = 0; j < n_kv; ++j) {
+        const int b = j & 1;
+        // a value tile that runs past the tile's last query: head A's
+        // thread r zeroes its row r past `last` before P_j V_j reads it
+        // (P is zero there, but those cache rows may hold anything)
+        const bool clip = j * kFa + kFa - 1 > last;
+        if (x == 0 && clip) {
+            good = good && fa_wait(&hd->v_full[b], (j >> 1) & 1, err);
+            if (j * kFa + r > last) {
+                unsigned char *vt = smem + kOffV + b * kTileBytes;
+#pragma unroll
+                for (int c = 0; c < kFa; c += 8)
+                    *reinterpret_cast<uint4 *>(vt + (c >> 6) * kHalfBytes +
+                                               swizzle_offset((uint32_t)r, (uint32_t)(c & 63))) =
+                        make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+        // the row's 128 scores of S_j
+        good = good && fa_wait(&hd->s_full[x], j & 1, err);
+        tc_fence_after();
+        float v[kFa];
+#pragma unroll
+        for (int c = 0; c < kFa; c += 32)
+            tmem_ld32(s_col + c, *reinterpret_cast<float(*)[32]>(&v[c]));
+        tmem_ld_wait();
+        const bool full = j * kFa + kFa - 1 <= p0;  // no position of the tile is masked
+        float hm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        if (full) {
+#pragma unroll
+            for (int i = 0; i < kFa; ++i) hm4[i & 3] = fmaxf(hm4[i & 3], v[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kFa; ++i)
+                if (j * kFa + i <= qpos) hm4[i & 3] = fmaxf(hm4[i & 3], v[i]);
+        }
+        // finite: position 128j <= qpos for every row of the tile
+        const float mrow = fmaxf(fmaxf(hm4[0], hm4[1]), fmaxf(hm4[2], hm4[3])) * sl2;
+        const bool bump = mrow > m + kFaRescale;
+        const float corr = bump ? exp2f(m - mrow) : 1.f;  // 0 on the first tile
+        if (bump) m = mrow;
+        // P_j in bf16 pairs over the first 64 columns of S_j, 64 positions
+        // at a time; the row sum takes the probabilities as stored, so the
+        // weights P V is normalised by sum to exactly one
+        const float2 sl2x2 = make_float2(sl2, sl2), nm2 = make_float2(-m, -m);
+        float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            uint32_t pw[32];
+#pragma unroll
+            for (int i = 0; i < 64; i += 2) {
+                const int c = half * 64 + i;
+                const float2 e = __ffma2_rn(make_float2(v[c], v[c + 1]), sl2x2, nm2);
+                float pa = fast_exp2(e.x);
+                float pb = fast_exp2(e.y);
+                if (!full) {
+                    if (j * kFa + c > qpos) pa = 0.f;
+                    if (j * kFa + c + 1 > qpos) pb = 0.f;
+                }
+                const __nv_bfloat162 p2 = __floats2bfloat162_rn(pa, pb);
+                sum2[(i >> 1) & 1] = __fadd2_rn(sum2[(i >> 1) & 1], __bfloat1622float2(p2));
+                pw[i >> 1] = *reinterpret_cast<const uint32_t *>(&p2);
+            }
+            tmem_st32(s_col + half * 32, pw);
+        }
+        // a new base rescales O (the scores are consumed by now): P_{j-1}
+        // V_{j-1} finished before S_j was issued, and P_j V_j waits for
+        // this warp's arrival; the whole warp loads and stores (rows
+        // without a new base scale by 1)
+        if (j >= 1 && __any_sync(0xffffffffu, bump) && __all_sync(0xffffffffu, good)) {
+#pragma unroll 1
+            for (int c = 0; c < kFa; c += 32) {
+                float ov[32];
+                uint32_t ow[32];
+                tmem_ld32(o_col + c, ov);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) ow[i] = __float_as_uint(ov[i] * corr);
+                tmem_st32(o_col + c, ow);
+            }
+        }
+        tmem_st_wait();
+        if (x == 0 && clip) fence_proxy_async_smem();  // the zeroed value rows
+        tc_fence_before();                             // P_j and a rescaled O
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&hd->p_ready[x]);
+        l = l * corr + ((sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y));
+    }
+    return good;
+}
+
+// The same with the probabilities in two terms, in loops of 32 positions: the
+// code is fetched for few units of a call, and unrolled over all 128 it took
+// 5 us longer where the kernels ahead had taken its lines (attention block,
+// 1000 tokens, 210 instead of 205 us; as a function of its own 208).
+__device__ __forceinline__ bool fa_softmax_two(FaHeader *hd, unsigned char *smem, uint32_t s_col,
+                                            uint32_t o_col, int n_kv, int p0, int rows, int r, int x,
+                                            float &l, unsigned *err) {
+    const int lane = threadIdx.x & 31;
+    const int qpos = p0 + r;
+    const int last = p0 + rows - 1;              // the tile's last query position
+    const float sl2 = 1.4426950408889634f / sqrtf((float)kHeadDimFa);
+    // m: the exponent base of the row (scaled scores), which may trail the
+    // row maximum by up to kFaRescale; l: the row sum relative to it
+    float m = -INFINITY;
+    l = 0.f;
+    bool good = true;
+    for (int j = 0; j < n_kv; ++j) {
+        const int b = j & 1;
+        // a value tile that runs past the tile's last query: head A's
+        // thread r zeroes its row r past `last` before P_j V_j reads it
+        // (P is zero there, but those cache rows may hold anything)
+        const bool clip = j * kFa + kFa - 1 > last;
+        if (x == 0 && clip) {
+            good = good && fa_wait(&hd->v_full[b], (j >> 1) & 1, err);
+            if (j * kFa + r > last) {
+                unsigned char *vt = smem + kOffV + b * kTileBytes;
+#pragma unroll
+                for (int c = 0; c < kFa; c += 8)
+                    *reinterpret_cast<uint4 *>(vt + (c >> 6) * kHalfBytes +
+                                               swizzle_offset((uint32_t)r, (uint32_t)(c & 63))) =
+                        make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+        // the row's scores of S_j are read twice: for their maximum, and for
+        // their probabilities, which take the place of the 32 they come from
+        good = good && fa_wait(&hd->s_full[x], j & 1, err);
+        tc_fence_after();
+        const int lim = qpos - j * kFa;  // the row's last position in the tile
+        float hm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+        for (int c0 = 0; c0 < kFa; c0 += 32) {
+            float v[32];
+            tmem_ld32(s_col + c0, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                hm4[i & 3] = fmaxf(hm4[i & 3], c0 + i <= lim ? v[i] : -INFINITY);
+        }
+        const float mrow = fmaxf(fmaxf(hm4[0], hm4[1]), fmaxf(hm4[2], hm4[3])) * sl2;
+        const bool bump = mrow > m + kFaRescale;
+        const float corr = bump ? exp2f(m - mrow) : 1.f;
+        if (bump) m = mrow;
+        const float2 sl2x2 = make_float2(sl2, sl2), nm2 = make_float2(-m, -m);
+        float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 1
+        for (int c0 = 0; c0 < kFa; c0 += 32) {
+            float v[32];
+            uint32_t w[32];  // first terms of 32 positions, second terms
+            tmem_ld32(s_col + c0, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) {
+                const float2 e = __ffma2_rn(make_float2(v[i], v[i + 1]), sl2x2, nm2);
+                const float2 p = make_float2(c0 + i <= lim ? fast_exp2(e.x) : 0.f,
+                                             c0 + i + 1 <= lim ? fast_exp2(e.y) : 0.f);
+                // (the row sum takes p itself: 2^-17 from what is stored)
+                sum2[(i >> 1) & 1] = __fadd2_rn(sum2[(i >> 1) & 1], p);
+                const __nv_bfloat162 p1 = __floats2bfloat162_rn(p.x, p.y);
+                const float2 rest = __ffma2_rn(__bfloat1622float2(p1), make_float2(-1.f, -1.f), p);
+                const __nv_bfloat162 p2 = __floats2bfloat162_rn(rest.x, rest.y);
+                w[i >> 1] = *reinterpret_cast<const uint32_t *>(&p1);
+                w[16 + (i >> 1)] = *reinterpret_cast<const uint32_t *>(&p2);
+            }
+            tmem_st32(s_col + c0, w);
+        }
+        // a new base rescales O (the scores are consumed by now): P_{j-1}
+        // V_{j-1} finished before S_j was issued, and P_j V_j waits for
+        // this warp's arrival; the whole warp loads and stores (rows
+        // without a new base scale by 1)
+        if (j >= 1 && __any_sync(0xffffffffu, bump) && __all_sync(0xffffffffu, good)) {
+#pragma unroll 1
+            for (int c = 0; c < kFa; c += 32) {
+                float ov[32];
+                uint32_t ow[32];
+                tmem_ld32(o_col + c, ov);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) ow[i] = __float_as_uint(ov[i] * corr);
+                tmem_st32(o_col + c, ow);
+            }
+        }
+        tmem_st_wait();
+        if (x == 0 && clip) fence_proxy_async_smem();  // the zeroed value rows
+        tc_fence_before();                             // P_j and a rescaled O
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&hd->p_ready[x]);
+        l = l * corr + ((sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y));
+    }
+    return good;
 }
 
 // 320 threads: three warps share two of the four schedulers' 16K-register
@@ -247,6 +515,7 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const int4 td = __ldcg(&plan.tiles[tile]);
     const int t0 = td.x, rows = td.y, p0 = td.z, sq = td.w;
     const int n_kv = (p0 + rows - 1) / kFa + 1;   // key/value tiles 0 .. n_kv-1
+    const bool two = rows < kFa || t0 % kFa != 0;  // probabilities in two terms (above)
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -297,41 +566,8 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            bool good = fa_wait(&hd->q_full, 0, err) && fa_wait(&hd->kv_full[0], 0, err);
-            if (good) {
-                tc_fence_after();
-                for (int x = 0; x < nh; ++x) {
-                    issue_qk(tmem + kColS + x * kFa, sbase + kOffQ + x * kTileBytes, sbase + kOffK);
-                    mma_commit(&hd->s_full[x]);
-                }
-                mma_commit(&hd->kv_empty[0]);  // key tile 0 read once these finish
-            }
-            for (int j = 0; j < n_kv && good; ++j) {
-                const int b = j & 1;
-                if (!(good = fa_wait(&hd->v_full[b], (j >> 1) & 1, err))) break;
-                for (int x = 0; x < nh && good; ++x) {
-                    // O += P_j V_j once the head's softmax warps have written P_j
-                    if (!(good = fa_wait(&hd->p_ready[x], j & 1, err))) break;
-                    tc_fence_after();
-                    issue_pv(tmem + kColO + x * kFa, tmem + kColS + x * kFa,
-                             sbase + kOffV + b * kTileBytes, j != 0);
-                    mma_commit(&hd->o_full[x]);
-                    if (x == nh - 1) mma_commit(&hd->v_empty[b]);  // value tile j read by both
-                    if (j + 1 < n_kv) {
-                        // S_{j+1} replaces P_j: only after P_j V_j has finished
-                        const int b1 = (j + 1) & 1;
-                        if (!(good = fa_wait(&hd->o_full[x], j & 1, err))) break;
-                        // (head B follows head A, which has waited for key tile j+1)
-                        if (x == 0 && !(good = fa_wait(&hd->kv_full[b1], ((j + 1) >> 1) & 1, err)))
-                            break;
-                        tc_fence_after();
-                        issue_qk(tmem + kColS + x * kFa, sbase + kOffQ + x * kTileBytes,
-                                 sbase + kOffK + b1 * kTileBytes);
-                        mma_commit(&hd->s_full[x]);
-                        if (x == nh - 1) mma_commit(&hd->kv_empty[b1]);
-                    }
-                }
-            }
+            bool good = two ? fa_issue<true>(hd, sbase, tmem, n_kv, nh, err)
+                            : fa_issue<false>(hd, sbase, tmem, n_kv, nh, err);
             mma_commit(&hd->done);
             good &= fa_wait(&hd->done, 0, err);
             if (!good) hd->gave_up = 1;
@@ -342,103 +578,12 @@ k_attn_prefill_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const int x = (warp - 2) / kFaWarpsPerHead;  // head h0 + x of the CTA
         const int q = warp & 3;                      // tensor-memory lane quarter
         const int r = q * 32 + lane;                 // query row of the tile
-        const int qpos = p0 + r;
-        const int last = p0 + rows - 1;              // the tile's last query position
-        const float sl2 = 1.4426950408889634f / sqrtf((float)kHeadDimFa);
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         const uint32_t s_col = tmem + lane_base + kColS + (uint32_t)x * kFa;
         const uint32_t o_col = tmem + lane_base + kColO + (uint32_t)x * kFa;
-        // m: the exponent base of the row (scaled scores), which may trail the
-        // row maximum by up to kFaRescale; l: the row sum relative to it
-        float m = -INFINITY, l = 0.f;
-        bool good = true;
-        for (int j = 0; j < n_kv; ++j) {
-            const int b = j & 1;
-            // a value tile that runs past the tile's last query: head A's
-            // thread r zeroes its row r past `last` before P_j V_j reads it
-            // (P is zero there, but those cache rows may hold anything)
-            const bool clip = j * kFa + kFa - 1 > last;
-            if (x == 0 && clip) {
-                good = good && fa_wait(&hd->v_full[b], (j >> 1) & 1, err);
-                if (j * kFa + r > last) {
-                    unsigned char *vt = smem + kOffV + b * kTileBytes;
-#pragma unroll
-                    for (int c = 0; c < kFa; c += 8)
-                        *reinterpret_cast<uint4 *>(vt + (c >> 6) * kHalfBytes +
-                                                   swizzle_offset((uint32_t)r, (uint32_t)(c & 63))) =
-                            make_uint4(0u, 0u, 0u, 0u);
-                }
-            }
-            // the row's 128 scores of S_j
-            good = good && fa_wait(&hd->s_full[x], j & 1, err);
-            tc_fence_after();
-            float v[kFa];
-#pragma unroll
-            for (int c = 0; c < kFa; c += 32)
-                tmem_ld32(s_col + c, *reinterpret_cast<float(*)[32]>(&v[c]));
-            tmem_ld_wait();
-            const bool full = j * kFa + kFa - 1 <= p0;  // no position of the tile is masked
-            float hm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            if (full) {
-#pragma unroll
-                for (int i = 0; i < kFa; ++i) hm4[i & 3] = fmaxf(hm4[i & 3], v[i]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < kFa; ++i)
-                    if (j * kFa + i <= qpos) hm4[i & 3] = fmaxf(hm4[i & 3], v[i]);
-            }
-            // finite: position 128j <= qpos for every row of the tile
-            const float mrow = fmaxf(fmaxf(hm4[0], hm4[1]), fmaxf(hm4[2], hm4[3])) * sl2;
-            const bool bump = mrow > m + kFaRescale;
-            const float corr = bump ? exp2f(m - mrow) : 1.f;  // 0 on the first tile
-            if (bump) m = mrow;
-            // P_j in bf16 pairs over the first 64 columns of S_j, 64 positions
-            // at a time; the row sum takes the probabilities as stored, so the
-            // weights P V is normalised by sum to exactly one
-            const float2 sl2x2 = make_float2(sl2, sl2), nm2 = make_float2(-m, -m);
-            float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                uint32_t pw[32];
-#pragma unroll
-                for (int i = 0; i < 64; i += 2) {
-                    const int c = half * 64 + i;
-                    const float2 e = __ffma2_rn(make_float2(v[c], v[c + 1]), sl2x2, nm2);
-                    float pa = fast_exp2(e.x);
-                    float pb = fast_exp2(e.y);
-                    if (!full) {
-                        if (j * kFa + c > qpos) pa = 0.f;
-                        if (j * kFa + c + 1 > qpos) pb = 0.f;
-                    }
-                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(pa, pb);
-                    sum2[(i >> 1) & 1] = __fadd2_rn(sum2[(i >> 1) & 1], __bfloat1622float2(p2));
-                    pw[i >> 1] = *reinterpret_cast<const uint32_t *>(&p2);
-                }
-                tmem_st32(s_col + half * 32, pw);
-            }
-            // a new base rescales O (the scores are consumed by now): P_{j-1}
-            // V_{j-1} finished before S_j was issued, and P_j V_j waits for
-            // this warp's arrival; the whole warp loads and stores (rows
-            // without a new base scale by 1)
-            if (j >= 1 && __any_sync(0xffffffffu, bump) && __all_sync(0xffffffffu, good)) {
-#pragma unroll 1
-                for (int c = 0; c < kFa; c += 32) {
-                    float ov[32];
-                    uint32_t ow[32];
-                    tmem_ld32(o_col + c, ov);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) ow[i] = __float_as_uint(ov[i] * corr);
-                    tmem_st32(o_col + c, ow);
-                }
-            }
-            tmem_st_wait();
-            if (x == 0 && clip) fence_proxy_async_smem();  // the zeroed value rows
-            tc_fence_before();                             // P_j and a rescaled O
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&hd->p_ready[x]);
-            l = l * corr + ((sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y));
-        }
+        float l = 0.f;
+        const bool good = two ? fa_softmax_two(hd, smem, s_col, o_col, n_kv, p0, rows, r, x, l, err)
+                              : fa_softmax(hd, smem, s_col, o_col, n_kv, p0, rows, r, x, l, err);
         const bool fin = good && fa_wait(&hd->o_full[x], (n_kv - 1) & 1, err);
         if (!fin) hd->gave_up = 1;
         if (__all_sync(0xffffffffu, fin)) {

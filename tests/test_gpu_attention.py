@@ -626,3 +626,54 @@ def test_projections_of_many_tokens(D, Hq, Hkv, T):
     scale = 1.0 / np.sqrt(np.mean((want - x) ** 2, axis=1, keepdims=True))
     assert_parity((to_numpy(resid) - x) * scale, (want - x) * scale, "bf16",
                   "attention block")
+
+
+# (Hq, Hkv, max_len, runs): as RAGGED above; tokens that no tile of 128 at a
+# multiple of 128 of the call's tokens holds: decode tokens (batches of 128 and
+# fewer), the tail of a prompt, chunks that start anywhere, two heads a unit and
+# one, an odd group of query heads, a whole tile at an odd start
+TERMS = [
+    (6, 2, 160, [(-1, 0, 200)]),
+    (12, 4, 300, [(-1, 0, 30), (0, 0, 100), (1, 40, 129)]),
+    (3, 1, 200, [(0, 0, 150)]),
+    (4, 2, 260, [(-1, 0, 3), (0, 100, 128), (1, 0, 17)]),
+    (8, 1, 300, [(0, 128, 60), (-1, 0, 80)]),
+]
+
+
+@pytest.mark.parametrize("Hq,Hkv,L,runs", TERMS, ids=lambda v: str(v)[:24])
+def test_probabilities_keep_their_bits(Hq, Hkv, L, runs):
+    """The probabilities of tokens outside full aligned tiles enter P V with 16
+    bits: each element of ctx is its 64-bit value within its own bf16 rounding
+    and 2^-15 of its sum of |p v| (2^-17 from each probability, as much from the
+    row sum; fp32 scores of |s| < 32 in base 2 move a probability by less than
+    2^-18 and the sums of up to 300 terms by less than 2^-17).  One bf16 term
+    (2^-9 of each) breaks that where the weighted values nearly cancel."""
+    m = moe()
+    rng = np.random.default_rng(L + Hq)
+    seq, pos, n_seq = [], [], 1 + max(r[0] for r in runs)
+    for s, p0, n in runs:
+        if s >= 0:
+            seq += [s] * n
+            pos += range(p0, p0 + n)
+        else:
+            seq += range(n_seq, n_seq + n)
+            pos += rng.integers(0, L, size=n).tolist()
+            n_seq += n
+    seq, pos = np.array(seq, np.int32), np.array(pos, np.int32)
+    T = seq.size
+    shape = gen.AttnShape(Hq * 128, Hq, Hkv, 128, 10000.0, "bf16")
+    kc, vc = (gen.store(rng.normal(size=(n_seq, Hkv, L, 128)), "bf16") for _ in range(2))
+    q = rng.normal(size=(T, Hq, 128)).astype(np.float32)
+    ctx = m.sa_attend(_sa(m, shape), torch.from_numpy(q).cuda(), torch.from_numpy(seq).cuda(),
+                      torch.from_numpy(pos).cuda(), dev(kc, "bf16"), dev(vc, "bf16"))
+    assert m.get_last_error() == 0
+    q64, k64, v64 = oracle.round_bf16(q.astype(np.float64)), gen.to_f64(kc, "bf16"), gen.to_f64(vc, "bf16")
+    want = oracle.attention(q64, k64, v64, seq, pos).reshape(T, Hq * 128)
+    size = oracle.attention(q64, k64, np.abs(v64), seq, pos).reshape(T, Hq * 128)
+    one = np.zeros(T, bool)  # full tiles at a multiple of 128: one term
+    for t in range(0, T - 127, 128):
+        one[t:t + 128] = np.all(seq[t:t + 128] == seq[t]) and np.all(np.diff(pos[t:t + 128]) == 1)
+    err = np.abs(to_numpy(ctx) - want)
+    lim = 2.0 ** -8 * np.abs(want) + 2.0 ** -15 * size
+    assert np.all(err[~one] <= lim[~one]), float(np.max((err / lim)[~one]))
