@@ -307,6 +307,8 @@ k_rope_cache(int T, int Hq, int Hkv, int n_seq, int L, RopeRates rates,
              bf16 *__restrict__ vc, int *__restrict__ dec_count, unsigned *err) {
     // the tensor-core attention, one CTA per SM on the SMs that this grid
     // leaves free, may launch now and set itself up while this kernel runs
+    // (ahead of this kernel's own wait: the projection before it ends without
+    // a trigger, so all that is ahead of the call is complete)
     ptx::launch_dependents();
     ptx::grid_dependency_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0) zero_dec_count(dec_count);
@@ -642,7 +644,8 @@ k_attn_merge(int n_split, const float *__restrict__ part_ml, const float *__rest
 
 // The tensor-core attention's bf16 copy of fp32 queries, for a call that
 // brings its own queries (moe_sa_attend); in the whole block the rotary
-// kernel writes it.  n4 groups of four elements.
+// kernel writes it.  n4 groups of four elements.  It lets no launch start before
+// its wait: the decode attention reads seq and pos ahead of its own.
 __global__ void __launch_bounds__(256)
 k_q_bf16(int T, long long n4, const float *__restrict__ q, bf16 *__restrict__ q16,
          int *__restrict__ dec_count, const PlanArgs pa) {

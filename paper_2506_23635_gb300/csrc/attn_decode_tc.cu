@@ -86,9 +86,13 @@
 // before storing, by when the wait is long satisfied.)
 //
 // The kernel launches while the one ahead of it (which writes the call's new
-// cache rows and the queries) runs; key and value tiles that lie wholly before
-// the call's own positions do not depend on it and are loaded at once (0.5-1.5
-// us of the attention block at 1-11 sequences).
+// cache rows and the queries) runs, and asks for its first tiles' lines in L2
+// meanwhile; it loads nothing before it has waited.  (Loads of tiles that the
+// call does not write were sent before the wait for a time: the wait then lasts
+// until these copies have landed, 3 us by clock stamps where every SM sends three
+// tiles.  Attention block of DBRX, no early copies, loads, lines asked for: 9
+// sequences of up to 2048 positions 52.2, 53.3 and 50.8 us, 16 60.2, 60.0 and 58.4,
+// 11 up to 4096 79.7 (other schedule), 68.1 and 66.2.)
 //
 // Numerics: bf16 queries, fp32 scores and accumulation, probabilities in two
 // bf16 terms (2^-17 of each at most unaccounted for: the padding rows of N hold
@@ -480,8 +484,8 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 #pragma unroll 1
     for (int t_base = 0; !LISTED || t_base < n_listed; t_base += kDecMaxTokens) {
     if (LISTED) T = min(kDecMaxTokens, n_listed - t_base);
-    // The producer warp sets up the barriers, finds the CTA's share and sends
-    // its first tiles before the block-wide barrier.
+    // The producer warp sets up the barriers and finds the CTA's share before
+    // the block-wide barrier.
     // the next tile to send: token, head, tile of its sequence, and the
     // sequence's tiles
     struct At {
@@ -491,7 +495,8 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     long long W = 0;
     int n_share = 1;
     bool whole_only = false;  // the shares are the (token, head)s
-    int cur = cta, total = 0, early = 0;  // the share, its tiles
+    int cur = cta, total = 0;  // the share, its tiles
+    int n_pre = 0;             // tiles sent right after the wait
     const uint64_t pol_kv = ptx::policy_evict_first();  // key and value tiles are read once
     // the tile after a, its share's j-th; false: there is none.  A split's
     // first kDecStages tiles are fixed (c, c + n_split, ...); `taken` is then
@@ -676,37 +681,17 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 find(at);
             }
         }
-        // key and value tiles that no token of this call writes into (all of
-        // the sequence's positions in them lie before the call's first one)
-        // hold what earlier calls left, complete before the kernel ahead of
-        // this one began: the first stages of them are loaded before the wait
-        // for that kernel
+        // the lines of the first stages' tiles, on their way into L2 while the
+        // kernel ahead runs
         At a = at;
         bool have = !LISTED && total > 0;
 #pragma unroll 1
         for (int j = 0; j < kDecStages && have; ++j) {
-            const int sq = hd->seq[a.t];
-            int first_pos = 0x7fffffff;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (tok_seq[i] == sq) first_pos = min(first_pos, tok_n[i] - 1);
-            first_pos = __reduce_min_sync(0xffffffffu, first_pos);
-            if (hd->n[a.t] > 0 && (a.tile + 1) * kDecPos <= first_pos) {
-                early |= 1 << j;
-                if (lane == 0) {
-                    const int row = (sq * Hkv + a.g) * L + a.tile * kDecPos;
-                    const bool first = j == 0 || (!SPLIT && a.tile == 0);
-                    ptx::mbar_arrive_expect_tx(&hd->k_full[j], kDecTile + (first ? kDecQ : 0u));
-                    ptx::mbar_arrive_expect_tx(&hd->v_full[j], kDecTile);
-                    for (int half = 0; half < 2; ++half)
-                        ptx::tma_load_2d(smem + kDecOffK + j * kDecTile + half * kDecHalf, &tmK,
-                                         half * 64, row, &hd->k_full[j], pol_kv);
-                    for (int half = 0; half < 2; ++half)
-                        ptx::tma_load_2d(smem + kDecOffV + j * kDecTile + half * kDecHalf, &tmV,
-                                         half * 64, row, &hd->v_full[j], pol_kv);
-                }
-            }
-            have = j + 1 < kDecStages && advance(a, j + 1, 0);
+            if (lane < 4)
+                ptx::tma_prefetch_2d(lane < 2 ? &tmK : &tmV, (lane & 1) * 64,
+                                     (hd->seq[a.t] * Hkv + a.g) * L + a.tile * kDecPos);
+            n_pre = j + 1;
+            have = n_pre < kDecStages && advance(a, n_pre, 0);
         }
     }
     if (warp == 1 && (!LISTED || t_base == 0)) tmem_alloc(&hd->tmem_base, kDecTmemCols);
@@ -725,11 +710,29 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         const uint64_t pol_q = ptx::policy_evict_normal();
-        if (!LISTED && lane == 0 && total > 0) {  // the first piece's query rows
-            if (!(early & 1)) ptx::mbar_arrive_expect_tx(&hd->k_full[0], kDecTile + kDecQ);
-            for (int half = 0; half < 2; ++half)
-                ptx::tma_load_2d(smem + kDecOffQ + half * kDecNHalf, &tmQ, half * 64,
-                                 token(at.t) * Hq + at.g * G, &hd->k_full[0], pol_q);
+        // the first stages' keys and values and their pieces' query rows, at once
+        if (lane == 0) {
+            At a = at;
+            int piece = -1;
+            for (int j = 0; j < n_pre; ++j) {
+                const bool first = j == 0 || (!SPLIT && a.tile == 0);
+                const int row = (hd->seq[a.t] * Hkv + a.g) * L + a.tile * kDecPos;
+                ptx::mbar_arrive_expect_tx(&hd->k_full[j], kDecTile + (first ? kDecQ : 0u));
+                if (first) {
+                    ++piece;
+                    for (int half = 0; half < 2; ++half)
+                        ptx::tma_load_2d(smem + kDecOffQ + piece * kDecQ + half * kDecNHalf, &tmQ,
+                                         half * 64, a.t * Hq + a.g * G, &hd->k_full[j], pol_q);
+                }
+                for (int half = 0; half < 2; ++half)
+                    ptx::tma_load_2d(smem + kDecOffK + j * kDecTile + half * kDecHalf, &tmK,
+                                     half * 64, row, &hd->k_full[j], pol_kv);
+                ptx::mbar_arrive_expect_tx(&hd->v_full[j], kDecTile);
+                for (int half = 0; half < 2; ++half)
+                    ptx::tma_load_2d(smem + kDecOffV + j * kDecTile + half * kDecHalf, &tmV,
+                                     half * 64, row, &hd->v_full[j], pol_kv);
+                advance(a, j + 1, 0);
+            }
         }
         if constexpr (SPLIT) cluster_wait();  // CTA 0's counter is initialised before the first take
         if (lane == 0) {
@@ -802,11 +805,11 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 d.flags = (d.flags & ~(kDecFirst | kDecLast | kDecEnd)) | (first ? kDecFirst : 0) |
                           (last ? kDecLast : 0) | (more ? 0 : kDecEnd);
                 const int row = (hd->seq[at.t] * Hkv + at.g) * L + at.tile * kDecPos;
-                const bool sent = j < kDecStages && ((early >> j) & 1);  // before the wait above
+                const bool sent = j < n_pre;  // above
                 if (!(good = dec_wait(&hd->k_empty[b], ph, err))) break;
-                if (!sent && (LISTED || j > 0))
+                if (!sent)
                     ptx::mbar_arrive_expect_tx(&hd->k_full[b], kDecTile + (first ? kDecQ : 0u));
-                if (first && (LISTED || j > 0))
+                if (first && !sent)
                     for (int half = 0; half < 2; ++half)
                         ptx::tma_load_2d(smem + kDecOffQ + (piece % kDecQBufs) * kDecQ +
                                              half * kDecNHalf,

@@ -395,7 +395,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 // flight: the reduction is split over gridDim.y CTAs per tile (split z writes
 // its partial sums to y_out + z*T*Nw; the caller adds the parts in order).
 // The weight loads of the first stages are issued before the kernel waits
-// for the previous grid (weights do not depend on it).
+// for the previous grid (weights do not depend on it; that one has waited for
+// all that is ahead of the call).  The kernel has no trigger of its own: the
+// rotary kernel and, through it, the decode attention rely on its end.
 template <int NTOK>
 struct SwapCfg {
     static constexpr uint32_t kStageW = BM * BK * 2;     // 16 KB of weights

@@ -27,6 +27,9 @@
 //    pair, whose CTAs hold N/2 slots each).  N is a field of the instruction
 //    descriptor, set per tile, so a ragged expert wastes at most 15 (31)
 //    columns per run rather than up to 127 rows of a fixed 128-slot tile.
+// No form has a trigger of its own: as a projection it is ahead of kernels that
+// start before their waits and rely on its end.
+//
 // Units are numbered expert by expert, weight tile outer and slot tile inner
 // (units running at the same time share weight tiles in L2); CTA (pair) b of
 // G takes units b, b+G, ... in full rounds, and a piece of one of the last

@@ -205,6 +205,14 @@ __device__ __forceinline__ void tma_load_2d(void *dst_smem, const void *tmap, in
         : "memory");
 }
 
+// The tile's lines into L2 (nothing is read by the caller: safe before a
+// dependency wait).
+__device__ __forceinline__ void tma_prefetch_2d(const void *tmap, int32_t x, int32_t y) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tmap),
+                 "r"(x), "r"(y)
+                 : "memory");
+}
+
 __device__ __forceinline__ void prefetch_tmap(const void *tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
 }

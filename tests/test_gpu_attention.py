@@ -677,3 +677,46 @@ def test_probabilities_keep_their_bits(Hq, Hkv, L, runs):
     err = np.abs(to_numpy(ctx) - want)
     lim = 2.0 ** -8 * np.abs(want) + 2.0 ** -15 * size
     assert np.all(err[~one] <= lim[~one]), float(np.max((err / lim)[~one]))
+
+
+# (Hq, Hkv, n_seq, max_len, longest): clusters of CTAs for a (token, head), a
+# CTA for each, and equal shares of all tiles (one sequence far longer than the rest)
+STEPS = [(6, 1, 3, 700, 600), (12, 4, 24, 700, 400), (12, 4, 24, 2600, 2500)]
+
+
+@pytest.mark.parametrize("Hq,Hkv,n_seq,L,longest", STEPS, ids=lambda v: str(v))
+def test_decode_steps_back_to_back(Hq, Hkv, n_seq, L, longest):
+    """Four decode steps on one stream with nothing between them, over positions
+    that cross the ends of 128-position tiles: a step reads the rows that the
+    step ahead of it wrote last."""
+    m = moe()
+    rng = np.random.default_rng(n_seq + L)
+    shape = gen.AttnShape(256, Hq, Hkv, 128, 10000.0, "bf16")
+    w_qkv, w_o = gen.host_attn_weights(shape, 17)
+    kc, vc = gen.host_kv_cache(shape, n_seq, L, 17)
+    first = rng.integers(1, 300, size=n_seq).astype(np.int32)
+    first[:3] = 126, 254, longest - 4
+    seq = np.arange(n_seq, dtype=np.int32)
+    nan = gen.store(np.full(1, np.nan), "bf16")[0]
+    kc, vc = kc.copy(), vc.copy()
+    for s in range(n_seq):
+        kc[s, :, first[s]:] = nan
+        vc[s, :, first[s]:] = nan
+    x = [rng.normal(size=(n_seq, 256)).astype(np.float32) for _ in range(4)]
+    pos = [first + i for i in range(4)]
+    a, dk, dv = _sa(m, shape), dev(kc, "bf16"), dev(vc, "bf16")
+    dq, do, ds = dev(w_qkv, "bf16"), dev(w_o, "bf16"), torch.from_numpy(seq).cuda()
+    resid = [torch.from_numpy(v.copy()).cuda() for v in x]
+    dpos = [torch.from_numpy(p).cuda() for p in pos]
+    ws = torch.empty(m.sa_workspace_size(a, n_seq), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(4):
+        m.sa_forward(a, resid[i], dq, do, ds, dpos[i], dk, dv, eps=EPS, ws=ws)
+    assert m.get_last_error() == 0
+    k64, v64 = gen.to_f64(kc, "bf16"), gen.to_f64(vc, "bf16")
+    for i in range(4):
+        want, k64, v64 = oracle.sa_forward(x[i].astype(np.float64), w_qkv, w_o, "bf16", Hq, Hkv,
+                                           shape.rope_base, EPS, seq, pos[i], k64, v64)
+        # (each row held to the bound on its own RMS, as above)
+        scale = 1.0 / np.sqrt(np.mean((want - x[i]) ** 2, axis=1, keepdims=True))
+        assert_parity((to_numpy(resid[i]) - x[i]) * scale, (want - x[i]) * scale, "bf16", f"step {i}")
