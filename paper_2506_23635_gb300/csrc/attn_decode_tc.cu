@@ -23,7 +23,8 @@
 //            W tiles, so every SM streams the same number of bytes whatever
 //            the sequences' lengths.  A share is a run of pieces: the end of
 //            one (token, head)'s tiles, whole ones, the start of another's.
-//            Where there are many (token, head)s to a CTA, it takes them whole,
+//            Where they are of like length, or no more than a CTA each, a CTA
+//            has one whole; where there are many to a CTA, it takes them whole,
 //            longest first and one after the other from a counter: parts and
 //            their merges cost more than the uneven ends (attention block at
 //            48 sequences of 512-2048 positions and a chunk of 8: 97 us with
@@ -183,6 +184,14 @@ constexpr int kDecMaxWhole = 4;
 // tokens of DBRX, 1.7, up to 4096 positions: 102 us in equal shares, 112 with
 // a CTA each)
 constexpr int kDecWholeMin = 2;
+// and where there is a CTA for each unless the longest has more tiles than an
+// equal share and this many: parts and their merges cost about as much as
+// these tiles take (attention block of DBRX, a CTA each against equal shares: 16
+// sequences of up to 864 positions, longest 3 tiles over the share, 49.9 and
+// 52.5 us, 1400: 5 over, 54.4 and 55.8, 2048: 7 over, 59.7 and 59.8, 4096: 15
+// over, 76.9 and 71.8; 12 of up to 1400: 7 over, 53.4 and 53.5, 2048: 10 over,
+// 58.8 and 57.0)
+constexpr int kDecWholeSlack = 5;
 // listed tokens: taken whole unless the longest has more tiles than twice an
 // equal share and this many.  The CTAs start one by one as the prefill
 // attention leaves them SMs, and an equal share that starts late ends late
@@ -495,6 +504,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     long long W = 0;
     int n_share = 1;
     bool whole_only = false;  // the shares are the (token, head)s
+    bool taking = false;      // and a CTA takes more than one
     int cur = cta, total = 0;  // the share, its tiles
     int n_pre = 0;             // tiles sent right after the wait
     const uint64_t pol_kv = ptx::policy_evict_first();  // key and value tiles are read once
@@ -642,14 +652,16 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             if (lane == 31) hd->before[kDecMaxTokens] = run;
             __syncwarp();
             W = (long long)hd->before[kDecMaxTokens] * Hkv;
-            if (LISTED) {
-                const int longest = __reduce_max_sync(
-                    0xffffffffu, max(max(nt[0], nt[1]), max(nt[2], nt[3])));
+            const int longest =
+                __reduce_max_sync(0xffffffffu, max(max(nt[0], nt[1]), max(nt[2], nt[3])));
+            if (LISTED)
                 whole_only = n_listed > kDecMaxTokens ||
                              longest <= 2 * W / (int)gridDim.x + kDecListedSlack;
-            } else {
-                whole_only = T * Hkv >= kDecWholeMin * (int)gridDim.x;
-            }
+            else
+                whole_only = T * Hkv >= kDecWholeMin * (int)gridDim.x ||
+                             (T * Hkv <= (int)gridDim.x &&
+                              longest <= W / (int)gridDim.x + kDecWholeSlack);
+            taking = whole_only && (LISTED || T * Hkv > (int)gridDim.x);
             n_share = whole_only ? T * Hkv
                                  : (int)min((long long)gridDim.x,
                                             max(1LL, W < (1 << 24)
@@ -783,7 +795,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 // a stage frees)
                 if (SPLIT && more && j + 2 >= kDecStages)
                     taken = kDecStages * n_split + (int)dec_take(counter);
-                if (!SPLIT && whole_only && at.tile == std::max(0, at.nt - 3)) share = take();
+                if (!SPLIT && taking && at.tile == std::max(0, at.nt - 3)) share = take();
                 const bool first = jj == 0 || (!SPLIT && at.tile == 0);
                 const bool last = !more || (!SPLIT && at.tile == at.nt - 1);
                 if (first) {
@@ -829,7 +841,7 @@ k_attn_decode_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 have = more;
                 ++jj;
                 if (!SPLIT && !have) {
-                    have = whole_only && next_share();
+                    have = taking && next_share();
                     nxt = at;
                 }
                 more = have && advance(nxt, SPLIT ? j + 2 : jj + 1, taken);
@@ -1220,18 +1232,17 @@ const DecClusters &dec_clusters() {
 // CTAs for each of `pairs` (token, key/value head)s: the largest cluster that
 // is resident for all of them at once (attention block of DBRX at 2 sequences
 // of 2048 positions: 6 CTAs 50.0 us, 8 CTAs, one cluster left over, 54.3 us).
-// 1: the shares of all tiles.  They lose to clusters while those fill the SMs
-// (8 sequences: 59.4 against 57.0 us at 2048 positions, the same up to 4096)
-// -- a part left in the workspace costs its CTA a fence and a count, the
-// merging CTA two more trips to L2 -- and win where clusters would leave more
-// than a quarter of the SMs out (6 sequences, clusters of 2: 63.5 against 65.5
-// us up to 4096 positions, 58.8 against 57.4 us at 2048), unless there are so
-// few (token, head)s that most would be merged (2 sequences: 53-56 us).
-int dec_splits(int pairs, int max_tiles, int sms) {
+// 1: whole ones or the shares of all tiles, chosen on the device.  Clusters of
+// two beat the shares up to 76 pairs, also where they leave a third of the SMs
+// out (6 sequences of up to 864, 2048 and 4096 positions: 47.0, 51.0 and 59.5
+// us against 49.3, 53.8 and 58.9; 7: 47.2, 51.7 and 60.1 against 49.8, 54.8
+// and 59.5; 9: 47.9, 52.6 and 60.8 against 51.0, 54.8 and 62.3): a part left in
+// the workspace costs its CTA a fence and a count, the merging CTA two more
+// trips to L2.
+int dec_splits(int pairs, int max_tiles) {
     const DecClusters &dc = dec_clusters();
     int n = std::min(max_tiles, kDecMaxSplit);
     while (n > 1 && dc.resident[n] < pairs) --n;
-    if (4 * n * pairs < 3 * sms && 4 * pairs > sms) n = 1;
     return std::max(1, n);
 }
 
@@ -1259,7 +1270,7 @@ cudaError_t launch_attn_decode_tc(int T, int Hq, int Hkv, int n_seq, int L, cons
     // (listed tokens are counted on the device: one CTA per SM)
     const int pairs = T * Hkv, sms = std::min(device_info().sm_count, kAttnDecodeMaxCtas);
     const int max_tiles = (L + kDecPos - 1) / kDecPos;
-    int n_split = plan ? 1 : dec_splits(pairs, max_tiles, sms);
+    int n_split = plan ? 1 : dec_splits(pairs, max_tiles);
     AttnPlan pl = plan ? *plan : AttnPlan{};
     const void *kern = plan          ? dec_kernel<kDecListed>(G)
                        : n_split > 1 ? dec_kernel<kDecSplits>(G)
