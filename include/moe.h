@@ -388,7 +388,7 @@ moe_status moe_sa_qkv(const moe_sa_dims *dims, int32_t T, const void *x_norm,
  * consecutive tokens that are consecutive positions of one sequence (a
  * prefill chunk) are attended by the tensor-core flash attention in tiles of
  * up to 128, all other tokens by the tensor-core decode attention.  (A call
- * of up to 128 tokens with fewer than 48 more of them than the caches have
+ * of under 128 tokens with fewer than 48 more of them than the caches have
  * sequences is taken as a decode step.)  MOE_ATTN_CUDA_CORES=1 in the
  * environment keeps the tokens outside tiles, and calls of under 128 tokens,
  * on the CUDA-core kernel. */

@@ -893,23 +893,23 @@ bool decode_tc() {
     return !off && attn_decode_tc_ok();
 }
 
-// Whether a call's tokens are sorted into prefill tiles and the rest.  A small
-// call with hardly more tokens than the caches have sequences is a decode
-// step: every token goes to the decode kernel, which takes any, and the launch
-// of the other is saved.  (The attention block of DBRX: 127 tokens from
-// position 512 on 107 us one by one, each streaming its keys and values for
-// itself, 76 us as a tile; 100 tokens at 0 72 and 70 us; 40 tokens at 300, and
-// 30 tokens beside 40 decode tokens, the same either way; 16 tokens at 0 48.6
-// against 50.6 us, four runs of 9 at 600 beside 40 decode tokens 100 against
-// 104 us.  A prompt of 1000 tokens whose last 104 had gone to the
-// CUDA cores: 376 -> 231 us; 24 decode tokens and chunks of 300 and 205, with
-// 273 tokens on the CUDA cores: 487 -> 197 us.)
+// Whether a call's tokens are sorted into prefill tiles and the rest.  A call
+// that cannot hold a full tile, with hardly more tokens than the caches have
+// sequences, is taken as a decode step: every token goes to the decode kernel,
+// which takes any, and the launch of the other is saved.  (The caches' sequences
+// are all that the host knows of how the tokens are spread: a chunk over caches
+// of many idle sequences is so taken one by one up to 127 tokens, as any call
+// below 128 was before there were ragged tiles: 127 tokens from position 512 on
+// over 96 sequences 92.8 us, 128 tokens there as a tile 65.4.)  The attention
+// block of DBRX, one by one and as a tile: 100 tokens at 0 72 and 70 us; 40
+// tokens at 300, and 30 tokens beside 40 decode tokens, the same either way; 16
+// tokens at 0 48.6 and 50.6 us, four runs of 9 at 600 beside 40 decode tokens
+// 100 and 104 us.
 constexpr int kPlanMinTokens = 48;  // beyond one for each sequence
 
 bool planned(int T, int n_seq) {
     if (!attn_prefill_tc_ok()) return false;
-    return decode_tc() ? T > kAttnDecodeMaxTokens || T - n_seq >= kPlanMinTokens
-                       : T >= kAttnTile;
+    return T >= kAttnTile || (decode_tc() && T - n_seq >= kPlanMinTokens);
 }
 
 AttnPlan plan_at(const SaCall &c) {

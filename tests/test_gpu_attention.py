@@ -720,3 +720,25 @@ def test_decode_steps_back_to_back(Hq, Hkv, n_seq, L, longest):
         # (each row held to the bound on its own RMS, as above)
         scale = 1.0 / np.sqrt(np.mean((want - x[i]) ** 2, axis=1, keepdims=True))
         assert_parity((to_numpy(resid[i]) - x[i]) * scale, (want - x[i]) * scale, "bf16", f"step {i}")
+
+
+@pytest.mark.parametrize("T,tile", [(128, True), (127, False)])
+def test_tile_of_128_over_many_sequences(T, tile):
+    """A chunk of a whole tile is one however many sequences the caches hold."""
+    m = moe()
+    shape = gen.AttnShape(256, 2, 1, 128, 10000.0, "bf16")
+    n_seq, L = 100, 200
+    kc, vc = gen.host_kv_cache(shape, n_seq, L, 5)
+    seq, pos = np.full(T, 41, np.int32), np.arange(30, 30 + T, dtype=np.int32)
+    q = np.random.default_rng(T).normal(size=(T, 2, 128)).astype(np.float32)
+    m.profile_reset()
+    m.profile_enable(True)
+    ctx = m.sa_attend(_sa(m, shape), torch.from_numpy(q).cuda(), torch.from_numpy(seq).cuda(),
+                      torch.from_numpy(pos).cuda(), dev(kc, "bf16"), dev(vc, "bf16"))
+    torch.cuda.synchronize()
+    m.profile_enable(False)
+    assert m.get_last_error() == 0
+    assert (m.profile_read().get("attention_tc", (0, 0))[0] > 0) == tile
+    want = oracle.attention(oracle.round_bf16(q.astype(np.float64)), gen.to_f64(kc, "bf16"),
+                            gen.to_f64(vc, "bf16"), seq, pos)
+    assert_parity(to_numpy(ctx), want.reshape(T, 256), "bf16", "one tile", True)
