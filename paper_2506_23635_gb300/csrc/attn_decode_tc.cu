@@ -186,11 +186,11 @@ constexpr int kDecMaxWhole = 4;
 constexpr int kDecWholeMin = 2;
 // and where there is a CTA for each unless the longest has more tiles than an
 // equal share and this many: parts and their merges cost about as much as
-// these tiles take (attention block of DBRX, a CTA each against equal shares: 16
-// sequences of up to 864 positions, longest 3 tiles over the share, 49.9 and
-// 52.5 us, 1400: 5 over, 54.4 and 55.8, 2048: 7 over, 59.7 and 59.8, 4096: 15
-// over, 76.9 and 71.8; 12 of up to 1400: 7 over, 53.4 and 53.5, 2048: 10 over,
-// 58.8 and 57.0)
+// these tiles take (attention block of DBRX, a CTA each and equal shares: 16
+// sequences of up to 864 positions, longest 4 tiles over the share, 49.3 and 51.4
+// us, 2047 each: 3 over, 62.0 and 64.5, up to 2048: 8 over, 59.4 and 58.1, 4096: 15
+// over, 76.2 and 70.9; 18 of up to 1400: 5 over, 54.5 and 56.2, 2048: 7 over, 59.8
+// and 60.4; 12 of up to 1400: 7 over, 54.1 and 52.5)
 constexpr int kDecWholeSlack = 5;
 // listed tokens: taken whole unless the longest has more tiles than twice an
 // equal share and this many.  The CTAs start one by one as the prefill
@@ -1234,9 +1234,9 @@ const DecClusters &dec_clusters() {
 // of 2048 positions: 6 CTAs 50.0 us, 8 CTAs, one cluster left over, 54.3 us).
 // 1: whole ones or the shares of all tiles, chosen on the device.  Clusters of
 // two beat the shares up to 76 pairs, also where they leave a third of the SMs
-// out (6 sequences of up to 864, 2048 and 4096 positions: 47.0, 51.0 and 59.5
-// us against 49.3, 53.8 and 58.9; 7: 47.2, 51.7 and 60.1 against 49.8, 54.8
-// and 59.5; 9: 47.9, 52.6 and 60.8 against 51.0, 54.8 and 62.3): a part left in
+// out (6 sequences of up to 864, 2048 and 4096 positions: 45.9, 50.3 and 59.1
+// us against 49.5, 53.1 and 56.9; 7: 46.0, 50.6 and 59.2 against 50.0, 53.7
+// and 58.1; 9: 47.1, 51.2 and 59.6 against 50.1, 54.2 and 61.0): a part left in
 // the workspace costs its CTA a fence and a count, the merging CTA two more
 // trips to L2.
 int dec_splits(int pairs, int max_tiles) {
