@@ -54,6 +54,7 @@ struct RtHeader {
     uint64_t empty[kRtMaxStages];
     uint64_t done;
     uint32_t tmem;
+    int gave_up;  // the issuer's wait ran out: some accumulators were not written
 };
 
 // Ring stages for nkb k-blocks a share: as many as fit beside the router's slice
@@ -139,6 +140,7 @@ k_route_tc(const __grid_constant__ CUtensorMap tmX, int T, int D, int E, int K, 
         }
         ptx::mbar_init(&hd->done, 1);
         ptx::fence_barrier_init();
+        hd->gave_up = 0;
         // the token rows may come from the previous kernel (so may W_r, whose
         // layout below waits too); the first stages of them are on the way
         // while W_r is laid out
@@ -210,7 +212,11 @@ k_route_tc(const __grid_constant__ CUtensorMap tmX, int T, int D, int E, int K, 
         if (lane == 0) {
             for (int i = 0; i < nkb; ++i) {
                 const uint32_t s = i % n_stage, ph = (i / n_stage) & 1;
-                if (!ptx::mbar_wait_hint(&hd->full[s], ph, err)) break;
+                if (!ptx::mbar_wait_hint(&hd->full[s], ph, err)) {
+                    hd->gave_up = 1;
+                    __threadfence_block();  // ahead of the arrival on `done`
+                    break;
+                }
                 tc_fence_after();
                 const uint64_t adesc = smem_desc(ptx::smem_u32(smem + s * kRtStageBytes));
                 const uint64_t bdesc = smem_desc(ptx::smem_u32(wt + i * kRtPanelBytes));
@@ -230,7 +236,8 @@ k_route_tc(const __grid_constant__ CUtensorMap tmX, int T, int D, int E, int K, 
     if (warp < 4) {
         // the partial logits of the warp's 32 tokens, to the CTAs that finish
         // them (zero for an empty share and after a wait that gave up)
-        const bool have = ptx::mbar_wait_hint(&hd->done, 0, err) && nkb > 0;
+        const bool have = ptx::mbar_wait_hint(&hd->done, 0, err) && nkb > 0 &&
+                          *(volatile int *)&hd->gave_up == 0;
         tc_fence_after();
         float p[16];
 #pragma unroll
