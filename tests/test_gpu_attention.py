@@ -65,7 +65,7 @@ CASES = [
     (1024, 8, 1, 4, 2500, "decode"),
     (384, 3, 1, 1, 1100, "decode1"),
     (512, 8, 4, 1, 100, "prefill"),  # one position split per token: ctx written directly
-    (256, 4, 2, 2, 400, "chunk300"),  # tensor-core prefill tiles + a CUDA-core tail
+    (256, 4, 2, 2, 400, "chunk300"),  # tensor-core prefill tiles, the last one ragged
 ]
 
 
@@ -228,7 +228,7 @@ def test_decoder_layers(kind):
 
 def test_prefill_ignores_cache_rows_past_the_chunk():
     """Positions 37..336 of sequence 1 (two tensor-core tiles whose last
-    key/value tile runs past their last query, and a CUDA-core tail) with NaN
+    key/value tile runs past their last query, and a ragged one) with NaN
     in every cache row the chunk does not reach: the result equals the
     oracle's, which reads only positions up to each token's own."""
     m = moe()
@@ -311,8 +311,7 @@ def _plateau_case(levels, T, L=600, seed=41):
 # (levels as (first, end, base-2 score), tokens): the exponent base moves in
 # the first tile, stays while the maximum rises by 4.5 (probabilities up to
 # 2^4.5), moves by 9 in the third tile and again inside the diagonal tile of
-# the fourth, then the scores drop by 20; a ragged CUDA-core tail after four
-# tensor-core tiles.  Then a maximum of 40 in the first tile that nothing
+# the fourth, then the scores drop by 20; a ragged tile after four full ones.  Then a maximum of 40 in the first tile that nothing
 # later approaches (every later probability ~2^-40).
 PLATEAUS = [
     ([(100, 230, 8.5), (230, 300, 13.0), (300, 420, 22.0), (420, 470, 31.0),
@@ -742,3 +741,88 @@ def test_tile_of_128_over_many_sequences(T, tile):
     want = oracle.attention(oracle.round_bf16(q.astype(np.float64)), gen.to_f64(kc, "bf16"),
                             gen.to_f64(vc, "bf16"), seq, pos)
     assert_parity(to_numpy(ctx), want.reshape(T, 256), "bf16", "one tile", True)
+
+
+# (Hq, Hkv, max_len, sequences, decode tokens, chunk at, which tokens are outside
+# the cache): a planned call whose run such tokens break at its ends and inside,
+# among listed tokens too; equal shares of all tiles (one long sequence), a CTA
+# for each (token, head), clusters
+OUTSIDE = [
+    (6, 2, 400, 120, 100, (110, 40, 150), [0, 37, 99, 100, 170, 249]),
+    (12, 4, 2600, 31, 30, None, [0, 11, 29]),
+    (12, 4, 300, 31, 30, None, [0, 11, 29]),
+    (3, 1, 700, 8, 5, None, [2, 4]),
+]
+
+
+@pytest.mark.parametrize("Hq,Hkv,L,n_seq,n_dec,chunk,out", OUTSIDE, ids=lambda v: str(v)[:20])
+def test_tokens_outside_the_cache_in_larger_calls(Hq, Hkv, L, n_seq, n_dec, chunk, out):
+    """Tokens whose sequence or position does not exist are reported, attend to
+    nothing (zero ctx: their residual row stays as it is) and write nothing; every
+    other token has the oracle's result."""
+    m = moe()
+    rng = np.random.default_rng(L + n_dec)
+    shape = gen.AttnShape(256, Hq, Hkv, 128, 10000.0, "bf16")
+    w_qkv, w_o = gen.host_attn_weights(shape, 29)
+    kc, vc = gen.host_kv_cache(shape, n_seq, L, 29)
+    seq = np.arange(n_dec, dtype=np.int32)
+    pos = rng.integers(0, min(L, 250), size=n_dec).astype(np.int32)
+    pos[1] = L - 1
+    if chunk:
+        s, p0, n = chunk
+        seq = np.concatenate([seq, np.full(n, s, np.int32)])
+        pos = np.concatenate([pos, np.arange(p0, p0 + n, dtype=np.int32)])
+    T = seq.size
+    for i, t in enumerate(out):  # a sequence below, past; a position below, past
+        if i % 4 < 2:
+            seq[t] = (-1, n_seq)[i % 4]
+        else:
+            pos[t] = (-1, L)[i % 4 - 2]
+    ok = np.setdiff1d(np.arange(T), out)
+    x = rng.normal(size=(T, 256)).astype(np.float32)
+    want, k64, v64 = oracle.sa_forward(x[ok].astype(np.float64), w_qkv, w_o, "bf16", Hq, Hkv,
+                                       shape.rope_base, EPS, seq[ok], pos[ok], gen.to_f64(kc, "bf16"),
+                                       gen.to_f64(vc, "bf16"))
+    resid = torch.from_numpy(x).cuda()
+    dk, dv = dev(kc, "bf16"), dev(vc, "bf16")
+    m.sa_forward(_sa(m, shape), resid, dev(w_qkv, "bf16"), dev(w_o, "bf16"),
+                 torch.from_numpy(seq).cuda(), torch.from_numpy(pos).cuda(), dk, dv, eps=EPS)
+    assert m.get_last_error() == 6 and m.get_last_error() == 0  # MOE_ERR_DEVICE_INDEX
+    got = to_numpy(resid)
+    assert np.array_equal(got[out], x[out].astype(np.float64))
+    scale = 1.0 / np.sqrt(np.mean((want - x[ok]) ** 2, axis=1, keepdims=True))
+    assert_parity((got[ok] - x[ok]) * scale, (want - x[ok]) * scale, "bf16", "tokens inside")
+    keep = ~_written(kc.shape, seq[ok], pos[ok])
+    for g, w in ((dk, kc), (dv, vc)):
+        h = g.cpu().view(torch.int16).numpy().view(np.uint16)
+        assert np.array_equal(h[keep], w[keep])
+
+
+def _cuda_core_child():
+    """(run in a child process) Calls of 128 tokens and more whose listed tokens
+    the CUDA-core kernel takes beside the prefill tiles."""
+    m = moe()
+    m.profile_enable(True)
+    test_prefill_ignores_cache_rows_past_the_chunk()
+    test_qkv_attend_and_block(CASES[-1])
+    for case in RAGGED[:1] + RAGGED[2:4]:
+        test_ragged_tiles_and_listed_tokens(*case)
+    test_probabilities_keep_their_bits(*TERMS[0])
+    ran = {k for k, v in m.profile_read().items() if v[0] > 0}
+    assert {"attention", "attention_tc"} <= ran and "attention_decode_tc" not in ran, sorted(ran)
+    print("listed tokens ok")
+
+
+def test_listed_tokens_on_the_cuda_cores():
+    """MOE_ATTN_CUDA_CORES=1 (a process of its own: the switch is read once)."""
+    need_gpu()
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c",
+                        "import tests.test_gpu_attention as t; t._cuda_core_child()"],
+                       cwd=root, env=dict(os.environ, MOE_ATTN_CUDA_CORES="1"), capture_output=True,
+                       text=True, timeout=600)
+    assert p.returncode == 0, (p.stdout + p.stderr)[-3000:]
+    assert "listed tokens ok" in p.stdout
