@@ -9,14 +9,19 @@
 // cache, no biases, resid += W_o . Attn(RMSNorm0(resid)).
 //
 // Kernels, in launch order:
-//   k_sa_prenorm   RMSNorm0 of the fp32 residual -> bf16 rows; block 0 also
-//                  writes the trivial dispatch of a one-"expert" projection
+//   k_sa_prenorm   RMSNorm0 of the fp32 residual -> bf16 rows; the first token's
+//                  block also writes the trivial dispatch of a one-"expert" projection
 //                  (offsets {0, T}), for the grouped GEMM of prefill batches;
+//                  in a planned call block 0 makes the attention's plan and the
+//                  tokens follow;
 //                  it lets the projection launch once its own wait is over (the
 //                  projection's weight loads do not depend on it);
-//   projection     W_qkv . x: the tcgen05 kernel with the weights as the M
-//                  operand (split reduction) for up to 640 tokens, the grouped
-//                  tcgen05 GEMM with E = 1 beyond (fp32 out);
+//   projection     W_qkv . x (fp32 out): the CTA-pair tcgen05 GEMM in equal
+//                  shares of its (unit, k-block)s where whole units would leave
+//                  a quarter of the pairs idle (proj_split, 257 to 2048 tokens), else
+//                  the tcgen05 kernel with the weights as the M operand (split
+//                  reduction) for up to 640 tokens, else the grouped tcgen05 GEMM
+//                  with E = 1;
 //   k_rope_cache   rotary embedding of q and k (angles formed and reduced in
 //                  fp64, evaluated in fp32), k and v written to the cache in
 //                  bf16;
@@ -29,8 +34,10 @@
 //                  of consecutive positions that the plan finds (a block of
 //                  k_sa_prenorm), the decode attention (attn_decode_tc.cu)
 //                  every other token;
-//   projection     W_o . ctx (the same two kernels), its partial sums added to
-//                  the residual by k_residual_add.
+//   projection     W_o . ctx (the weights-as-M kernel up to 640 tokens, the
+//                  grouped GEMM beyond): a projection in one part is added to
+//                  the residual by its epilogue, partial sums by
+//                  k_residual_add or, in decoder layers, k_residual_prenorm.
 #include <math.h>
 #include <stdlib.h>
 
@@ -769,9 +776,11 @@ SaWs sa_ws(const moe_sa_dims &d, int64_t T) {
     size_t o = 0;
     L.offsets = o; o += up(2 * 4);
     L.xn = o; o += up((size_t)T * d.d_model * 2);
-    // projection outputs (partial sums of a split reduction for up to
-    // kRowsMaxTokens tokens): qkv first, later the output projection's rows
-    // (as many rows as any smaller call needs, too)
+    // projection outputs: qkv first, later the output projection's rows, as many
+    // as any call of up to T tokens needs: partial sums of a split reduction for up
+    // to kRowsMaxTokens tokens, two parts of the equal shares for up to
+    // kProjSplitMaxTokens (whatever proj_split says of this shape: it asks the
+    // device and the environment, and the size must not depend on either)
     const size_t part_rows =
         std::max({(size_t)T, (size_t)kRowsMaxParts * std::min<int64_t>(T, kRowsMaxTokens),
                   (size_t)2 * std::min<int64_t>(T, kProjSplitMaxTokens)});
@@ -980,7 +989,6 @@ cudaError_t attend(const SaCall &c, const float *q, const int32_t *seq, const in
                       c.st, args);
 }
 
-// resid += W_o . ctx
 // resid += W_o . ctx; with xn_next (decoder layers, D <= 4 * 4 * 1024) the
 // MoE block's normalised input is written in the same pass.
 cudaError_t out_proj(const SaCall &c, const void *ctx, const void *w_o, float *resid,

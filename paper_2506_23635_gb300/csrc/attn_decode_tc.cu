@@ -41,9 +41,13 @@
 //            CTA 0, so a split whose share of the memory bandwidth runs ahead
 //            takes more.
 //   listed   the same for the tokens that a plan lists (the tokens of a call
-//            that no prefill tile holds), 128 tokens after the other (none of
-//            more than 128 is in two shares: there are 6 or more (token,
-//            head)s to a CTA then).  The CTAs start as the prefill
+//            that no prefill tile holds), 128 tokens after the other.  More than
+//            128 are taken whole: batches in equal shares would need slots and
+//            counters of their own, and with 8 key/value heads there are 6 or
+//            more (token, head)s to a CTA.  With 1 or 2 a batch has about
+//            one for each CTA, and a sequence far longer than the others keeps
+//            one CTA busy while the rest idle (1 key/value head, 160 tokens, one
+//            of 32,768 positions: 294 us; 1,050 on the CUDA cores).  The CTAs start as the prefill
 //            attention ahead leaves them SMs: that kernel started after the
 //            queries and cache rows were complete, and its own results are not
 //            read here, so they wait for it only at their end (for the kernels
@@ -51,8 +55,8 @@
 //
 //   warp 0      TMA: a piece's bf16 query rows into one of four buffers, key
 //               and value tiles into three-stage rings (each 32 KB: two boxes
-//               of 64 dims with the 128-byte swizzle), the first three before
-//               the block-wide barrier of the set-up; each tile is described
+//               of 64 dims with the 128-byte swizzle), the first three right
+//               after the dependency wait; each tile is described
 //               to the other warps in a ring of DecDesc;
 //   warp 1      tensor memory (S^T twice, O^T: 48 of 64 columns) and the
 //               MMAs: S_{j+1} is issued as soon as its key tile has landed
