@@ -20,8 +20,8 @@
 //                  shares of its (unit, k-block)s where whole units would leave
 //                  a quarter of the pairs idle (proj_split, 257 to 2048 tokens), else
 //                  the tcgen05 kernel with the weights as the M operand (split
-//                  reduction) for up to 640 tokens, else the grouped tcgen05 GEMM
-//                  with E = 1;
+//                  reduction) for up to 512 or 640 tokens (gemm_rows_fits), else
+//                  the grouped tcgen05 GEMM with E = 1;
 //   k_rope_cache   rotary embedding of q and k (angles formed and reduced in
 //                  fp64, evaluated in fp32), k and v written to the cache in
 //                  bf16;
@@ -34,8 +34,8 @@
 //                  of consecutive positions that the plan finds (a block of
 //                  k_sa_prenorm), the decode attention (attn_decode_tc.cu)
 //                  every other token;
-//   projection     W_o . ctx (the weights-as-M kernel up to 640 tokens, the
-//                  grouped GEMM beyond): a projection in one part is added to
+//   projection     W_o . ctx (the weights-as-M kernel or, where that does not
+//                  fit, the grouped GEMM): a projection in one part is added to
 //                  the residual by its epilogue, partial sums by
 //                  k_residual_add or, in decoder layers, k_residual_prenorm.
 #include <math.h>
@@ -865,7 +865,7 @@ cudaError_t qkv_rope(const SaCall &c, const void *xn, const void *w_qkv, const i
     if (proj_split(c.T, c.d.d_model, c.nr(), &split)) {
         n_part = 0;
         e = launch_proj_wm(c.T, c.d.d_model, c.nr(), xn, w_qkv, qkv, split, c.st, "qkv_gemm_tc");
-    } else if (c.T <= kRowsMaxTokens) {
+    } else if (gemm_rows_fits(c.T, c.nr())) {
         n_part = gemm_rows_parts(c.T, c.d.d_model, c.nr());
         e = launch_gemm_rows_tc(c.T, c.d.d_model, c.nr(), xn, w_qkv, n_part, qkv, c.st,
                                 "qkv_rows_tc");
@@ -996,12 +996,13 @@ cudaError_t out_proj(const SaCall &c, const void *ctx, const void *w_o, float *r
     const moe_dims pd = proj_dims(c.d.d_model, c.nq());
     const int32_t *offsets = at<int32_t>(c.ws, c.L.offsets);
     float *y = at<float>(c.ws, c.L.qkv);
-    int n_part = c.T <= kRowsMaxTokens ? gemm_rows_parts(c.T, c.nq(), c.d.d_model) : 1;
+    const bool rows = gemm_rows_fits(c.T, c.d.d_model);
+    int n_part = rows ? gemm_rows_parts(c.T, c.nq(), c.d.d_model) : 1;
     // a projection in one part is added to the residual by its epilogue
     const bool add = n_part == 1;
     float *dst = add ? resid : y;
     cudaError_t e =
-        c.T <= kRowsMaxTokens
+        rows
             ? launch_gemm_rows_tc(c.T, c.nq(), c.d.d_model, ctx, w_o, n_part, dst, c.st,
                                   "o_rows_tc", add)
             : launch_gemm_down_wm(pd, c.T, ctx, offsets, w_o, dst, c.st, "o_gemm_tc", add);

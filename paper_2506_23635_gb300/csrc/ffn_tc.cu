@@ -717,6 +717,11 @@ cudaError_t launch_gemm_down_tc(const moe_dims &d, int T, const void *h, const i
                                         y_sorted, st, name, y_tail);
 }
 
+bool gemm_rows_fits(int T, int Nw) {
+    const int ctas = (Nw + BM - 1) / BM * ((T + 255) / 256);
+    return T <= kRowsMaxTokens && (T <= 512 || ctas <= device_info().sm_count);
+}
+
 int gemm_rows_parts(int T, int Kdim, int Nw) {
     const int tiles = (Nw + BM - 1) / BM * ((T + 255) / 256), nk = (Kdim + BK - 1) / BK;
     const int by_sms = std::max(1, device_info().sm_count / std::max(1, tiles));

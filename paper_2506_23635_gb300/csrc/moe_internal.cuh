@@ -258,11 +258,18 @@ cudaError_t launch_gemm_up_tc(const moe_dims &d, int T, const void *x_sorted,
 // reduction split into `parts` (<= kRowsMaxParts) shares whose partial sums
 // land in y + p*T*Nw for p < parts (the caller adds them in order).
 // gemm_rows_parts: the split that keeps the SMs streaming for this shape.
-// (the last size that the CTA-pair GEMM does not beat: attention block of DBRX,
-// two projections, on this kernel and on that: 300 tokens 94 and 106 us, 400:
-// 105 and 115, 512: 125 and 127, 600: 148 and 152, 700: 170 and 161)
+// The sizes at which the CTA-pair GEMM does not beat it (gemm_rows_fits):
+// measured on attention blocks, this kernel and that one: DBRX (QKV 8192 rows,
+// d_model 6144) 300 tokens 85 and 101 us, 400: 100 and 112, 512: 115 and 117,
+// 700: 170 and 161; 6144 rows, d_model 4096: 300: 61 and 79, 640: 83 and 95; 10,240
+// rows, d_model 8192: 300: 124 and 129, 512: 152 and 148.  Above 512 tokens (three
+// runs of tokens) only where its CTAs, one for each 128 rows and run, fit one round
+// on the SMs: 10,240 rows at 600 tokens, 240 CTAs, 220 and 204 us.  (Smaller
+// matrices would gain from it up to 1024 tokens: 3072 rows, d_model 2048, 900
+// tokens 72 and 82 us.)
 constexpr int kRowsMaxTokens = 640;
 constexpr int kRowsMaxParts = 4;
+bool gemm_rows_fits(int T, int Nw);
 int gemm_rows_parts(int T, int Kdim, int Nw);
 // add (one part): the result is added to y.
 cudaError_t launch_gemm_rows_tc(int T, int Kdim, int Nw, const void *x, const void *w, int parts,

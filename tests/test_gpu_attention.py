@@ -826,3 +826,24 @@ def test_listed_tokens_on_the_cuda_cores():
                        text=True, timeout=600)
     assert p.returncode == 0, (p.stdout + p.stderr)[-3000:]
     assert "listed tokens ok" in p.stdout
+
+
+# (D, Hq, Hkv, tokens), the kernels of the QKV and of the output projection
+PROJ_ROUTES = [((264, 64, 8, 530), "qkv_gemm_tc", "o_rows_tc"), ((6600, 6, 1, 530), "qkv_rows_tc", "o_gemm_tc"),
+               ((6400, 6, 1, 530), "qkv_rows_tc", "o_rows_tc")]
+
+
+@pytest.mark.parametrize("case,qkv,out", PROJ_ROUTES, ids=lambda v: str(v))
+def test_wide_projections_above_512_tokens(case, qkv, out):
+    """The weights-as-M kernel takes three runs of tokens only where its CTAs fit
+    one round (80 weight tiles do not, nor do 52; 50 do on 152 SMs), the pair
+    GEMM the others; the values are the oracle's either way."""
+    m = moe()
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("routes of 152 SMs")
+    m.profile_reset()
+    m.profile_enable(True)
+    test_projections_of_many_tokens(*case)
+    m.profile_enable(False)
+    ran = {k for k, v in m.profile_read().items() if v[0] > 0}
+    assert {qkv, out} <= ran, sorted(ran)
