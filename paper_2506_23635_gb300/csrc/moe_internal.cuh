@@ -362,6 +362,11 @@ struct ProjSplit {
         return owner(first + nk - 1) - owner(first) + 1;
     }
 };
+// (up to 256 tokens the weights-as-M kernel splits the reduction itself; above
+// 2048, nine runs of tokens and more, whole units leave a quarter of 76 pairs idle
+// only with 18 weight tiles, 4608 rows, or fewer, and the two parts of every
+// output would go on widening the workspace; the share of idle pairs is what
+// decides between, measured on the widths that proj_split names)
 constexpr int kProjSplitMinTokens = 257;
 constexpr int kProjSplitMaxTokens = 2048;
 bool proj_split(int T, int Kdim, int Nw, ProjSplit *split);
